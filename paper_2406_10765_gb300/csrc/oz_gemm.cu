@@ -16,8 +16,9 @@
 //   * The slice products d_p(a) d_q(b) with p + q = g are summed in one FP32
 //     tensor-memory accumulator per group g (g = 2..S+1; the pairs with
 //     p + q > S + 1 are below 2^-55 of the largest product and dropped).  Over
-//     a chunk of 64 real K every partial sum is an integer below 2^22, so the
-//     FP32 accumulation is exact whatever its rounding.
+//     a chunk of 96 real K every partial sum is an integer below 2^22 (two
+//     pairs of at most 2^13 and six of at most 2^12 per K: 2.5 2^14 96), so
+//     the FP32 accumulation is exact whatever its rounding.
 //   * After each chunk the epilogue adds every group, shifted to a common
 //     binary point 2^-L, into a 64-bit integer per output (exact except for
 //     a rounding of the lowest groups below 2^-L), and at the end converts
@@ -33,8 +34,23 @@
 // CTA; warp 0 = TMA producer, warp 1 = MMA issuer (one thread), warps 2..9 =
 // epilogue.  Two shared-memory stages of 32 real K, each holding all S slices
 // of the A and B tiles (64-byte swizzle); eight 64-column FP32 accumulators
-// fill the 512 tensor-memory columns.  Every mbarrier wait is bounded; on
-// timeout the CTA records an error word, frees its tensor memory and returns.
+// fill the 512 tensor-memory columns.
+//
+// The slices of B lie one after the other in a stage, behind three slices of
+// zeros, and the accumulators of the groups one after the other in tensor
+// memory.  So slice p of A times four consecutive slices of B is ONE MMA of
+// 256 columns onto four consecutive groups, the pairs that do not exist
+// (q < 1) multiplying zeros: 12 MMAs of one shape per 16 K, 8 onto the upper
+// four groups and 4 onto the lower four, instead of 36 of 64 columns.  A is
+// read from shared memory 12 times instead of 36 (94 B/clock at the tensor
+// peak instead of 192; 128 are available), and the issuing thread no longer
+// limits the rate.  The two halves of the groups are emptied half a chunk
+// apart, so that the MMAs of one run while the epilogue reads the other.
+// Measured, 3,456 x 1,152 x 3,456: 6.15 ms with one MMA per slice pair, 3.35 ms
+// so (33 TFLOP/s FP64-equivalent); what it issues, zeros included, is 1.58
+// PFLOP/s, 0.82 of the measured cuBLAS burst rate: the tensor pipe bounds it.
+// Every mbarrier wait is bounded; on timeout the CTA records an error word,
+// frees its tensor memory and returns.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_fp16.h>
@@ -51,14 +67,21 @@ namespace {
 
 using namespace pw_umma;
 
-constexpr int NG = S;                 // accumulator groups g = 2..S+1
 constexpr int BM = 128, BN = 64, BK = 32;   // real rows, real columns, real K per stage
 constexpr int A_T = BM * BK * 2;      // 8 KB per slice
 constexpr int B_T = BN * BK * 2;      // 4 KB per slice
-constexpr int STAGE = S * (A_T + B_T);   // 96 KB
+constexpr int HG = S / 2;             // groups emptied together (a half of them)
+constexpr int ZB_T = (HG - 1) * B_T;  // zero slices in front of B's
+constexpr int OFF_Z = S * A_T, OFF_B = OFF_Z + ZB_T;
+constexpr int STAGE = OFF_B + S * B_T;   // 108 KB
+constexpr int STAGE_LOAD = S * (A_T + B_T);   // of which TMA writes 96 KB
 constexpr int NSTAGE = 2;
-constexpr int CHUNK_KB = 2;           // K blocks per exact accumulation chunk (64 real K)
+constexpr int CHUNK_KB = 3;           // K blocks per exact accumulation chunk (96 real K)
+constexpr int STEPS_KB = BK / 16;     // MMA steps (16 real K) per K block
+constexpr int CHUNK = CHUNK_KB * STEPS_KB;
+constexpr int NH = 2;
 constexpr int SMEM_BYTES = NSTAGE * STAGE + 1024 + 512;
+static_assert(SMEM_BYTES <= 232448, "shared memory per CTA");
 constexpr int TMEM_COLS = 512;
 constexpr int EPI_WARPS = 8;
 constexpr int NTHREADS = 64 + 32 * EPI_WARPS;
@@ -73,8 +96,34 @@ __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, u
 // shared-memory matrix descriptor: K-major, 64-byte swizzle (rows of 32
 // FP16), 8-row groups 512 B apart
 __device__ __forceinline__ uint64_t smem_desc_sw64(uint32_t addr) { return smem_desc(addr, 16, 512, 4); }
-// instruction descriptor, kind::f16: FP16 A and B, FP32 D, both K-major, M = 128, N = 64
-__host__ __device__ constexpr uint32_t idesc_oz() { return idesc_f16(BM, BN, false); }
+
+// whether half h (0: groups 2..5, 1: groups 6..9) is emptied after MMA step t
+// of nsteps: every CHUNK steps, the halves CHUNK / 2 apart, and at the end
+__device__ __forceinline__ bool oz_flush(int h, int t, int nsteps) {
+  return (t + 1 + (h == 0 ? CHUNK / 2 : 0)) % CHUNK == 0 || t == nsteps - 1;
+}
+
+// The slice products of half H for one step: slice p of A times the slices
+// q0..q0 + 3 of B, q0 = 4 H + 2 - p, onto the groups p + q = 4 H + 2.. (q < 1:
+// zeros).  Every MMA has the same shape and accumulators, which is what
+// orders them.  `first`: the step opens the half's chunk, and its first MMA
+// overwrites the accumulators.  db: the stage's first zero slice.
+template <int H>
+__device__ __forceinline__ void oz_mmas(uint32_t tmem, uint64_t da, uint64_t db, bool first) {
+#pragma unroll
+  for (int p = 1; p <= (H + 1) * HG; ++p) {
+    const int q0 = H * HG + 2 - p;
+    mma_f16(tmem + (uint32_t)(H * HG * BN), da + (uint64_t)((p - 1) * (A_T >> 4)),
+            db + (uint64_t)((q0 + HG - 2) * (B_T >> 4)), idesc_f16(BM, HG * BN, false), !(first && p == 1));
+  }
+}
+
+// bits of the FP32 accumulator value v + 1.5 2^23 (an integer |v| < 2^22): kBias + v
+constexpr uint32_t kBias = 0x4B400000u;
+__device__ __forceinline__ uint32_t biased(uint32_t v) {
+  return __float_as_uint(__uint_as_float(v) + 12582912.0f);
+}
+
 __global__ void __launch_bounds__(NTHREADS, 1)
     k_oz_gemm(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
               int a_slice_rows, int b_slice_rows, int m, int n, int kblocks, int mtiles, int ntiles,
@@ -85,9 +134,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint64_t *full = (uint64_t *)(smem + NSTAGE * STAGE);
   uint64_t *empty = full + NSTAGE;
-  uint64_t *accf = empty + NSTAGE;     // [NG] group accumulator ready
-  uint64_t *acce = accf + NG;          // [NG] group accumulator drained
-  uint32_t *tmem_slot = (uint32_t *)(acce + NG);
+  uint64_t *accf = empty + NSTAGE;     // [NH] a half's accumulators ready
+  uint64_t *acce = accf + NH;          // [NH] a half's accumulators drained
+  uint32_t *tmem_slot = (uint32_t *)(acce + NH);
 
   const int tile = blockIdx.x;
   const int mt = tile / ntiles, nt = tile % ntiles;
@@ -114,7 +163,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   const int c0 = min(nch, (int)blockIdx.y * per), c1 = min(nch, c0 + per);
   const int kb_beg = kb_lo + c0 * CHUNK_KB;
   const int nkb = max(0, min(kb_hi, kb_lo + c1 * CHUNK_KB) - kb_beg);
-  const int nchunk = (nkb + CHUNK_KB - 1) / CHUNK_KB;
+  const int nsteps = nkb * STEPS_KB;
   // binary point of the fixed-point sum: |sum| <= K' (scaled entries < 1)
   int lg = 0;
   while ((1 << lg) < max(1, nkb * BK)) ++lg;
@@ -123,9 +172,14 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int s = 0; s < NSTAGE; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
-    for (int g = 0; g < NG; ++g) { mbar_init(&accf[g], 1); mbar_init(&acce[g], EPI_WARPS); }
+    for (int h = 0; h < NH; ++h) { mbar_init(&accf[h], 1); mbar_init(&acce[h], EPI_WARPS); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  // the zero slices, for the tensor core's reads (the async proxy)
+  for (int s = 0; s < NSTAGE; ++s)
+    for (int w = threadIdx.x; w < ZB_T / 16; w += NTHREADS)
+      *(uint4 *)(smem + s * STAGE + OFF_Z + w * 16) = make_uint4(0u, 0u, 0u, 0u);
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                  "r"(TMEM_COLS));
@@ -144,51 +198,50 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         const uint32_t u = i / NSTAGE;
         if (!mbar_wait(&empty[s], (u & 1) ^ 1)) { atomicOr(err, 1); break; }
         unsigned char *st = smem + s * STAGE;
-        mbar_expect_tx(&full[s], STAGE);
+        mbar_expect_tx(&full[s], STAGE_LOAD);
         const int x = (kb_beg + i) * BK;
 #pragma unroll
         for (int p = 0; p < S; ++p) {
           tma_load_2d(st + p * A_T, &mapA, &full[s], x, p * a_slice_rows + m0);
-          tma_load_2d(st + S * A_T + p * B_T, &mapB, &full[s], x, p * b_slice_rows + (real_out ? j0 : 2 * j0));
+          tma_load_2d(st + OFF_B + p * B_T, &mapB, &full[s], x, p * b_slice_rows + (real_out ? j0 : 2 * j0));
         }
       }
     }
   } else if (warp == 1) {
     if (lane == 0) {
-      // ---------------- MMA issuer
-      const uint32_t idesc = idesc_oz();
-      bool ok = true;
-      for (int i = 0; i < nkb && ok; ++i) {
+      // ---------------- MMA issuer.  The descriptors are formed once; slices,
+      // K steps and stages only move their start address (16-byte units in the
+      // low 14 bits, which cover all of shared memory, so nothing carries out)
+      const uint64_t da0 = smem_desc_sw64(smem_u32(smem)), db0 = smem_desc_sw64(smem_u32(smem + OFF_Z));
+      uint32_t nfl0 = 0, nfl1 = 0;          // times each half was handed to the epilogue
+      bool first0 = true, first1 = true;    // the next step opens the half's chunk
+      for (int i = 0; i < nkb; ++i) {
         const int s = i % NSTAGE;
         const uint32_t u = i / NSTAGE;
-        const int ch = i / CHUNK_KB;
-        const bool first = (i % CHUNK_KB) == 0;
-        const bool last = (i % CHUNK_KB) == CHUNK_KB - 1 || i == nkb - 1;
         if (!mbar_wait(&full[s], u & 1)) { atomicOr(err, 2); break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t base = smem_u32(smem + s * STAGE);
+        bool ok = true;
 #pragma unroll
-        for (int kk = 0; kk < BK / 16; ++kk) {
-#pragma unroll
-          for (int g = 0; g < NG; ++g) {
-            const int d = g + 2;
-            if (first && kk == 0) {
-              // the epilogue has read this group's previous chunk
-              if (!mbar_wait(&acce[g], ((uint32_t)ch & 1) ^ 1)) { atomicOr(err, 8); ok = false; break; }
-              asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            }
-            const int plo = max(1, d - S), phi = min(S, d - 1);
-#pragma unroll
-            for (int p = plo; p <= phi; ++p) {
-              const int q = d - p;
-              const uint64_t da = smem_desc_sw64(base + (p - 1) * A_T) + 2 * kk;
-              const uint64_t db = smem_desc_sw64(base + S * A_T + (q - 1) * B_T) + 2 * kk;
-              mma_f16(tmem + (uint32_t)(g * BN), da, db, idesc, !(first && kk == 0 && p == plo));
-            }
-            if (last && kk == BK / 16 - 1) mma_commit(&accf[g]);
+        for (int kk = 0; kk < STEPS_KB; ++kk) {
+          const int t = i * STEPS_KB + kk;
+          const uint64_t off = (uint64_t)(s * (STAGE >> 4) + 2 * kk);
+          if (first1) {
+            // the epilogue has read the half's previous chunk
+            if (!mbar_wait(&acce[1], (nfl1 & 1) ^ 1)) { atomicOr(err, 8); ok = false; break; }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           }
-          if (!ok) break;
+          oz_mmas<1>(tmem, da0 + off, db0 + off, first1);
+          first1 = oz_flush(1, t, nsteps);
+          if (first1) { mma_commit(&accf[1]); ++nfl1; }
+          if (first0) {
+            if (!mbar_wait(&acce[0], (nfl0 & 1) ^ 1)) { atomicOr(err, 8); ok = false; break; }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          }
+          oz_mmas<0>(tmem, da0 + off, db0 + off, first0);
+          first0 = oz_flush(0, t, nsteps);
+          if (first0) { mma_commit(&accf[0]); ++nfl0; }
         }
+        if (!ok) break;
         mma_commit(&empty[s]);
       }
     }
@@ -196,25 +249,51 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     // ---------------- epilogue: warps 2..9; lane quarter q, column half h
     const int q = warp & 3, h = (warp - 2) >> 2;
     const uint32_t lanes = (uint32_t)(q * 32) << 16;
-    long long acc[32];
+    // 64-bit fixed-point sums modulo 2^64; groups with a left shift add
+    // kBias + v, and the biases are taken off at the end
+    unsigned long long acc[32];
 #pragma unroll
     for (int i = 0; i < 32; ++i) acc[i] = 0;
     bool ok = true;
-    for (int ch = 0; ch < nchunk && ok; ++ch) {
-#pragma unroll 1
-      for (int g = 0; g < NG; ++g) {
-        if (!mbar_wait(&accf[g], (uint32_t)ch & 1)) { atomicOr(err, 4); ok = false; break; }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        uint32_t v[32];
-        tmem_ld32(tmem + lanes + (uint32_t)(g * BN + h * 32), v);
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&acce[g]);
-        const int sh = Lfix - BETA * (g + 2);
+    uint32_t nfl[NH] = {0, 0};
+    unsigned long long bias = 0;
+    for (int t = 0; t < nsteps && ok; ++t) {
 #pragma unroll
-        for (int i = 0; i < 32; ++i) acc[i] += shifted(f2i_exact(v[i]), sh);
+      for (int hh = NH - 1; hh >= 0; --hh) {
+        if (!ok || !oz_flush(hh, t, nsteps)) continue;
+        if (!mbar_wait(&accf[hh], nfl[hh] & 1)) { atomicOr(err, 4); ok = false; continue; }
+        ++nfl[hh];
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll 1
+        for (int g = hh * HG; g < hh * HG + HG; ++g) {
+          uint32_t v[32];
+          tmem_ld32(tmem + lanes + (uint32_t)(g * BN + h * 32), v);
+          if (g == hh * HG + HG - 1) {
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&acce[hh]);
+          }
+          const int sh = Lfix - BETA * (g + 2);
+          if (sh >= 32) {
+#pragma unroll
+            for (int i = 0; i < 32; ++i) acc[i] += (unsigned long long)(biased(v[i]) << (sh - 32)) << 32;
+          } else if (sh >= 0) {
+            const uint32_t f = 1u << sh;
+#pragma unroll
+            for (int i = 0; i < 32; ++i) acc[i] += (unsigned long long)biased(v[i]) * f;
+          } else {
+            // rounded to nearest
+            const int half = 1 << (-sh - 1);
+#pragma unroll
+            for (int i = 0; i < 32; ++i)
+              acc[i] += (unsigned long long)(long long)(((int)(biased(v[i]) - kBias) + half) >> -sh);
+          }
+          if (sh >= 0) bias += (unsigned long long)kBias << sh;
+        }
       }
     }
+#pragma unroll
+    for (int i = 0; i < 32; ++i) acc[i] -= bias;
     const int i = m0 + q * 32 + lane;              // complex output row
     if (ok && i < m && real_out) {
       double *Cr = (double *)C;
@@ -223,7 +302,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       for (int t = 0; t < 32; ++t) {
         const int j = j0 + h * 32 + t;
         if (j >= n) continue;
-        double r = alpha.x * scale_pow2((double)acc[t], ka - eb[j]);
+        double r = alpha.x * scale_pow2((double)(long long)acc[t], ka - eb[j]);
         if (beta.x != 0.0) r += beta.x * Cr[i + (long)j * ldc];
         Cr[i + (long)j * ldc] = r;
       }
@@ -236,8 +315,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         if (j >= n) continue;
         if (herm == 2 && ((joff + j) >> 6) > ((ioff + i) >> 6)) continue;
         const int k = ka - eb[j];
-        const double re = scale_pow2((double)acc[2 * t], k);
-        const double im = scale_pow2((double)acc[2 * t + 1], k);
+        const double re = scale_pow2((double)(long long)acc[2 * t], k);
+        const double im = scale_pow2((double)(long long)acc[2 * t + 1], k);
         if (part) {
           part[(long)blockIdx.y * m * n + i + (long)j * m] = make_double2(re, im);
         } else {
