@@ -76,6 +76,7 @@ constexpr int OFF_Z = S * A_T, OFF_B = OFF_Z + ZB_T;
 constexpr int STAGE = OFF_B + S * B_T;   // 108 KB
 constexpr int STAGE_LOAD = S * (A_T + B_T);   // of which TMA writes 96 KB
 constexpr int NSTAGE = 2;
+constexpr int NG = S;                 // accumulator groups g = 2..S+1
 constexpr int CHUNK_KB = 3;           // K blocks per exact accumulation chunk (96 real K)
 constexpr int STEPS_KB = BK / 16;     // MMA steps (16 real K) per K block
 constexpr int CHUNK = CHUNK_KB * STEPS_KB;
@@ -254,6 +255,14 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     unsigned long long acc[32];
 #pragma unroll
     for (int i = 0; i < 32; ++i) acc[i] = 0;
+    // the two lowest groups, weights 2^-56 and 2^-63, are added in units of
+    // 2^-63, and what lies below the sum's binary point stays in rem until the
+    // end: one rounding instead of two per chunk
+    uint32_t rem[32];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) rem[i] = 0;
+    const int slow = BETA * (S + 1) - Lfix;      // 7..
+    const uint32_t mlow = (1u << slow) - 1u;
     bool ok = true;
     uint32_t nfl[NH] = {0, 0};
     unsigned long long bias = 0;
@@ -264,14 +273,15 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         if (!mbar_wait(&accf[hh], nfl[hh] & 1)) { atomicOr(err, 4); ok = false; continue; }
         ++nfl[hh];
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const int gend = hh == NH - 1 ? NG - 2 : (hh + 1) * HG;
 #pragma unroll 1
-        for (int g = hh * HG; g < hh * HG + HG; ++g) {
+        for (int g = hh * HG; g < gend; ++g) {
           uint32_t v[32];
           tmem_ld32(tmem + lanes + (uint32_t)(g * BN + h * 32), v);
-          if (g == hh * HG + HG - 1) {
+          if (g == HG - 1) {
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
-            if (lane == 0) mbar_arrive(&acce[hh]);
+            if (lane == 0) mbar_arrive(&acce[0]);
           }
           const int sh = Lfix - BETA * (g + 2);
           if (sh >= 32) {
@@ -282,7 +292,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 #pragma unroll
             for (int i = 0; i < 32; ++i) acc[i] += (unsigned long long)biased(v[i]) * f;
           } else {
-            // rounded to nearest
+            // rounded to nearest (the third lowest group of very long sums)
             const int half = 1 << (-sh - 1);
 #pragma unroll
             for (int i = 0; i < 32; ++i)
@@ -290,8 +300,30 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           }
           if (sh >= 0) bias += (unsigned long long)kBias << sh;
         }
+        if (hh == NH - 1) {
+          const uint32_t tv = tmem + lanes + (uint32_t)((NG - 2) * BN + h * 32), tu = tv + BN;
+#pragma unroll
+          for (int c = 0; c < 32; c += 16) {
+            uint32_t v[16], u[16];
+            tmem_ld16x2(tv + c, tu + c, v, u);
+            if (c == 16) {
+              asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+              __syncwarp();
+              if (lane == 0) mbar_arrive(&acce[NH - 1]);
+            }
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+              // |v| 2^7 + |u| + rem < 2^29 + 2^22 + 2^30: a signed 32-bit sum
+              const uint32_t w = (biased(v[i]) << BETA) + biased(u[i]) + (rem[c + i] - ((kBias << BETA) + kBias));
+              acc[c + i] += (unsigned long long)(long long)((int)w >> slow);
+              rem[c + i] = w & mlow;
+            }
+          }
+        }
       }
     }
+#pragma unroll
+    for (int i = 0; i < 32; ++i) acc[i] += (rem[i] + (1u << (slow - 1))) >> slow;
 #pragma unroll
     for (int i = 0; i < 32; ++i) acc[i] -= bias;
     const int i = m0 + q * 32 + lane;              // complex output row
