@@ -61,6 +61,52 @@ __device__ double block_max(double v, double *sh) {
   return r;
 }
 
+// 1 / x by one cubic Newton-Raphson step on the hardware's approximate
+// reciprocal (relative error e -> e^3, about an ulp for normal x): three FP64
+// operations instead of the ten of a rounded reciprocal.  The FP64 pipe issues
+// one warp instruction per sub-partition in 64 clocks on this part, so the
+// count of FP64 instructions is what the kernels below cost.
+__device__ __forceinline__ double rcp_approx(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  return r;
+}
+__device__ __forceinline__ double rcp_newton(double x) {
+  const double r = rcp_approx(x);
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+// a / x with the remainder of the first quotient folded in (error below one
+// ulp for normal quotients)
+__device__ __forceinline__ double div_newton(double a, double x) {
+  const double r = rcp_newton(x);
+  const double q = a * r;
+  return fma(fma(-q, x, a), r, q);
+}
+// sums over the warp of four values at once, every lane getting all four:
+// the lanes are split between the values while they are added, six FP64
+// additions instead of twenty
+__device__ __forceinline__ void warp_sum4(double &a, double &b, double &c, double &d) {
+  const int lane = threadIdx.x & 31;
+  const bool h16 = lane & 16, h8 = lane & 8;
+  double x = (h16 ? b : a) + __shfl_xor_sync(0xffffffffu, h16 ? a : b, 16);   // a | b
+  double y = (h16 ? d : c) + __shfl_xor_sync(0xffffffffu, h16 ? c : d, 16);   // c | d
+  double v = (h8 ? y : x) + __shfl_xor_sync(0xffffffffu, h8 ? x : y, 8);      // a c | b d
+  v += __shfl_xor_sync(0xffffffffu, v, 4);
+  v += __shfl_xor_sync(0xffffffffu, v, 2);
+  v += __shfl_xor_sync(0xffffffffu, v, 1);
+  a = __shfl_sync(0xffffffffu, v, 0);
+  c = __shfl_sync(0xffffffffu, v, 8);
+  b = __shfl_sync(0xffffffffu, v, 16);
+  d = __shfl_sync(0xffffffffu, v, 24);
+}
+// order-preserving integer of a (finite or infinite) double: comparisons then
+// run on the integer pipe
+__device__ __forceinline__ long long ordered_bits(double v) {
+  const long long b = __double_as_longlong(v + 0.0);   // -0 -> +0
+  return b < 0 ? (long long)0x8000000000000000ull - b : b;
+}
+
 // ======================================================================
 // Cholesky, scaling, triangular inverse
 // ======================================================================
@@ -864,14 +910,22 @@ __device__ int block_excl_scan(int v, int *s_scan, int *total) {
   __syncthreads();
   s_scan[threadIdx.x] = v;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    int acc = 0;
-    for (int t = 0; t < (int)blockDim.x; ++t) {
-      const int c = s_scan[t];
-      s_scan[t] = acc;
+  if (threadIdx.x < 32) {      // blockDim / 32 consecutive counts per lane, then the lanes
+    const int per = blockDim.x >> 5, b = threadIdx.x * per;
+    int sum = 0;
+    for (int q = 0; q < per; ++q) sum += s_scan[b + q];
+    int inc = sum;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, inc, o);
+      if ((int)threadIdx.x >= o) inc += u;
+    }
+    int acc = inc - sum;
+    for (int q = 0; q < per; ++q) {
+      const int c = s_scan[b + q];
+      s_scan[b + q] = acc;
       acc += c;
     }
-    s_scan[blockDim.x] = acc;
+    if (threadIdx.x == 31) s_scan[blockDim.x] = acc;
   }
   __syncthreads();
   *total = s_scan[blockDim.x];
@@ -880,10 +934,8 @@ __device__ int block_excl_scan(int v, int *s_scan, int *total) {
 
 // sort, z-vector, deflation and compaction for one node per CTA.  The merge
 // of the two sorted halves places each value by its rank in the other half
-// (ties: left first); the deflation scan (each decision depends on the
-// previous surviving index) runs on one thread over the node's arrays and
-// records its rotations, which the block then applies in order; the
-// compactions are block-wide prefix sums.
+// (ties: left first); the deflating rotations are recorded in order, and the
+// block then applies them; the compactions are block-wide prefix sums.
 __global__ void __launch_bounds__(256) k_dc_deflate(const int *nodes, int n, const double *e,
                                                     DcArrays a) {
   __shared__ double sh[32];
@@ -931,36 +983,70 @@ __global__ void __launch_bounds__(256) k_dc_deflate(const int *nodes, int n, con
   dmax = block_max(dmax, sh);
   const double rho2 = 2.0 * rho;
   const double tol = 8.0 * kEps * fmax(dmax, rho2);
-  // 2. deflation scan; rotation list in this node's own columns of W (W is
-  // rewritten by k_dc_gemm later in the level)
+  // 2. deflation.  Small z entries deflate at once (a parallel test); a pair
+  // of consecutive survivors rotates if |z_j z_p (D_p - D_j)| <= tol (z_j^2 +
+  // z_p^2).  A decision depends on an earlier one only behind a rotation, which
+  // changes the pair's later entry: the tests run in parallel on the unrotated
+  // values, and one thread walks the pairs that pass and, behind each rotation,
+  // the pairs after it until one does not rotate.  (The whole scan on one
+  // thread was 1.4 us per index: 9.5 ms of the order-3,456 eigensolve.)
+  // Rotation list in this node's own columns of W (W is rewritten by k_dc_gemm
+  // later in the level); survivors in colK, passing pairs in dcol (both filled
+  // again below).
   double *rot = a.W + (long)lo * n;
+  int *surv = a.colK + lo, *pass = a.dcol + lo;
+  const int chunk = (size + blockDim.x - 1) / blockDim.x;
+  const int p0 = min(size, (int)threadIdx.x * chunk), p1 = min(size, p0 + chunk);
+  int cnt = 0;
+  for (int p = p0; p < p1; ++p) {
+    const bool tiny = rho2 * fabs(a.zs[lo + p]) <= tol;
+    if (tiny) a.defl[lo + p] = 1;
+    cnt += !tiny;
+  }
+  int ns;
+  int t = block_excl_scan(cnt, s_scan, &ns);
+  for (int p = p0; p < p1; ++p)
+    if (!a.defl[lo + p]) surv[t++] = p;
+  __syncthreads();
+  auto pair_rotates = [&](int q) {   // survivors q - 1 and q
+    const int j = lo + surv[q - 1], p = lo + surv[q];
+    const double zj = a.zs[j], zp = a.zs[p];
+    return fabs(zj * zp * (a.Ds[p] - a.Ds[j])) <= tol * fma(zj, zj, zp * zp);
+  };
+  const int sch = (ns + blockDim.x - 1) / blockDim.x;
+  const int q0 = min(ns, (int)threadIdx.x * sch), q1 = min(ns, q0 + sch);
+  cnt = 0;
+  for (int q = max(q0, 1); q < q1; ++q) cnt += pair_rotates(q);
+  int npass;
+  t = block_excl_scan(cnt, s_scan, &npass);
+  if (npass > 0)
+    for (int q = max(q0, 1); q < q1; ++q)
+      if (pair_rotates(q)) pass[t++] = q;
+  __syncthreads();
   if (threadIdx.x == 0) {
-    int prev = -1, nrot = 0;
-    for (int p = 0; p < size; ++p) {
-      const double zp = a.zs[lo + p];
-      if (rho2 * fabs(zp) <= tol) { a.defl[lo + p] = 1; continue; }
-      if (prev >= 0) {
-        const int j = prev;
-        const double zj = a.zs[lo + j];
+    int nrot = 0, next = 0;          // pairs below `next` are decided
+    for (int k = 0; k < npass; ++k) {
+      for (int q = max(pass[k], next); q < ns; ++q) {
+        next = q + 1;
+        if (!pair_rotates(q)) break;
+        const int j = surv[q - 1], p = surv[q];
+        const double zj = a.zs[lo + j], zp = a.zs[lo + p];
         const double r = hypot(zp, zj);
         const double c = zp / r, s = -zj / r;
         const double Dj = a.Ds[lo + j], Dp = a.Ds[lo + p];
-        if (fabs(c * s * (Dp - Dj)) <= tol) {
-          const int cj = lo + a.perm[lo + j], ci = lo + a.perm[lo + p];
-          if (a.ctype[cj] != a.ctype[ci]) a.ctype[cj] = a.ctype[ci] = 2;
-          rot[4 * nrot] = cj;
-          rot[4 * nrot + 1] = ci;
-          rot[4 * nrot + 2] = c;
-          rot[4 * nrot + 3] = s;
-          ++nrot;
-          a.Ds[lo + j] = c * c * Dj + s * s * Dp;
-          a.Ds[lo + p] = s * s * Dj + c * c * Dp;
-          a.zs[lo + j] = 0.0;
-          a.zs[lo + p] = r;
-          a.defl[lo + j] = 1;
-        }
+        const int cj = lo + a.perm[lo + j], ci = lo + a.perm[lo + p];
+        if (a.ctype[cj] != a.ctype[ci]) a.ctype[cj] = a.ctype[ci] = 2;
+        rot[4 * nrot] = cj;
+        rot[4 * nrot + 1] = ci;
+        rot[4 * nrot + 2] = c;
+        rot[4 * nrot + 3] = s;
+        ++nrot;
+        a.Ds[lo + j] = c * c * Dj + s * s * Dp;
+        a.Ds[lo + p] = s * s * Dj + c * c * Dp;
+        a.zs[lo + j] = 0.0;
+        a.zs[lo + p] = r;
+        a.defl[lo + j] = 1;
       }
-      prev = p;
     }
     s_nrot = nrot;
   }
@@ -979,12 +1065,10 @@ __global__ void __launch_bounds__(256) k_dc_deflate(const int *nodes, int n, con
   }
   // 3. compaction: survivors -> (DK, zK, colK), deflated -> (dD, dcol), in order
   const bool all_defl = !(rho2 > 0.0);   // no coupling: everything deflates
-  const int chunk = (size + blockDim.x - 1) / blockDim.x;
-  const int p0 = min(size, (int)threadIdx.x * chunk), p1 = min(size, p0 + chunk);
-  int cnt = 0;
+  cnt = 0;
   for (int p = p0; p < p1; ++p) cnt += (!all_defl && !a.defl[lo + p]);
   int k_total;
-  int t = block_excl_scan(cnt, s_scan, &k_total);
+  t = block_excl_scan(cnt, s_scan, &k_total);
   int q = p0 - t;
   for (int p = p0; p < p1; ++p) {
     const int col = lo + a.perm[lo + p];
@@ -1027,7 +1111,17 @@ __global__ void __launch_bounds__(256) k_dc_deflate(const int *nodes, int n, con
   }
 }
 
-// one warp per root t of the secular equation 1 + rho sum z_i^2 / (D_i - lam) = 0
+// One warp per root t of the secular equation f = 1 + rho sum z_i^2 / (D_i -
+// lam) = 0: lam = D_o + tau with the nearer pole as origin; rational
+// interpolation with the poles left and right of the root, safeguarded by a
+// bracket.  The iteration ends when |f| is below what its own evaluation may
+// be off (R.-C. Li, Solving secular equations stably and efficiently, 1993):
+// a few ulps of 1 + |psi| + |phi| and of tau's effect on f -- the accuracy the
+// recomputed z of k_dc_zhat needs.  Run until the bracket closed instead, f's
+// own rounding kept it going for ~50 iterations (187 us at order 54, 13.6 ms
+// over the levels of order 3,456).  The step to the next iterate needs a few
+// digits only (f carries the small factor), so it uses approximate
+// reciprocals and square roots.
 __global__ void __launch_bounds__(256) k_dc_roots(const int *nodes, DcArrays a) {
   const int node = blockIdx.y;
   const int lo = nodes[3 * node];
@@ -1037,66 +1131,61 @@ __global__ void __launch_bounds__(256) k_dc_roots(const int *nodes, DcArrays a) 
   if (t >= k) return;
   const double rho = a.rhonode[node];
   const double *D = a.DK + lo, *z = a.zK + lo;
-  int o;
-  double blo, bhi;
-  if (t < k - 1) {
-    const double half = 0.5 * (D[t + 1] - D[t]);
+  const double Dt = D[t];
+  int o = t;
+  double blo = 0.0, bhi;
+  {
+    const double half = t < k - 1 ? 0.5 * (D[t + 1] - Dt) : 0.0;
     double s = 0.0;
-    for (int i = lane; i < k; i += 32) s += z[i] * z[i] / ((D[i] - D[t]) - half);
+    for (int i = lane; i < k; i += 32) {
+      const double zi = z[i];
+      s = t < k - 1 ? fma(zi * zi, rcp_newton((D[i] - Dt) - half), s) : fma(zi, zi, s);
+    }
     s = warp_sum(s);
-    if (1.0 + rho * s >= 0.0) { o = t; blo = 0.0; bhi = half; }
+    if (t == k - 1) bhi = rho * s;
+    else if (1.0 + rho * s >= 0.0) bhi = half;
     else { o = t + 1; blo = -half; bhi = 0.0; }
-  } else {
-    double s = 0.0;
-    for (int i = lane; i < k; i += 32) s += z[i] * z[i];
-    s = warp_sum(s);
-    o = t; blo = 0.0; bhi = rho * s;
   }
   const double Do = D[o];
-  const double da = D[t] - Do;                          // left pole
+  const double da = Dt - Do;                            // left pole
   const double db = (t < k - 1) ? D[t + 1] - Do : 0.0;  // right pole (if any)
   double tau = 0.5 * (blo + bhi);
   for (int it = 0; it < 100; ++it) {
     double psi = 0.0, dpsi = 0.0, phi = 0.0, dphi = 0.0;
     for (int i = lane; i < k; i += 32) {
-      // one reciprocal per term (FP64 divisions are the costly part here)
-      const double r = __drcp_rn((D[i] - Do) - tau);
+      const double r = rcp_newton((D[i] - Do) - tau);
       const double term = z[i] * z[i] * r;
       if (i <= t) { psi += term; dpsi = fma(term, r, dpsi); }
       else { phi += term; dphi = fma(term, r, dphi); }
     }
-    psi = rho * warp_sum(psi);
-    dpsi = rho * warp_sum(dpsi);
-    phi = rho * warp_sum(phi);
-    dphi = rho * warp_sum(dphi);
+    warp_sum4(psi, dpsi, phi, dphi);
+    psi *= rho;
+    dpsi *= rho;
+    phi *= rho;
+    dphi *= rho;
     const double f = 1.0 + psi + phi;
-    if (f < 0.0) blo = fmax(blo, tau); else bhi = fmin(bhi, tau);
-    if (f == 0.0 || bhi - blo <= 4.0 * kEps * fmax(fabs(blo), fabs(bhi))) break;
-    const double q = dpsi * (da - tau) * (da - tau);
-    const double pp = psi - dpsi * (da - tau);
-    double x;
+    if (f < 0.0) blo = tau; else bhi = tau;
+    if (!(fabs(f) > kEps * fma(8.0, 1.0 + phi - psi, fabs(tau) * (dpsi + dphi)))) break;
+    // zero of c + dpsi a^2 / (a - eta) + dphi b^2 / (b - eta), the function
+    // with f's value and the derivatives of psi and phi at tau, eta = x - tau
+    const double pa = da - tau, p1 = dpsi * pa;
+    double eta;
     if (t < k - 1) {
-      const double s = dphi * (db - tau) * (db - tau);
-      const double r = phi - dphi * (db - tau);
-      const double Cc = 1.0 + pp + r;
-      const double A2 = Cc, B2 = -(Cc * (da + db) + q + s), C2 = Cc * da * db + q * db + s * da;
-      x = 0.5 * (blo + bhi);
-      if (A2 == 0.0) {
-        if (B2 != 0.0) x = -C2 / B2;
-      } else {
-        const double disc = fmax(B2 * B2 - 4.0 * A2 * C2, 0.0);
-        const double sq = sqrt(disc);
-        const double r1 = (B2 >= 0.0) ? (-B2 - sq) / (2.0 * A2) : (-B2 + sq) / (2.0 * A2);
-        const double r2 = (r1 != 0.0) ? C2 / (A2 * r1) : r1;
-        if (r1 > da && r1 < db) x = r1;
-        else if (r2 > da && r2 < db) x = r2;
-      }
+      const double pb = db - tau, p2 = dphi * pb;
+      const double c = f - p1 - p2;
+      const double A2 = fma(c, pa + pb, fma(p1, pa, p2 * pb)), w = pa * pb * f;
+      const double disc = fmax(fma(A2, A2, -4.0 * w * c), 0.0);
+      double sq;
+      asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(sq) : "d"(disc));
+      sq = disc > 0.0 ? disc * sq : 0.0;
+      eta = A2 > 0.0 ? 2.0 * w * rcp_approx(A2 + sq) : (A2 - sq) * rcp_approx(2.0 * c);
     } else {
-      const double Cc = 1.0 + pp + phi;
-      x = (Cc > 0.0) ? da + q / Cc : 0.5 * (blo + bhi);
+      const double c = f - p1;                        // zero of c + dpsi a^2 / (a - eta)
+      eta = c > 0.0 ? pa * f * rcp_approx(c) : bhi - blo;
     }
+    double x = tau + eta;
     if (!(x > blo && x < bhi)) x = 0.5 * (blo + bhi);
-    if (fabs(x - tau) <= 2.0 * kEps * fabs(x)) { tau = x; break; }
+    if (x == tau || x == blo || x == bhi) { tau = x; break; }   // no double between the bounds
     tau = x;
   }
   if (lane == 0) {
@@ -1119,7 +1208,7 @@ __global__ void __launch_bounds__(256) k_dc_zhat(const int *nodes, DcArrays a) {
   double prod = 1.0;
   for (int j = lane; j < k; j += 32) {
     const double num = (D[a.orig[lo + j]] - Di) + a.tauK[lo + j];
-    prod *= (j == i) ? num : num / (D[j] - Di);
+    prod *= (j == i) ? num : div_newton(num, D[j] - Di);
   }
   prod = warp_prod(prod);
   if (lane == 0) {
@@ -1139,37 +1228,44 @@ __global__ void __launch_bounds__(256) k_dc_vectors(const int *nodes, int n, DcA
   const double *D = a.DK + lo;
   const double Do = D[a.orig[lo + t]], tau = a.tauK[lo + t];
   double s = 0.0;
+  double *Ucol = a.U + (long)(lo + t) * n + lo;
   for (int i = lane; i < k; i += 32) {
-    const double u = a.zh[lo + i] / ((D[i] - Do) - tau);
-    s += u * u;
+    const double u = div_newton(a.zh[lo + i], (D[i] - Do) - tau);
+    Ucol[i] = u;
+    s = fma(u, u, s);
   }
   const double inv = 1.0 / sqrt(warp_sum(s));
-  double *Ucol = a.U + (long)(lo + t) * n + lo;
-  for (int i = lane; i < k; i += 32) Ucol[i] = inv * a.zh[lo + i] / ((D[i] - Do) - tau);
+  for (int i = lane; i < k; i += 32) Ucol[i] *= inv;      // the lane's own entries
 }
 
 // W[rows, lo + t] = Z[rows, colK] U[:, t]  (node rows lo..hi-1).  Z is block
 // diagonal apart from the columns a deflating rotation mixed, so row tiles of
 // the upper half run over the root columns qL only, those of the lower half
 // over qR; only the roots t < kneed are formed.
+// Tile of 16 R x 16 R outputs per CTA, R x R per thread: the FP64 pipe is the
+// bound whatever the tile, so the tile only has to fill the SMs -- R = 4 where
+// a level has tiles enough, R = 1 for the small nodes (at order 54 one 64 x 64
+// tile kept one SM busy for 27 us).
+template <int R>
 __global__ void __launch_bounds__(256) k_dc_gemm(const int *nodes, int n, DcArrays a) {
+  constexpr int T = 16 * R;
   const int node = blockIdx.z;
   const int lo = nodes[3 * node], mid = nodes[3 * node + 1], hi = nodes[3 * node + 2];
-  const int tl = (mid - lo + 63) / 64;
+  const int tl = (mid - lo + T - 1) / T;
   const bool upper = (int)blockIdx.x < tl;
-  const int rbeg = upper ? lo + (int)blockIdx.x * 64 : mid + ((int)blockIdx.x - tl) * 64;
+  const int rbeg = upper ? lo + (int)blockIdx.x * T : mid + ((int)blockIdx.x - tl) * T;
   const int rend = upper ? mid : hi;
   const int kneed = a.kneed[node];
-  const int t0 = blockIdx.y * 64;
+  const int t0 = blockIdx.y * T;
   if (rbeg >= rend || t0 >= kneed) return;
   const int *ql = upper ? a.qL + lo : a.qR + lo;
   const int kq = a.kLR[2 * node + (upper ? 0 : 1)];
-  __shared__ double As[16][65], Bs[16][65];
+  __shared__ double As[16][T + 1], Bs[16][T + 1];
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  double acc[4][4] = {};
+  double acc[R][R] = {};
   for (int k0 = 0; k0 < kq; k0 += 16) {
-    for (int e = threadIdx.x; e < 1024; e += 256) {
-      const int r = e & 63, kk = e >> 6;
+    for (int e = threadIdx.x; e < 16 * T; e += 256) {
+      const int r = e % T, kk = e / T;
       double v = 0.0;
       if (rbeg + r < rend && k0 + kk < kq) v = a.Z[(rbeg + r) + (long)a.colK[lo + ql[k0 + kk]] * n];
       As[kk][r] = v;
@@ -1181,23 +1277,33 @@ __global__ void __launch_bounds__(256) k_dc_gemm(const int *nodes, int n, DcArra
     __syncthreads();
 #pragma unroll
     for (int kk = 0; kk < 16; ++kk) {
-      double av[4], bv[4];
+      double av[R], bv[R];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) { av[q] = As[kk][tx + 16 * q]; bv[q] = Bs[kk][ty + 16 * q]; }
+      for (int q = 0; q < R; ++q) { av[q] = As[kk][tx + 16 * q]; bv[q] = Bs[kk][ty + 16 * q]; }
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
+      for (int q = 0; q < R; ++q)
 #pragma unroll
-        for (int r = 0; r < 4; ++r) acc[q][r] = fma(av[q], bv[r], acc[q][r]);
+        for (int r = 0; r < R; ++r) acc[q][r] = fma(av[q], bv[r], acc[q][r]);
     }
     __syncthreads();
   }
 #pragma unroll
-  for (int q = 0; q < 4; ++q)
+  for (int q = 0; q < R; ++q)
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
+    for (int r = 0; r < R; ++r) {
       const int row = rbeg + tx + 16 * q, t = t0 + ty + 16 * r;
       if (row < rend && t < kneed) a.W[row + (long)(lo + t) * n] = acc[q][r];
     }
+}
+template <int R>
+void launch_dc_gemm(const int *nodes, int nn, int maxsize, int cols, int n, const DcArrays &a, cudaStream_t st) {
+  constexpr int T = 16 * R;
+  k_dc_gemm<R><<<dim3((maxsize + T - 1) / T + 1, (cols + T - 1) / T, nn), 256, 0, st>>>(nodes, n, a);
+}
+// 16 R x 16 R tiles of a level's merge products
+long dc_tiles(int R, int nn, int maxsize, int cols) {
+  const long T = 16 * R;
+  return nn * ((maxsize + T - 1) / T) * ((cols + T - 1) / T);
 }
 
 // The merge product of k_dc_gemm for one node and half (upper rows lo..mid
@@ -1242,10 +1348,12 @@ __global__ void k_dc_rank(const int *nodes, DcArrays a, int keep) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= size) return;
   const double v = e < k ? a.lamK[lo + e] : a.dD[lo + e - k];
+  const long long vb = ordered_bits(v);
   int rank = 0;
+#pragma unroll 8
   for (int f = 0; f < size; ++f) {
-    const double w = f < k ? a.lamK[lo + f] : a.dD[lo + f - k];
-    rank += (w < v) || (w == v && f < e);
+    const long long w = ordered_bits(f < k ? a.lamK[lo + f] : a.dD[lo + f - k]);
+    rank += (w < vb) || (w == vb && f < e);
   }
   a.lnew[lo + rank] = v;
   a.src[lo + rank] = lo + e;     // W column: roots at lo..lo+k-1, deflated copied after them
@@ -1711,7 +1819,11 @@ pw_status stage_dc(pw_dense_ws *ws, int n, int nb, double *lam, cudaStream_t st)
       }
     } else {
       pw_count_launch();
-      k_dc_gemm<<<dim3((maxsize + 63) / 64 + 1, (maxsize + 63) / 64, nn), 256, 0, st>>>(nodes, n, a);
+      // the largest tile that still gives every SM four
+      const int cols = std::min(maxsize, keep);
+      if (dc_tiles(4, nn, maxsize, cols) >= 4 * 152) launch_dc_gemm<4>(nodes, nn, maxsize, cols, n, a, st);
+      else if (dc_tiles(2, nn, maxsize, cols) >= 4 * 152) launch_dc_gemm<2>(nodes, nn, maxsize, cols, n, a, st);
+      else launch_dc_gemm<1>(nodes, nn, maxsize, cols, n, a, st);
     }
     pw_count_launch();
     k_dc_copy_defl<<<dim3(maxsize, nn), 128, 0, st>>>(nodes, n, a);
