@@ -880,13 +880,33 @@ __global__ void k_last_diag_plain(const double2 *A, int n, double *d) {
 // divide and conquer on the symmetric tridiagonal (d, e)
 // ======================================================================
 
-// leaves of size 1: every boundary is a split, so d_i loses |e_{i-1}| + |e_i|
-__global__ void k_dc_init(const double *d, const double *e, int n, double *lam, double *Z) {
+// leaves of size 1: every boundary is a split, so d_i loses |e_{i-1}| + |e_i|.
+// The tridiagonal is scaled by a power of two to entries of at most 1 (scale[0];
+// scale[1] undoes it in the root's k_dc_write): the secular equation squares
+// lengths down to 2^-53 of the largest and inverts them.
+__global__ void __launch_bounds__(256) k_dc_init(const double *d, const double *e, int n, double *lam, double *scale) {
+  __shared__ unsigned long long sh[8];
+  unsigned long long mb = 0;
+  for (int i = threadIdx.x; i < n; i += 256) {
+    mb = max(mb, (unsigned long long)(__double_as_longlong(d[i]) & 0x7FFFFFFFFFFFFFFFll));
+    if (i < n - 1) mb = max(mb, (unsigned long long)(__double_as_longlong(e[i]) & 0x7FFFFFFFFFFFFFFFll));
+  }
+  for (int o = 16; o > 0; o >>= 1) mb = max(mb, __shfl_xor_sync(0xffffffffu, mb, o));
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = mb;
+  __syncthreads();
+  for (int w = 0; w < 8; ++w) mb = max(mb, sh[w]);
+  // 2^(1022 - ex) and its inverse, both normal numbers (1 for a zero matrix)
+  const int ex = mb ? max(1, min(2043, (int)(mb >> 52))) : 1022;
+  const double sc = n == 1 ? 1.0 : __longlong_as_double((long long)(2045 - ex) << 52);
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0) {
+    scale[0] = sc;
+    scale[1] = n == 1 ? 1.0 : __longlong_as_double((long long)(ex + 1) << 52);
+  }
   if (i >= n) return;
-  double v = d[i];
-  if (i > 0) v -= fabs(e[i - 1]);
-  if (i < n - 1) v -= fabs(e[i]);
+  double v = d[i] * sc;
+  if (i > 0) v -= fabs(e[i - 1] * sc);
+  if (i < n - 1) v -= fabs(e[i] * sc);
   lam[i] = v;
 }
 __global__ void k_identity(double *Z, int n) {
@@ -901,6 +921,7 @@ struct DcArrays {
   int *perm, *colK, *orig, *dcol, *src, *defl;
   int *knode;
   double *rhonode;
+  double *scale;
   int *ctype, *qL, *qR, *kLR, *kneed;
 };
 
@@ -944,7 +965,7 @@ __global__ void __launch_bounds__(256) k_dc_deflate(const int *nodes, int n, con
   const int node = blockIdx.x;
   const int lo = nodes[3 * node], mid = nodes[3 * node + 1], hi = nodes[3 * node + 2];
   const int size = hi - lo, m1 = mid - lo;
-  const double beta = e[mid - 1];
+  const double beta = e[mid - 1] * a.scale[0];
   const double rho = fabs(beta), sgn = beta >= 0.0 ? 1.0 : -1.0;
   // 1. merge: left value -> its index + #(right < v); right -> index + #(left <= v)
   for (int p = threadIdx.x; p < size; p += blockDim.x) {
@@ -1372,12 +1393,12 @@ __global__ void k_dc_copy_defl(const int *nodes, int n, DcArrays a) {
   for (int r = lo + threadIdx.x; r < hi; r += blockDim.x) dst[r] = src[r];
 }
 
-__global__ void k_dc_write(const int *nodes, int n, DcArrays a, int keep) {
+__global__ void k_dc_write(const int *nodes, int n, DcArrays a, int keep, bool root) {
   const int node = blockIdx.y;
   const int lo = nodes[3 * node], hi = nodes[3 * node + 2];
   const int p = blockIdx.x;
   if (p >= hi - lo) return;
-  if (threadIdx.x == 0) a.lam[lo + p] = a.lnew[lo + p];
+  if (threadIdx.x == 0) a.lam[lo + p] = root ? a.lnew[lo + p] * a.scale[1] : a.lnew[lo + p];
   if (p >= keep) return;   // every eigenvalue, only the kept vectors
   const double *src = a.W + (long)a.src[lo + p] * n;
   double *dst = a.Z + (long)(lo + p) * n;
@@ -1698,6 +1719,9 @@ pw_status stage_tridiag(pw_dense_ws *ws, int n, double2 *A, cudaStream_t st) {
   const bool hs = (mode == 0 || mode == 3) && ws->hsl && pw_dense_products_mode() == 1 &&
                   n - 1 >= PW_HS_MIN_ORDER;
   const int hgrid = hs && mode == 3 ? pw_hs_panel_grid() : 0;
+  // the last columns (all of a small matrix) in one cluster
+  const int ncl = pw_house_cluster_max();
+  if (n <= ncl) return pw_house_cluster(ws, A, n, 0, st);
   // 1. Householder tridiagonalisation: panels of TPB columns (lower triangle)
   PW_CUDA(cudaMemsetAsync(ws->ticket, 0, sizeof(unsigned), st));
   if (hs) PW_CUDA(cudaMemsetAsync(ws->hsmax, 0, (size_t)(n / TPB + 2) * 8, st));
@@ -1705,6 +1729,10 @@ pw_status stage_tridiag(pw_dense_ws *ws, int n, double2 *A, cudaStream_t st) {
     const double2 mone = make_double2(-1.0, 0.0), one = make_double2(1.0, 0.0);
     double2 *dotpart = ws->w;
     for (int j0 = 0; j0 + 1 < n; j0 += TPB) {
+      if (n - j0 <= ncl) {
+        PW_TRY(pw_house_cluster(ws, A, n, j0, st));
+        return pw_check_launch("tridiag");
+      }
       const int b = std::min(TPB, n - 1 - j0);
       const bool ptc = hs && n - j0 - 1 >= PW_HS_MIN_ORDER;
       PW_CUDA(cudaMemsetAsync(ws->panel, 0, (size_t)n * 3 * b * sizeof(double2), st));
@@ -1764,9 +1792,9 @@ pw_status stage_dc(pw_dense_ws *ws, int n, int nb, double *lam, cudaStream_t st)
   DcArrays a{lam, ws->Z, ws->W, ws->U, ws->Ds, ws->zs, ws->DK, ws->zK, ws->tauK, ws->zh,
              ws->lamK, ws->dD, ws->lnew, ws->perm, ws->colK, ws->orig, ws->dcol, ws->src,
              (int *)ws->p /* defl scratch: n ints fit in n double2 */, ws->knode, ws->rhonode,
-             ws->ctype, ws->qL, ws->qR, ws->kLR, ws->kneed};
+             (double *)ws->hscal, ws->ctype, ws->qL, ws->qR, ws->kLR, ws->kneed};
   pw_count_launch();
-  k_dc_init<<<(n + 255) / 256, 256, 0, st>>>(ws->d, ws->e, n, lam, ws->Z);
+  k_dc_init<<<(n + 255) / 256, 256, 0, st>>>(ws->d, ws->e, n, lam, a.scale);
   pw_count_launch();
   k_identity<<<(unsigned)(((long)n * n + 255) / 256), 256, 0, st>>>(ws->Z, n);
   for (int l = (int)ws->levels.size() - 1; l >= 0; --l) {
@@ -1828,7 +1856,7 @@ pw_status stage_dc(pw_dense_ws *ws, int n, int nb, double *lam, cudaStream_t st)
     pw_count_launch();
     k_dc_copy_defl<<<dim3(maxsize, nn), 128, 0, st>>>(nodes, n, a);
     pw_count_launch();
-    k_dc_write<<<dim3(maxsize, nn), 128, 0, st>>>(nodes, n, a, keep);
+    k_dc_write<<<dim3(maxsize, nn), 128, 0, st>>>(nodes, n, a, keep, l == 0);
   }
   PW_TRY(pw_check_launch("divide and conquer"));
 

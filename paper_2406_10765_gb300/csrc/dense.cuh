@@ -100,6 +100,11 @@ pw_status pw_hs_hemv(pw_dense_ws *ws, const double2 *A, int n, int c, int i, int
 // panel [V | W | V], tau, d, e as the chained kernels and k_pfinal do.
 int pw_hs_panel_grid();
 pw_status pw_hs_panel(pw_dense_ws *ws, double2 *A, int n, int j0, int b, int grid, cudaStream_t st);
+// The reduction from column j0 on (order n - j0 <= pw_house_cluster_max(), the
+// trailing matrix up to date) in one thread-block cluster, leaving reflectors,
+// tau, d (to the last entry) and e as the chained kernels do.
+int pw_house_cluster_max();
+pw_status pw_house_cluster(pw_dense_ws *ws, double2 *A, int n, int j0, cudaStream_t st);
 // Runs `launch` (one cooperative launch on st) after the previous
 // cooperative launch on the current device, whatever its stream.
 pw_status pw_coop_ordered(cudaStream_t st, const std::function<pw_status()> &launch);
