@@ -1428,52 +1428,62 @@ __global__ void k_copy_panel(const double2 *A, int n, int j0, int b, double2 *Vb
 
 // T (b x b, upper, ld b): T_ii = tau_i; T[0:i, i] = -tau_i T[0:i, 0:i] G[0:i, i],
 // G = Vb^H Vb.  Row r of T depends only on itself (T[r, i] = -tau_i
-// sum_{m=r}^{i-1} T[r, m] G[m, i]), so each warp owns one row: the lanes split
-// the sum, the row is kept in shared memory, and the next column of G is
-// fetched while the current one is reduced.
+// sum_{m=r}^{i-1} T[r, m] G[m, i]), so each warp owns one row, and the sums are
+// kept for all later i at once, one i per lane: a finished entry T[r, m] is
+// broadcast and adds T[r, m] G[m, i] to every lane.  No reduction over lanes:
+// 14 FP64 instructions per entry instead of 35 (dot-product form: 158 us for b =
+// 128, 68 us for b = 53).  -tau_i is folded into the sums' columns at the start.
 constexpr int BT_WARPS = 4;
 __global__ void __launch_bounds__(32 * BT_WARPS) k_build_T(const double2 *G, const double2 *tau, int j0, int b,
                                                            double2 *T) {
-  __shared__ double2 trow[BT_WARPS][BTB];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int r = blockIdx.x * BT_WARPS + w;
   if (r >= b) return;
-  double2 *tr = trow[w];
   constexpr int KMAX = BTB / 32;
-  double2 gnext[KMAX];
-  auto fetch = [&](int col) {
+  double2 s[KMAX], mt[KMAX];       // columns lane + 32 k: sum, -tau
+#pragma unroll
+  for (int k = 0; k < KMAX; ++k) {
+    const int i = lane + 32 * k;
+    s[k] = make_double2(0.0, 0.0);
+    mt[k] = i < b ? tau[j0 + i] : make_double2(0.0, 0.0);
+    if (i == r) s[k] = mt[k];
+    mt[k] = make_double2(-mt[k].x, -mt[k].y);
+  }
+  double2 gn[KMAX];                // row m of G, fetched one entry ahead
+  auto fetch = [&](int m) {
 #pragma unroll
     for (int k = 0; k < KMAX; ++k) {
-      const int m = r + lane + 32 * k;
-      gnext[k] = (col < b && m < col) ? G[m + (long)col * b] : make_double2(0.0, 0.0);
+      const int i = lane + 32 * k;
+      gn[k] = m < b && i > m && i < b ? G[m + (long)i * b] : make_double2(0.0, 0.0);
     }
   };
-  if (lane == 0) tr[r] = tau[j0 + r];
-  fetch(r + 1);
-  __syncwarp();
-  for (int c = r + 1; c < b; ++c) {
-    double2 g[KMAX];
+  fetch(r);
 #pragma unroll
-    for (int k = 0; k < KMAX; ++k) g[k] = gnext[k];
-    fetch(c + 1);
-    double2 s = make_double2(0.0, 0.0);
+  for (int km = 0; km < KMAX; ++km) {
+    for (int m = max(r, 32 * km); m < min(b, 32 * km + 32); ++m) {
+      double2 g[KMAX];
 #pragma unroll
-    for (int k = 0; k < KMAX; ++k) {
-      const int m = r + lane + 32 * k;
-      if (m < c) cmac(s, tr[m], g[k]);
-    }
+      for (int k = 0; k < KMAX; ++k) g[k] = gn[k];
+      fetch(m + 1);
+      // the sum of column m is complete: T[r, m] (its diagonal is tau itself)
+      double2 t = m > r ? cmul(mt[km], s[km]) : s[km];
+      if (lane == (m & 31)) s[km] = t;
+      t.x = __shfl_sync(0xffffffffu, t.x, m & 31);
+      t.y = __shfl_sync(0xffffffffu, t.y, m & 31);
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      s.x += __shfl_xor_sync(0xffffffffu, s.x, off);
-      s.y += __shfl_xor_sync(0xffffffffu, s.y, off);
+      for (int k = km; k < KMAX; ++k)
+        if (32 * k + 31 > m && 32 * k < b) {
+          double2 u = s[k];
+          cmac(u, t, g[k]);
+          if (lane + 32 * k > m) s[k] = u;
+        }
     }
-    if (lane == 0) {
-      const double2 t = cmul(tau[j0 + c], s);
-      tr[c] = make_double2(-t.x, -t.y);
-    }
-    __syncwarp();
   }
-  for (int c = lane; c < b; c += 32) T[r + (long)c * b] = c >= r ? tr[c] : make_double2(0.0, 0.0);
+#pragma unroll
+  for (int k = 0; k < KMAX; ++k) {
+    const int i = lane + 32 * k;
+    if (i < b) T[r + (long)i * b] = i >= r ? s[k] : make_double2(0.0, 0.0);
+  }
 }
 
 void build_tree(pw_dense_ws *ws, int n, cudaStream_t st) {
