@@ -374,10 +374,11 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 // sum of the K-split parts (in part order), then alpha, beta; same element
 // selection as the single-part epilogue
 __global__ void k_oz_reduce(const double2 *__restrict__ part, int splits, int m, int n, double2 alpha,
-                            double2 beta, double2 *__restrict__ C, int ldc) {
+                            double2 beta, double2 *__restrict__ C, int ldc, int herm, int ioff, int joff) {
   const long idx = blockIdx.x * (long)blockDim.x + threadIdx.x;
   if (idx >= (long)m * n) return;
   const int i = (int)(idx % m), j = (int)(idx / m);
+  if (herm == 1 && ioff + i > joff + j) return;     // mirrored later; tiles below the diagonal have no parts
   double2 s = make_double2(0.0, 0.0);
   for (int z = 0; z < splits; ++z) {
     const double2 v = part[(long)z * m * n + idx];
@@ -730,11 +731,16 @@ pw_status oz_block(pw_oz_ws *w, char opA, char opB, int mb, int nb, int k, doubl
     return PW_ERR_CUDA;
   PW_TRY(allow_smem());
   const int mtiles = arows / BM, ntiles = brows / BN, tiles = mtiles * ntiles;
-  // K split when the tiles alone leave SMs idle (>= 8 chunks per part)
+  // K split when the tiles alone leave SMs idle (herm 1: about half of them
+  // are skipped).  A part is at least two chunks, 12 steps of ~0.8 us, which is
+  // what its start and its share of the reduction cost; a tile alone on its SM
+  // takes ~1.1 us a step (S^H S of the 8-atom cell, 72 x 72 x 1,647: 227 us in
+  // one part, 28 us split).
   const int nch = (kblocks + CHUNK_KB - 1) / CHUNK_KB;
+  const int act = herm == 1 ? (tiles + 1) / 2 : tiles;
   int parts = 1;
-  if (herm == 0 && tiles < 152) {
-    parts = std::min({(2 * 152 + tiles - 1) / tiles, std::max(1, nch / 8), g_max_parts});
+  if (herm <= 1 && act < 152) {
+    parts = std::min({(2 * 152 + act - 1) / act, std::max(1, nch / 2), g_max_parts});
     const size_t pbytes = (size_t)parts * mb * nb * 16;
     if (parts > 1 && pbytes > w->part_bytes) {
       if (w->part) cudaFree(w->part);
@@ -753,7 +759,7 @@ pw_status oz_block(pw_oz_ws *w, char opA, char opB, int mb, int nb, int k, doubl
   if (parts > 1) {
     pw_count_launch();
     k_oz_reduce<<<(unsigned)(((long)mb * nb + 255) / 256), 256, 0, st>>>(w->part, parts, mb, nb, alpha, beta, C,
-                                                                          ldc);
+                                                                          ldc, herm, ioff, joff);
     PW_TRY(pw_check_launch("oz reduce"));
   }
   return PW_OK;
