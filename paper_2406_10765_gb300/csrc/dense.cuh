@@ -2,6 +2,7 @@
 #pragma once
 #include <functional>
 
+#include "house.cuh"
 #include "oz_gemm.cuh"
 #include "pw_internal.cuh"
 
@@ -44,7 +45,6 @@ struct pw_dense_ws {
   int last_key[3][2] = {{-1, -1}, {-1, -1}, {-1, -1}};
   // blocked back-transformation: reflector panel, its Gram, T, two work blocks
   double2 *Vb = nullptr, *Gv = nullptr, *Tb = nullptr, *Wk = nullptr, *Wk2 = nullptr;
-  unsigned *ticket = nullptr;   // last-block-done counter of the Householder steps
   // blocked Householder reduction: panel [V | W | V] (nmax x 3*32), partial
   // norms of a column, the panel correction dots
   double2 *panel = nullptr, *ucorr = nullptr, *hscal = nullptr;
@@ -55,6 +55,10 @@ struct pw_dense_ws {
   void *hsl = nullptr;
   unsigned long long *hsmax = nullptr;
   double *nrm_part = nullptr;
+  // chained columns: the finished column, the next one without its pending
+  // part, per-block partials (HhCol::dot, norms)
+  double2 *xcol = nullptr, *acol = nullptr;
+  double *hpart = nullptr;
   // host side tree for the current n
   int tree_n = -1;
   std::vector<std::vector<int>> levels;   // per level: flat (lo, mid, hi) triples
@@ -85,21 +89,23 @@ pw_status pw_dense_alloc(pw_dense_ws *ws, int nmax, int nbmax);
 // (hemv_tc.cu): used for the panels whose trailing order is at least
 // PW_HS_MIN_ORDER when the product mode is 1.  pw_hs_bytes: slice buffer
 // bytes for order nmax (0 below the threshold).  pw_hs_slice: the slices of
-// the trailing matrix of the panel starting at column j0.  pw_hs_hemv: the
-// product for column c (panel index i, width b): partials into ws->part
-// (*nslots slots per row, part[s * nmax + row] with the global row index),
-// ucorr and v into the panel, as the FP64 k_phemv does.
+// the trailing matrix of the panel starting at column j0.  The column product
+// on them (pw_hs_hemv) is declared in house.cuh.
 #define PW_HS_MIN_ORDER 1024
 size_t pw_hs_bytes(int nmax);
 pw_status pw_hs_slice(pw_dense_ws *ws, const double2 *A, int n, int j0, cudaStream_t st);
-pw_status pw_hs_hemv(pw_dense_ws *ws, const double2 *A, int n, int c, int i, int b, int j0, int *nslots,
-                     cudaStream_t st);
 // All columns of the panel at j0 (width b, trailing order >= PW_HS_MIN_ORDER,
 // its slices written) in one cooperative launch of `grid` CTAs (from
 // pw_hs_panel_grid, 0 when the device cannot hold one per SM), leaving the
-// panel [V | W | V], tau, d, e as the chained kernels and k_pfinal do.
+// panel [V | W | V], tau, d, e as the chained kernels do.
 int pw_hs_panel_grid();
 pw_status pw_hs_panel(pw_dense_ws *ws, double2 *A, int n, int j0, int b, int grid, cudaStream_t st);
+// All columns of the panel at j0 (width b) as chained kernels (house_cols.cu),
+// with the Hermitian products on the tensor cores (tc: the panel's slices are
+// written) or on the FP64 pipe; leaves the panel, tau, d, e as above.
+// pw_house_parts: blocks its arrays of partials hold.
+size_t pw_house_parts(int nmax);
+pw_status pw_house_panel(pw_dense_ws *ws, double2 *A, int n, int j0, int b, bool tc, cudaStream_t st);
 // The reduction from column j0 on (order n - j0 <= pw_house_cluster_max(), the
 // trailing matrix up to date) in one thread-block cluster, leaving reflectors,
 // tau, d (to the last entry) and e as the chained kernels do.

@@ -8,8 +8,8 @@
 // the slices instead of the FP64 matrix:
 //   * A22 2^eA = sum_p a_p 2^(-7p) (p = 1..8, the digit split of the
 //     FP64-accurate product, one scale for the whole trailing matrix), and
-//     v / 2 = sum_q b_q 2^(-7q) (|v| <= 1 for a Householder vector whose head
-//     is 1);
+//     x 2^ex = sum_q b_q 2^(-7q) for the vector x (the column itself, scaled
+//     by its norm);
 //   * the products a_p b_q with p + q = g (g = 2..9) are summed in one FP32
 //     tensor-memory accumulator per g: the B operand for slice p holds the
 //     digit q = g - p of v in its row for g, so all slices p of a tile
@@ -38,16 +38,17 @@
 // are stored as full Hermitian blocks and give only A v; off-diagonal tiles
 // give A v for their rows and A^H v for their columns.
 //
-// Kernel (k_hemv_tc, one column per launch, chained with k_pcol and k_prows
-// by programmatic dependent launch): persistent, one CTA per SM, each CTA a
+// Kernel (k_hemv_tc, one column per launch, chained with k_col_rows by
+// programmatic dependent launch): persistent, one CTA per SM, each CTA a
 // contiguous range of work units (tile, real or imaginary part, and for
 // short trailing orders a piece of its eight slices, so that every SM has
 // work).  Warp 0 = bulk-copy producer (six 32 KB stages), warp 1 = MMA
 // issuer (one thread), warps 2..5 = B-operand builders and epilogue, warps
-// 6..7 = v into the panel and the panel's correction dots; B operands and
-// accumulators are double-buffered, so a unit's MMAs run while the previous
-// unit's sums are read and the next unit's digits of v are written.  The
-// same roles run inside k_panel_tc, one cooperative launch per panel.
+// 6..9 = the finished column and the panel's correction dots on the otherwise
+// idle FP64 pipe; B operands and accumulators are double-buffered, so a unit's
+// MMAs run while the previous unit's sums are read and the next unit's digits
+// are written.  The same roles run inside k_panel_tc, one cooperative launch
+// per panel, on the reflector v.
 // Every mbarrier wait is bounded; on timeout the CTA records an error word
 // and leaves in order.
 #include <cuda_fp16.h>
@@ -87,12 +88,13 @@ template <int NS>
 struct HsL {
   static constexpr int OFF_B = NS * SUB;
   static constexpr int OFF_RED = OFF_B + 4 * BDIR;
-  static constexpr int OFF_BAR = OFF_RED + 64;
+  static constexpr int OFF_BAR = OFF_RED + 128;
   static constexpr int SMEM = OFF_BAR + (2 * NS + NBAR_FIXED) * 8 + 16 + 1024;
 };
 constexpr int NST_HEMV = 6;                  // one column per launch
 constexpr int NST_PANEL = 5;                 // cooperative panel (its column phases need static scratch)
-constexpr int NTHR = 256;                    // producer, MMA, 4 epilogue warps, 2 side warps
+constexpr int SIDE_WARPS = 4;
+constexpr int NTHR = 192 + 32 * SIDE_WARPS;  // producer, MMA, 4 epilogue warps, side warps
 constexpr int NTHR_PANEL = 256;
 static_assert(HsL<NST_HEMV>::SMEM <= 232448, "shared memory per CTA");
 static_assert(HsL<NST_PANEL>::SMEM + 8 * 1024 <= 232448, "shared memory per CTA");
@@ -173,28 +175,26 @@ __global__ void __launch_bounds__(256) k_hs_slice(const double2 *__restrict__ A,
   uint32_t wr[S][4], wi[S][4];
 #pragma unroll
   for (int k = 0; k < 8; k += 2) {
-    int dr[2][S], di[2][S];
+    double2 z[2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int r = I * HT + r8 * 8 + k + h;
-      double2 z = make_double2(0.0, 0.0);
+      z[h] = make_double2(0.0, 0.0);
       if (r < n && c < n && r >= j0 && c >= j0) {
-        if (r >= c) z = A[r + (long)c * n];
+        if (r >= c) z[h] = A[r + (long)c * n];
         else {
-          z = A[c + (long)r * n];
-          z.y = -z.y;
+          z[h] = A[c + (long)r * n];
+          z[h].y = -z[h].y;
         }
       }
-      digits_i(z.x, e, dr[h]);
-      digits_i(z.y, e, di[h]);
     }
+    uint32_t d[S];
+    digit_pairs(z[0].x, z[1].x, e, d);
 #pragma unroll
-    for (int p = 0; p < S; ++p) {
-      wr[p][k >> 1] = (uint32_t)__half_as_ushort(__int2half_rn(dr[0][p])) |
-                      ((uint32_t)__half_as_ushort(__int2half_rn(dr[1][p])) << 16);
-      wi[p][k >> 1] = (uint32_t)__half_as_ushort(__int2half_rn(di[0][p])) |
-                      ((uint32_t)__half_as_ushort(__int2half_rn(di[1][p])) << 16);
-    }
+    for (int p = 0; p < S; ++p) wr[p][k >> 1] = d[p];
+    digit_pairs(z[0].y, z[1].y, e, d);
+#pragma unroll
+    for (int p = 0; p < S; ++p) wi[p][k >> 1] = d[p];
   }
   const uint32_t off = sub_off(r8, cl);
   unsigned char *base = hsl + (size_t)tile_index(I, J) * 2 * UNIT + off;
@@ -214,7 +214,8 @@ struct HsSmem {
   uint64_t *bready, *mdone;    // [2] a unit's B operands built (and its accumulators free) / its MMAs done
   uint64_t *fin;
   uint32_t *tmem_slot;
-  double *red;                 // block-sum scratch
+  double *red;                 // block-sum scratch (8), then
+  uint32_t *vmax;              // [2][2][4] largest entries of a unit's two blocks per warp
   __device__ explicit HsSmem(unsigned char *smem) {
     base = smem;
     full = (uint64_t *)(smem + HsL<NS>::OFF_BAR);
@@ -224,6 +225,7 @@ struct HsSmem {
     fin = mdone + 2;
     tmem_slot = (uint32_t *)(fin + 1);
     red = (double *)(smem + HsL<NS>::OFF_RED);
+    vmax = (uint32_t *)(red + 8);
   }
 };
 
@@ -248,7 +250,6 @@ __device__ void hs_setup(const HsSmem<NS> &m) {
 
 // one CTA's share of one column's product
 struct HsCol {
-  const double2 *A;            // column c holds x (rows c + 1..)
   int n, c;
   long ub;                     // first unit of this CTA
   int nunit;                   // its units
@@ -365,27 +366,56 @@ __device__ __forceinline__ double2 refl_v(const double2 *xcol, int x, int m, dou
   return x == 0 ? make_double2(1.0, 0.0) : cmul(__ldcg(&xcol[x]), s);
 }
 
+// The vector of a product: entry(row), zero before row c + 1
+struct VecRefl {                       // the reflector v = x s below its unit head
+  const double2 *xk;
+  int o, mm;
+  double2 scal;
+  __device__ double2 entry(int r) const { return refl_v(xk, r - o, mm, scal); }
+};
+struct VecCol {                        // the column x
+  const HhCol &h;
+  double k2;
+  __device__ double2 entry(int r) const {
+    return r > h.c && r < h.n ? hh_x(h, r, k2) : make_double2(0.0, 0.0);
+  }
+};
+
 // Warps 2..5 (et = threadIdx.x - 64, the K entry of the B operands):
-// digits of v over unit u's tile columns (dir 0, A v) and rows (dir 1, A^H v)
-// into buffer ug & 1, rows 14..29 of the window layout
-template <int NS>
-__device__ void hs_build(const HsCol &w, const HsSmem<NS> &m, int u, int ug, double2 scal) {
+// digits of the vector over unit u's tile columns (dir 0, A v) and rows (dir
+// 1, A^H v) into buffer ug & 1, rows 14..29 of the window layout, each block of
+// 128 entries scaled by its own largest one; ev: the blocks' exponents
+template <int NS, class Vec>
+__device__ void hs_build(const HsCol &w, const HsSmem<NS> &m, int u, int ug, const Vec &vec, int (&ev)[2]) {
   const int et = threadIdx.x - 64;
-  const int o = w.c + 1, mm = w.n - o;
-  const double2 *xk = w.A + o + (long)w.c * w.n;
   const Unit un = unit_of(w.ub + u, w.ks);
-  const int ndir = un.I == un.J ? 1 : 2;
   const int I = un.I + w.J0, J = un.J + w.J0;
-  for (int dir = 0; dir < ndir; ++dir) {
-    const double2 v = refl_v(xk, (dir == 0 ? J : I) * HT + et - o, mm, scal);
-    int dr[S], di[S];
-    digits_i(v.x, -1, dr);
-    digits_i(v.y, -1, di);
-    __half *col = (__half *)(m.base + HsL<NS>::OFF_B + (2 * (ug & 1) + dir) * BDIR + (et >> 3) * BKC) + (et & 7);
+  const bool diag = un.I == un.J;
+  double2 v[2];
+  v[0] = vec.entry(J * HT + et);
+  v[1] = diag ? v[0] : vec.entry(I * HT + et);
+  // the exponents, from the high words of the largest entries of both blocks
+  uint32_t *mx = m.vmax + (ug & 1) * 8;
+#pragma unroll
+  for (int dir = 0; dir < 2; ++dir) {
+    const uint32_t hb = (uint32_t)(max(abs_bits(v[dir].x), abs_bits(v[dir].y)) >> 32);
+    const uint32_t wm = __reduce_max_sync(0xffffffffu, hb);
+    if ((et & 31) == 0) mx[dir * 4 + (et >> 5)] = wm;
+  }
+  named_sync(3, 128);
+#pragma unroll
+  for (int dir = 0; dir < 2; ++dir) {
+    const uint32_t hb = max(max(mx[dir * 4], mx[dir * 4 + 1]), max(mx[dir * 4 + 2], mx[dir * 4 + 3]));
+    ev[dir] = row_exp((unsigned long long)hb << 32);
+    if (dir == 1 && diag) break;
+    uint32_t d[S];
+    digit_pairs(v[dir].x, v[dir].y, ev[dir], d);
+    unsigned short *col =
+        (unsigned short *)(m.base + HsL<NS>::OFF_B + (2 * (ug & 1) + dir) * BDIR + (et >> 3) * BKC) + (et & 7);
 #pragma unroll
     for (int t = 0; t < S; ++t) {
-      col[(2 * (t + 7)) * 8] = __int2half_rn(dr[t]);
-      col[(2 * (t + 7) + 1) * 8] = __int2half_rn(di[t]);
+      col[(2 * (t + 7)) * 8] = (unsigned short)d[t];
+      col[(2 * (t + 7) + 1) * 8] = (unsigned short)(d[t] >> 16);
     }
   }
   // the B operands (generic-proxy writes) to the tensor core, and the
@@ -397,13 +427,12 @@ __device__ void hs_build(const HsCol &w, const HsSmem<NS> &m, int u, int ug, dou
 
 // warps 2..5: unit u's sums (buffer ug & 1) into the partial slots
 template <int NS>
-__device__ bool hs_epilogue(const HsCol &w, const HsSmem<NS> &m, uint32_t tmem, int u, int ug, int eA) {
+__device__ bool hs_epilogue(const HsCol &w, const HsSmem<NS> &m, uint32_t tmem, int u, int ug, int eA, const int (&ev)[2]) {
   if (!mbar_wait(&m.mdone[ug & 1], (uint32_t)(ug >> 1) & 1)) { atomicOr(w.err, 4); return false; }
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const int q4 = (threadIdx.x >> 5) & 3, lane = threadIdx.x & 31;   // tensor-memory lane quarter
   const uint32_t lanes = (uint32_t)(q4 * 32) << 16;
   const int o = w.c + 1;
-  const int ksc = -LFIX - eA + 1;               // value = acc 2^ksc (digits of v / 2)
   const Unit un = unit_of(w.ub + u, w.ks);
   const int part = un.part;
   const int I = un.I + w.J0, J = un.J + w.J0;
@@ -421,6 +450,7 @@ __device__ bool hs_epilogue(const HsCol &w, const HsSmem<NS> &m, uint32_t tmem, 
         R += shifted(f2i_exact(r[h * 16 + 2 * j]), sh);
         Q += shifted(f2i_exact(r[h * 16 + 2 * j + 1]), sh);
       }
+    const int ksc = -LFIX - eA - ev[dir];         // value = acc 2^ksc
     // A = Ar + i Ai, v = vr + i vi; rows (dir 0): Ar v -> (R, Q), i Ai v -> (-Q, R);
     // columns (dir 1, conj(A)^T v): Ar -> (R, Q), -i Ai -> (Q, -R)
     long long yr, yi;
@@ -437,16 +467,22 @@ __device__ bool hs_epilogue(const HsCol &w, const HsSmem<NS> &m, uint32_t tmem, 
 
 // warps 2..5 over the column: the first two units' B operands, then each
 // unit's sums before the B operands of the unit two later replace its buffer
-template <int NS>
-__device__ void hs_epi_start(const HsCol &w, const HsSmem<NS> &m, double2 scal, int ug) {
-  if (w.nunit > 0) hs_build(w, m, 0, ug, scal);
-  if (w.nunit > 1) hs_build(w, m, 1, ug + 1, scal);
-}
-template <int NS>
-__device__ void hs_epi_rest(const HsCol &w, const HsSmem<NS> &m, uint32_t tmem, double2 scal, int eA, int &ug) {
+template <int NS, class Vec>
+__device__ void hs_epi(const HsCol &w, const HsSmem<NS> &m, uint32_t tmem, const Vec &vec, int eA, int &ug) {
+  int e0[2], e1[2], e2[2];             // exponents of unit u, u + 1, u + 2
+  if (w.nunit > 0) hs_build(w, m, 0, ug, vec, e0);
+  if (w.nunit > 1) hs_build(w, m, 1, ug + 1, vec, e1);
+  // after a wait that ran out the warps go through the rest without waiting:
+  // hs_build's barrier needs all four of them
+  bool dead = false;
   for (int u = 0; u < w.nunit; ++u) {
-    if (hs_failed(w.err) || !hs_epilogue(w, m, tmem, u, ug + u, eA)) break;
-    if (u + 2 < w.nunit) hs_build(w, m, u + 2, ug + u + 2, scal);
+    if (!dead) dead = hs_failed(w.err) || !hs_epilogue(w, m, tmem, u, ug + u, eA, e0);
+    if (u + 2 < w.nunit) hs_build(w, m, u + 2, ug + u + 2, vec, e2);
+#pragma unroll
+    for (int d = 0; d < 2; ++d) {
+      e0[d] = e1[d];
+      e1[d] = e2[d];
+    }
   }
   ug += w.nunit;
 }
@@ -495,10 +531,9 @@ __device__ void hs_side(const HsSide &a, double2 scal, double *red, int id, int 
 
 // ------------------------------------------------ one column per launch ----
 struct HsArgs {
-  HsSide side;
+  HhCol h;
   const unsigned char *hsl;    // slices of the panel's trailing tiles
   const unsigned long long *slot;   // max bits of the trailing matrix (its scale)
-  const double2 *hscal;        // reflector scale s (v = x s below the unit head)
   double2 *part;               // tile partials [slot][nmax]
   int nmax;
   int J0, ks, units;           // first trailing tile, pieces per (tile, part), units
@@ -511,9 +546,8 @@ __global__ void __launch_bounds__(NTHR, 1) k_hemv_tc(const __grid_constant__ HsA
   const HsSmem<NS> m((unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   HsCol w;
-  w.A = a.side.A;
-  w.n = a.side.n;
-  w.c = a.side.c;
+  w.n = a.h.n;
+  w.c = a.h.c;
   hs_range(a.units, w.ub, w.nunit);
   w.J0 = a.J0;
   w.ks = a.ks;
@@ -530,8 +564,8 @@ __global__ void __launch_bounds__(NTHR, 1) k_hemv_tc(const __grid_constant__ HsA
 
   if (warp == 0) {
     if (lane == 0) {
-      // the slices were written before the panel's first column, two or more
-      // launches back, so the producer needs no dependency wait
+      // the slices were written before the panel's first column, which is
+      // launched without overlap, so the producer needs no dependency wait
       int k = 0;
       uint32_t issued = 0, last_ph = 0;
       hs_produce(w, m, 0, hs_subtiles(w), k, issued, last_ph);
@@ -543,18 +577,34 @@ __global__ void __launch_bounds__(NTHR, 1) k_hemv_tc(const __grid_constant__ HsA
       hs_mma(w, m, tmem, k, ug);
       hs_mma_finish(m, w.err);
     }
-  } else if (warp < 6) {
-    pdl_wait();
-    pdl_trigger();
-    const double2 scal = *a.hscal;
-    const int eA = row_exp(*a.slot);
-    int ug = 0;
-    hs_epi_start(w, m, scal, ug);
-    hs_epi_rest(w, m, tmem, scal, eA, ug);
   } else {
     pdl_wait();
     pdl_trigger();
-    hs_side(a.side, *a.hscal, m.red, 1, 64, threadIdx.x - 192);
+    // the previous column's k2, by one warp
+    if (warp == 6) {
+      const double k = hh_k2(a.h);
+      if (lane == 0) m.red[0] = k;
+    }
+    named_sync(1, NTHR - 64);
+    const double k2 = m.red[0];
+    if (warp < 6) {
+      const VecCol vec{a.h, k2};
+      int ug = 0;
+      hs_epi(w, m, tmem, vec, row_exp(*a.slot), ug);
+    } else {
+      // the finished column (a share of the rows per CTA, warp 6), then the
+      // dots, one (dot, chunk) per warp
+      if (warp == 6) {
+        const int rows = a.h.n - a.h.c, per = (rows + gridDim.x - 1) / gridDim.x;
+        const int r1 = min(a.h.n, a.h.c + (int)(blockIdx.x + 1) * per);
+        double s = 0.0;
+        for (int r = a.h.c + blockIdx.x * per + lane; r < r1; r += 32) s += hh_row(a.h, k2, r);
+        s = warp_sum(s);
+        if (lane == 0) a.h.nrm[blockIdx.x] = s;
+      }
+      for (int u = blockIdx.x + gridDim.x * (warp - 6); u < 2 * a.h.i * HH_CHUNKS; u += gridDim.x * SIDE_WARPS)
+        hh_dot(a.h, k2, u / HH_CHUNKS, u % HH_CHUNKS);
+    }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -579,8 +629,6 @@ __global__ void __launch_bounds__(NTHR, 1) k_hemv_tc(const __grid_constant__ HsA
 //      of x, partial dots p^H v;
 //   -- barrier --
 // The first stages of a column's slices are requested during its phase A.
-// The same arithmetic as the chained kernels (k_pcol, the product, k_prows)
-// up to the order of the column update's sums.
 struct PanelArgs {
   double2 *A;
   int n, j0, b;
@@ -625,7 +673,6 @@ __global__ void __launch_bounds__(NTHR_PANEL, 1) k_panel_tc(const __grid_constan
   for (int i = 0; i < b; ++i) {
     const int c = a.j0 + i, o = c + 1, mrow = n - o;
     HsCol w;
-    w.A = a.A;
     w.n = n;
     w.c = c;
     w.J0 = o / HT;
@@ -643,7 +690,7 @@ __global__ void __launch_bounds__(NTHR_PANEL, 1) k_panel_tc(const __grid_constan
       hs_produce(w, m, 0, pos0, kprod, issued, last_ph);
     }
     // ---- phase A: column c receives the panel's earlier rank-2 updates.
-    // Two 32-row blocks per pass, four warps each, in k_pcol's order.
+    // Two 32-row blocks per pass, four warps each.
     double2 al = make_double2(0.0, 0.0);
     if (i > 0) {
       al = panel_alpha(a.dotpart, ndot, tk, sh, 128);   // tk: tau of column c - 1
@@ -698,8 +745,7 @@ __global__ void __launch_bounds__(NTHR_PANEL, 1) k_panel_tc(const __grid_constan
       __syncthreads();
     }
     grid.sync();
-    // reflector scalars from x = A[c+1:, c] (every block, in the order of
-    // k_pcol's last block)
+    // reflector scalars from x = A[c+1:, c] (every block)
     {
       const double2 alpha = __ldcg(&a.A[(c + 1) + (long)c * n]);
       if (g == 0) {
@@ -726,8 +772,8 @@ __global__ void __launch_bounds__(NTHR_PANEL, 1) k_panel_tc(const __grid_constan
     } else if (warp == 1) {
       if (lane == 0) hs_mma(w, m, tmem, kmma, ug_mma);
     } else if (warp < 6) {
-      hs_epi_start(w, m, scal, ug_epi);
-      hs_epi_rest(w, m, tmem, scal, eA, ug_epi);
+      const VecRefl vec{a.A + o + (long)c * n, o, mrow, scal};
+      hs_epi(w, m, tmem, vec, eA, ug_epi);
     } else {
       HsSide sd;
       sd.A = a.A;
@@ -846,24 +892,16 @@ pw_status pw_hs_slice(pw_dense_ws *ws, const double2 *A, int n, int j0, cudaStre
   return pw_check_launch("householder slices");
 }
 
-pw_status pw_hs_hemv(pw_dense_ws *ws, const double2 *A, int n, int c, int i, int b, int j0, int *nslots,
-                     cudaStream_t st) {
+pw_status pw_hs_hemv(pw_dense_ws *ws, const HhCol &h, int j0, int *nslots, int *nnrm, cudaStream_t st) {
   PW_TRY(allow_smem());
   HsArgs a;
-  a.side.A = A;
-  a.side.n = n;
-  a.side.c = c;
-  a.side.i = i;
-  a.side.b = b;
-  a.side.P = ws->panel;
-  a.side.ucorr = ws->ucorr;
+  a.h = h;
   a.hsl = (const unsigned char *)ws->hsl;
   a.slot = ws->hsmax + j0 / 32;
-  a.hscal = ws->hscal;
   a.part = ws->part;
   a.nmax = ws->nmax;
-  a.J0 = (c + 1) / HT;
-  const int ntp = (n + HT - 1) / HT - a.J0;
+  a.J0 = (h.c + 1) / HT;
+  const int ntp = (h.n + HT - 1) / HT - a.J0;
   // pieces per (tile, part): enough units for every SM, within the partial
   // slots ws->part holds ((nmax + 31) / 32)
   const int sms = sm_count();
@@ -872,6 +910,7 @@ pw_status pw_hs_hemv(pw_dense_ws *ws, const double2 *A, int n, int c, int i, int
   a.err = ws->oz.err;
   *nslots = 2 * ntp * a.ks;
   const int grid = std::min(a.units, sms);
+  *nnrm = grid;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(NTHR);
@@ -881,7 +920,7 @@ pw_status pw_hs_hemv(pw_dense_ws *ws, const double2 *A, int n, int c, int i, int
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = h.i > 0 ? 1 : 0;      // the panel's first column: after the slicing
   pw_count_launch();
   PW_CUDA(cudaLaunchKernelEx(&cfg, k_hemv_tc, a));
   return PW_OK;

@@ -3,9 +3,9 @@
 // the trailing matrix in distributed shared memory: the whole reduction of
 // small orders, and the end of larger ones.
 //
-// Why: a column of the chained kernels (k_pcol, k_phemv, k_prows) costs about
-// 18 us at small orders, three dependent launches whose reductions, square
-// roots and divisions run in FP64 one after the other (a warp-wide FP64
+// Why: a column of chained kernels cost about 18 us at small orders (three
+// dependent launches; 10 with the two of house_cols.cu), whose reductions,
+// square roots and divisions run in FP64 one after the other (a warp-wide FP64
 // instruction takes 65 clocks on this part whatever the number of its active
 // lanes, a division 700).  Sixteen CTAs that exchange vectors through
 // distributed shared memory need two cluster barriers (400 clocks each) per
@@ -50,45 +50,6 @@ constexpr int HC_MAX = 256;
 size_t hc_smem(int m) {
   return ((size_t)((m + HC_CTAS - 1) / HC_CTAS) * m + 4 * (size_t)m + 2) * sizeof(double2) +
          2 * HC_CTAS * HC_WARPS * sizeof(double) + 64;
-}
-
-// sum of a complex value over the warp, the lanes split between its parts
-// after the first exchange: five additions instead of ten
-__device__ __forceinline__ double2 warp_sum_c(double2 s) {
-  const bool hi = threadIdx.x & 16;
-  double v = (hi ? s.y : s.x) + __shfl_xor_sync(0xffffffffu, hi ? s.x : s.y, 16);
-  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return make_double2(__shfl_sync(0xffffffffu, v, 0), __shfl_sync(0xffffffffu, v, 16));
-}
-
-// reflector_scalars with Newton steps on the hardware's approximate reciprocal
-// square root and reciprocal (cubic each, then the square root's remainder):
-// about an ulp, a third of the time; outside the range where the squares are
-// normal numbers the rounded operations
-__device__ __forceinline__ void reflector_scalars_fast(double xn2, double2 alpha, double &beta, double2 &tk,
-                                                       double2 &scal) {
-  const double s2 = fma(alpha.x, alpha.x, fma(alpha.y, alpha.y, xn2));
-  if ((xn2 == 0.0 && alpha.y == 0.0) || !(s2 > 1e-280 && s2 < 1e280)) {
-    reflector_scalars(xn2, alpha, beta, tk, scal);
-    return;
-  }
-  double r;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(s2));
-  const double h = fma(-s2 * r, r, 1.0);               // r = (1 - h / 2 + ..) / sqrt(s2)
-  r = fma(r * h, fma(h, 0.375, 0.5), r);
-  const double b = s2 * r;
-  const double nrm = fma(fma(-b, b, s2), 0.5 * r, b);
-  const double sg = alpha.x < 0.0 || (alpha.x == 0.0 && signbit(alpha.x)) ? 1.0 : -1.0;
-  beta = sg * nrm;
-  const double ib = sg * r;
-  const double dx = alpha.x - beta;                    // no cancellation: opposite signs
-  tk = make_double2(-dx * ib, -alpha.y * ib);
-  const double dd = fma(dx, dx, alpha.y * alpha.y);
-  double q;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(q) : "d"(dd));
-  const double e = fma(-dd, q, 1.0);
-  q = fma(q, fma(e, e, e), q);
-  scal = make_double2(dx * q, -alpha.y * q);
 }
 
 __global__ void __launch_bounds__(HC_THREADS) k_house_cluster(double2 *A, int n, int j0, double2 *tau, double *d,

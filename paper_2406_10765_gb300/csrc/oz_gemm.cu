@@ -409,6 +409,26 @@ __global__ void k_oz_mirror(double2 *C, int ldc, int n) {
 // conjugated if conj.  bside = 0: one real row r = (re, im) over K' = 2k;
 // bside = 1: two real rows 2r = (re, -im), 2r + 1 = (im, re).
 // out: [S][rows_total][kpad] FP16, e: row exponents (one per complex row).
+// Bound: memory (48 or 80 bytes per element); S^H S and S^H (H S) of the
+// 216-atom cell's FP64 step were at a fifth of it while each digit was peeled
+// and converted on its own.
+__device__ __forceinline__ void store_slices(double re, double im, int ex, int bside, int r, int t, int kpad,
+                                             long slice, __half *__restrict__ out) {
+  uint32_t d[S];
+  digit_pairs(re, im, ex, d);
+  if (!bside) {
+    __half *o = out + (long)r * kpad + 2 * t;
+#pragma unroll
+    for (int p = 0; p < S; ++p) *(uint32_t *)(o + p * slice) = d[p];
+  } else {
+    __half *o0 = out + (long)(2 * r) * kpad + 2 * t, *o1 = o0 + kpad;
+#pragma unroll
+    for (int p = 0; p < S; ++p) {
+      *(uint32_t *)(o0 + p * slice) = d[p] ^ 0x80000000u;            // (re, -im)
+      *(uint32_t *)(o1 + p * slice) = __byte_perm(d[p], 0, 0x1032);  // (im, re)
+    }
+  }
+}
 __global__ void __launch_bounds__(256) k_oz_slice_contig(const double2 *__restrict__ X, int ld, int k, int conj,
                                                          int bside, int kpad, int rows_total,
                                                          __half *__restrict__ out, int *__restrict__ e) {
@@ -436,21 +456,7 @@ __global__ void __launch_bounds__(256) k_oz_slice_contig(const double2 *__restri
       re = v.x;
       im = conj ? -v.y : v.y;
     }
-    __half dr[S], di[S];
-    digits(re, ex, dr);
-    digits(im, ex, di);
-    if (!bside) {
-      __half *o = out + (long)r * kpad + 2 * t;
-#pragma unroll
-      for (int p = 0; p < S; ++p) *(__half2 *)(o + p * slice) = __halves2half2(dr[p], di[p]);
-    } else {
-      __half *o0 = out + (long)(2 * r) * kpad + 2 * t, *o1 = o0 + kpad;
-#pragma unroll
-      for (int p = 0; p < S; ++p) {
-        *(__half2 *)(o0 + p * slice) = __halves2half2(dr[p], __hneg(di[p]));
-        *(__half2 *)(o1 + p * slice) = __halves2half2(di[p], dr[p]);
-      }
-    }
+    store_slices(re, im, ex, bside, r, t, kpad, slice, out);
   }
 }
 
@@ -507,21 +513,7 @@ __global__ void __launch_bounds__(256) k_oz_slice_strided(const double2 *__restr
       const int t = t0 + tt;
       if (2 * t >= kpad) continue;
       const double2 v = tileS[tt][rr];
-      __half dr[S], di[S];
-      digits(v.x, ex, dr);
-      digits(v.y, ex, di);
-      if (!bside) {
-        __half *o = out + (long)r * kpad + 2 * t;
-#pragma unroll
-        for (int p = 0; p < S; ++p) *(__half2 *)(o + p * slice) = __halves2half2(dr[p], di[p]);
-      } else {
-        __half *o0 = out + (long)(2 * r) * kpad + 2 * t, *o1 = o0 + kpad;
-#pragma unroll
-        for (int p = 0; p < S; ++p) {
-          *(__half2 *)(o0 + p * slice) = __halves2half2(dr[p], __hneg(di[p]));
-          *(__half2 *)(o1 + p * slice) = __halves2half2(di[p], dr[p]);
-        }
-      }
+      store_slices(v.x, v.y, ex, bside, r, t, kpad, slice, out);
     }
   }
 }
@@ -549,12 +541,11 @@ __global__ void __launch_bounds__(256) k_ozr_slice_contig(const double *__restri
   const long slice = (long)rows_total * kpad;
   for (int t2 = threadIdx.x; t2 < kpad / 2; t2 += blockDim.x) {
     const int t = 2 * t2;
-    __half d0[S], d1[S];
-    digits(t < k ? x[t] : 0.0, ex, d0);
-    digits(t + 1 < k ? x[t + 1] : 0.0, ex, d1);
+    uint32_t d[S];
+    digit_pairs(t < k ? x[t] : 0.0, t + 1 < k ? x[t + 1] : 0.0, ex, d);
     __half *o = out + (long)r * kpad + t;
 #pragma unroll
-    for (int p = 0; p < S; ++p) *(__half2 *)(o + p * slice) = __halves2half2(d0[p], d1[p]);
+    for (int p = 0; p < S; ++p) *(uint32_t *)(o + p * slice) = d[p];
   }
 }
 __global__ void __launch_bounds__(256) k_ozr_rowmax(const double *__restrict__ X, int ld, int nrows, int k,
@@ -594,12 +585,11 @@ __global__ void __launch_bounds__(256) k_ozr_slice_strided(const double *__restr
     if (blockIdx.y == 0 && tx == 0) e[r] = ex;
     const int t = t0 + 2 * tx;
     if (t >= kpad) continue;
-    __half d0[S], d1[S];
-    digits(tileS[2 * tx][rr], ex, d0);
-    digits(tileS[2 * tx + 1][rr], ex, d1);
+    uint32_t d[S];
+    digit_pairs(tileS[2 * tx][rr], tileS[2 * tx + 1][rr], ex, d);
     __half *o = out + (long)r * kpad + t;
 #pragma unroll
-    for (int p = 0; p < S; ++p) *(__half2 *)(o + p * slice) = __halves2half2(d0[p], d1[p]);
+    for (int p = 0; p < S; ++p) *(uint32_t *)(o + p * slice) = d[p];
   }
 }
 
