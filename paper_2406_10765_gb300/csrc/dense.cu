@@ -1242,8 +1242,7 @@ pw_status pw_dense_gemm(pw_dense_ws *ws, char opA, char opB, int m, int n, int k
                                   std::max(pw_oz_ws_bytes(ws->nmax, 256, ws->nmax),
                                            pw_oz_ws_bytes(ws->nmax, ws->nbmax, ws->nmax)));
       void *p = nullptr;
-      if (cudaMalloc(&p, big) == cudaSuccess) { ws->oz.buf = p; ws->oz.bytes = big; ++ws->oz.gen; }
-      else cudaGetLastError();
+      if (pw_mem_alloc(ws->oz.mem, &p, big) == cudaSuccess) { ws->oz.buf = p; ws->oz.bytes = big; ++ws->oz.gen; }
     }
     return pw_zgemm_oz(&ws->oz, opA, opB, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, st, herm);
   }
@@ -1259,9 +1258,11 @@ pw_status pw_dense_alloc(pw_dense_ws *ws, int nmax, int nbmax) {
   pw_dense_free(ws);
   const size_t n2 = (size_t)nmax * nmax;
   size_t total = 0;
+  // one allocation for all of them: the buffers' offsets first
+  std::vector<std::pair<void **, size_t>> bufs;
   auto get = [&](void **p, size_t bytes) -> bool {
-    if (cudaMalloc(p, bytes) != cudaSuccess) { cudaGetLastError(); *p = nullptr; return false; }
-    total += bytes;
+    bufs.push_back({p, total});
+    total += (bytes + 255) / 256 * 256;
     return true;
   };
   bool ok = get((void **)&ws->G, n2 * 16) && get((void **)&ws->A, n2 * 16) &&
@@ -1288,14 +1289,8 @@ pw_status pw_dense_alloc(pw_dense_ws *ws, int nmax, int nbmax) {
        get((void **)&ws->nrm_part, (size_t)(nmax / 32 + 2) * 8) &&
        get((void **)&ws->hsmax, (size_t)(nmax / TPB + 2) * 8) && get((void **)&ws->xcol, (size_t)nmax * 16) &&
        get((void **)&ws->acol, (size_t)nmax * 16) && get((void **)&ws->hpart, 2 * pw_house_parts(nmax) * 8);
-  if (ok && pw_hs_bytes(nmax)) {
-    // zeroed once: a slice tile is only read where the panel's slicing wrote it
-    ok = get(&ws->hsl, pw_hs_bytes(nmax)) && cudaMemset(ws->hsl, 0, pw_hs_bytes(nmax)) == cudaSuccess;
-  }
-  if (ok && !ws->oz.err) {
-    ok = cudaMalloc((void **)&ws->oz.err, 16) == cudaSuccess && cudaMemset(ws->oz.err, 0, 16) == cudaSuccess;
-    if (!ok) { cudaGetLastError(); ws->oz.err = nullptr; }
-  }
+  // a slice tile is only read where the panel's slicing wrote it
+  if (pw_hs_bytes(nmax)) ok = ok && get(&ws->hsl, pw_hs_bytes(nmax));
   ok = ok && get((void **)&ws->Vb, (size_t)nmax * BTB * 16) && get((void **)&ws->Gv, BTB * BTB * 16) &&
        get((void **)&ws->Tb, BTB * BTB * 16) && get((void **)&ws->Wk, (size_t)BTB * nbmax * 16) &&
        get((void **)&ws->Wk2, (size_t)BTB * nbmax * 16);
@@ -1303,9 +1298,20 @@ pw_status pw_dense_alloc(pw_dense_ws *ws, int nmax, int nbmax) {
   ws->gemm_ws_elems = std::max(ws->gemm_ws_elems, pw_zgemm_ws_elems(BTB, nbmax, nmax));
   ws->gemm_ws_elems = std::max(ws->gemm_ws_elems, pw_zgemm_ws_elems(BTB, BTB, nmax));
   if (ok && ws->gemm_ws_elems) ok = get((void **)&ws->gemm_ws, ws->gemm_ws_elems * 16);
-  if (!ok) { pw_dense_free(ws); return PW_ERR_OOM; }
+  if (!ok || pw_mem_alloc(ws->mem, &ws->arena, total) != cudaSuccess) {
+    for (auto &b : bufs) *b.first = nullptr;
+    pw_dense_free(ws);
+    return PW_ERR_OOM;
+  }
+  for (auto &b : bufs) *b.first = (char *)ws->arena + b.second;
+  if (!ws->oz.err) {
+    ok = pw_mem_alloc(ws->mem, (void **)&ws->oz.err, 16) == cudaSuccess &&
+         (ws->mem.pooled ? cudaMemsetAsync(ws->oz.err, 0, 16, ws->mem.st) : cudaMemset(ws->oz.err, 0, 16)) ==
+             cudaSuccess;
+    if (!ok) { pw_dense_free(ws); return PW_ERR_OOM; }
+  }
   for (cudaEvent_t &e : ws->ev)
-    if (!e && cudaEventCreate(&e) != cudaSuccess) { pw_dense_free(ws); return PW_ERR_CUDA; }
+    if (ws->timed && !e && cudaEventCreate(&e) != cudaSuccess) { pw_dense_free(ws); return PW_ERR_CUDA; }
   ws->nmax = nmax;
   ws->nbmax = nbmax;
   ws->bytes = total;
@@ -1317,18 +1323,14 @@ void pw_dense_free(pw_dense_ws *ws) {
   for (auto &g : ws->graphs) cudaGraphExecDestroy(g.exec);
   ws->graphs.clear();
   pw_oz_free(&ws->oz);
-  void *ptrs[] = {ws->G, ws->A, ws->T, ws->Linv, ws->Y, ws->dscale, ws->piv, ws->flag, ws->d, ws->e,
-                  ws->lam, ws->tau, ws->p, ws->w, ws->part, ws->Z, ws->W, ws->U, ws->Ds, ws->zs,
-                  ws->DK, ws->zK, ws->tauK, ws->zh, ws->lamK, ws->dD, ws->lnew, ws->perm, ws->colK,
-                  ws->orig, ws->dcol, ws->src, ws->nodes, ws->knode, ws->rhonode, ws->ctype, ws->qL, ws->qR,
-                  ws->kLR, ws->kneed, ws->gemm_ws,
-                  ws->Vb, ws->Gv, ws->Tb, ws->Wk, ws->Wk2, ws->panel, ws->ucorr,
-                  ws->hscal, ws->nrm_part, ws->Li, ws->hsl, ws->hsmax, ws->xcol, ws->acol, ws->hpart};
-  for (void *p : ptrs)
-    if (p) cudaFree(p);
+  const pw_mem m = ws->mem;
+  const bool timed = ws->timed;
+  pw_mem_free(m, ws->arena);
   for (cudaEvent_t e : ws->ev)
     if (e) cudaEventDestroy(e);
   *ws = pw_dense_ws();
+  ws->mem = ws->oz.mem = m;
+  ws->timed = timed;
 }
 
 void pw_dense_stage_ms(pw_dense_ws *ws, float out[5]) {
@@ -1657,15 +1659,18 @@ extern "C" pw_status pw_dense_graphs(int on) {
 pw_status pw_heev_lowest(pw_dense_ws *ws, int n, int nb, double2 *A, double *lam, double2 *Y,
                          cudaStream_t st) {
   if (n <= 0 || nb <= 0 || nb > n || n > ws->nmax || nb > ws->nbmax) return PW_ERR_ARG;
+  // the merge tree is built and uploaded outside any capture, and first: its
+  // copy is waited for, which would leave the stages behind it to be launched
+  // one by one against an idle GPU
+  if (ws->tree_n != n) build_tree(ws, n, st);
   // 1. Householder tridiagonalisation: panels of TPB columns (lower triangle)
   if (ws->ev[2]) cudaEventRecord(ws->ev[2], st);
   // with cooperative panels the stage is ~5 launches per 32 columns and is
   // ordered across streams by an event, so it runs uncaptured
   if ((g_coop.load() == 1 && coop_grid() > 0) || g_coop.load() == 3) PW_TRY(stage_tridiag(ws, n, A, st));
   else PW_TRY(run_stage(ws, 0, n, nb, A, nullptr, st, [&] { return stage_tridiag(ws, n, A, st); }));
-  // 2. divide and conquer (the merge tree is built and uploaded outside any capture)
+  // 2. divide and conquer
   if (ws->ev[3]) cudaEventRecord(ws->ev[3], st);
-  if (ws->tree_n != n) build_tree(ws, n, st);
   PW_TRY(run_stage(ws, 1, n, nb, lam, nullptr, st, [&] { return stage_dc(ws, n, nb, lam, st); }));
   // 3. back-transformation of the wanted columns
   if (ws->ev[4]) cudaEventRecord(ws->ev[4], st);
@@ -1805,6 +1810,8 @@ extern "C" pw_status pw_heev(int n, int nb, void *A, double *w, void *Y, void *s
   if (n < 1 || nb < 1 || nb > n || !A || !w || !Y) return PW_ERR_ARG;
   cudaStream_t st = (cudaStream_t)stream;
   pw_dense_ws ws;
+  ws.mem = ws.oz.mem = pw_mem{true, st};
+  ws.timed = false;
   PW_TRY(pw_dense_alloc(&ws, n, nb));
   pw_status r = pw_heev_lowest(&ws, n, nb, (double2 *)A, w, (double2 *)Y, st);
   if (r == PW_OK && cudaStreamSynchronize(st) != cudaSuccess) r = PW_ERR_CUDA;

@@ -65,6 +65,9 @@ struct pw_dense_ws {
   std::vector<int> level_off;             // offset of each level in `nodes` (in triples)
   int max_level_nodes = 0;
   size_t bytes = 0;
+  void *arena = nullptr;      // every buffer above, one allocation from mem
+  pw_mem mem;
+  bool timed = true;          // with the events below
   // sub-stage timing of the last Rayleigh-Ritz: events at the boundaries of
   // scale+Cholesky+L^-1 | L^-1 A L^-H | tridiagonal | divide & conquer |
   // back-transform + coefficients

@@ -209,7 +209,7 @@ __global__ void k_orth_err(const double2 *G, int n, double *out) {
 }
 
 pw_status alloc(void **p, size_t bytes, size_t *acc) {
-  if (cudaMalloc(p, bytes) != cudaSuccess) { cudaGetLastError(); *p = nullptr; return PW_ERR_OOM; }
+  if (pw_cuda_malloc(p, bytes) != cudaSuccess) { cudaGetLastError(); *p = nullptr; return PW_ERR_OOM; }
   *acc += bytes;
   return PW_OK;
 }

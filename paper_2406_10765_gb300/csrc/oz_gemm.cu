@@ -667,10 +667,12 @@ size_t pw_oz_ws_bytes(int m, int n, int k) {
 }
 
 void pw_oz_free(pw_oz_ws *w) {
-  if (w->buf) cudaFree(w->buf);
-  if (w->part) cudaFree(w->part);
-  if (w->err) cudaFree(w->err);
+  const pw_mem m = w->mem;
+  pw_mem_free(m, w->buf);
+  pw_mem_free(m, w->part);
+  pw_mem_free(m, w->err);
   *w = pw_oz_ws();
+  w->mem = m;
 }
 
 pw_status pw_oz_check(pw_oz_ws *w, cudaStream_t st) {
@@ -697,15 +699,15 @@ pw_status oz_block(pw_oz_ws *w, char opA, char opB, int mb, int nb, int k, doubl
   const size_t mxrows = (size_t)std::max(arows, brows);
   const size_t need = abytes + bbytes + ((size_t)arows + brows) * 4 + 256 + mxrows * 8 + 1024;
   if (need > w->bytes) {
-    if (w->buf) cudaFree(w->buf);
+    pw_mem_free(w->mem, w->buf);
     w->buf = nullptr;
     w->bytes = 0;
     ++w->gen;
-    if (cudaMalloc(&w->buf, need) != cudaSuccess) { cudaGetLastError(); return PW_ERR_OOM; }
+    if (pw_mem_alloc(w->mem, &w->buf, need) != cudaSuccess) return PW_ERR_OOM;
     w->bytes = need;
   }
   if (!w->err) {
-    if (cudaMalloc((void **)&w->err, 16) != cudaSuccess) { cudaGetLastError(); return PW_ERR_OOM; }
+    if (pw_mem_alloc(w->mem, (void **)&w->err, 16) != cudaSuccess) return PW_ERR_OOM;
     PW_CUDA(cudaMemsetAsync(w->err, 0, 16, st));
     ++w->gen;
   }
@@ -733,11 +735,11 @@ pw_status oz_block(pw_oz_ws *w, char opA, char opB, int mb, int nb, int k, doubl
     parts = std::min({(2 * 152 + act - 1) / act, std::max(1, nch / 2), g_max_parts});
     const size_t pbytes = (size_t)parts * mb * nb * 16;
     if (parts > 1 && pbytes > w->part_bytes) {
-      if (w->part) cudaFree(w->part);
+      pw_mem_free(w->mem, w->part);
       w->part = nullptr;
       w->part_bytes = 0;
       ++w->gen;
-      if (cudaMalloc((void **)&w->part, pbytes) != cudaSuccess) { cudaGetLastError(); parts = 1; }
+      if (pw_mem_alloc(w->mem, (void **)&w->part, pbytes) != cudaSuccess) parts = 1;
       else w->part_bytes = pbytes;
     }
   }
@@ -771,15 +773,15 @@ pw_status pw_dgemm_oz(pw_oz_ws *w, int m, int n, int k, const double *A, int lda
   const size_t abytes = (size_t)S * arows * kpad * 2, bbytes = (size_t)S * brows * kpad * 2;
   const size_t need = abytes + bbytes + ((size_t)arows + brows) * 4 + 256 + (size_t)arows * 8 + 1024;
   if (need > w->bytes) {
-    if (w->buf) cudaFree(w->buf);
+    pw_mem_free(w->mem, w->buf);
     w->buf = nullptr;
     w->bytes = 0;
     ++w->gen;
-    if (cudaMalloc(&w->buf, need) != cudaSuccess) { cudaGetLastError(); return PW_ERR_OOM; }
+    if (pw_mem_alloc(w->mem, &w->buf, need) != cudaSuccess) return PW_ERR_OOM;
     w->bytes = need;
   }
   if (!w->err) {
-    if (cudaMalloc((void **)&w->err, 16) != cudaSuccess) { cudaGetLastError(); return PW_ERR_OOM; }
+    if (pw_mem_alloc(w->mem, (void **)&w->err, 16) != cudaSuccess) return PW_ERR_OOM;
     PW_CUDA(cudaMemsetAsync(w->err, 0, 16, st));
     ++w->gen;
   }
@@ -896,6 +898,7 @@ extern "C" pw_status pw_zgemm_f64tc(char opA, char opB, int m, int n, int k, con
   if (ldc < m || lda < (opA == 'N' ? m : k) || ldb < (opB == 'N' ? k : n)) return PW_ERR_ARG;
   cudaStream_t st = (cudaStream_t)stream;
   pw_oz_ws w;
+  w.mem = pw_mem{true, st};
   pw_status r = pw_zgemm_oz(&w, opA, opB, m, n, k, make_double2(alpha[0], alpha[1]), (const double2 *)A, lda,
                             (const double2 *)B, ldb, make_double2(beta[0], beta[1]), (double2 *)C, ldc, st, 0);
   if (r == PW_OK) r = pw_oz_check(&w, st);

@@ -16,6 +16,7 @@ struct pw_oz_ws {
   size_t part_bytes = 0;
   int *err = nullptr;         // device error word (a bounded wait ran out)
   unsigned gen = 0;           // bumped whenever buf or part is reallocated
+  pw_mem mem;                 // where the buffers come from
 };
 
 // C = alpha op(A) op(B) + beta C, column-major complex128, op in {N, C};

@@ -222,5 +222,21 @@ pw_status pw_zgemm_batched(char opA, char opB, int m, int n, int k, double2 alph
 pw_status pw_zgemm_herm(int n, int k, const double2 *A, int lda, const double2 *B, int ldb,
                         double2 *C, int ldc, double2 *ws, size_t ws_elems, cudaStream_t st);
 
+// Device memory (pool.cu).  pooled: stream-ordered, from the library's pool,
+// for workspaces that live within one call on st; else cudaMalloc / cudaFree.
+// A failed allocation is tried again after the pool has given everything back;
+// *p is nullptr and the error cleared if it still fails.
+struct pw_mem {
+  bool pooled = false;
+  cudaStream_t st = nullptr;
+};
+cudaError_t pw_mem_alloc(const pw_mem &m, void **p, size_t bytes);
+void pw_mem_free(const pw_mem &m, void *p);
+void pw_pool_trim();
+template <typename T>
+cudaError_t pw_cuda_malloc(T **p, size_t bytes) {
+  return pw_mem_alloc(pw_mem{}, (void **)p, bytes);
+}
+
 // grow a device buffer
 pw_status pw_ensure(void **ptr, size_t *cur_bytes, size_t need_bytes);

@@ -108,7 +108,7 @@ extern "C" pw_status pw_cell_set_hxc(pw_cell *c, const double *v_hxc, void *stre
   const long npts = (long)c->N[0] * c->N[1] * c->N[2];
   if (!c->d_V0) {
     if (!v_hxc) return PW_OK;                 // already the cell's own V_loc
-    if (cudaMalloc(&c->d_V0, npts * sizeof(double)) != cudaSuccess) {
+    if (pw_cuda_malloc(&c->d_V0, npts * sizeof(double)) != cudaSuccess) {
       cudaGetLastError();
       c->d_V0 = nullptr;
       return PW_ERR_OOM;
@@ -137,9 +137,9 @@ extern "C" pw_status pw_scf(pw_cell *c, const pw_scf_opts *o, double *eig, doubl
     for (void *p : ptrs)
       if (p) cudaFree(p);
   };
-  if (cudaMalloc(&nin, npts * 8) != cudaSuccess || cudaMalloc(&nout, npts * 8) != cudaSuccess ||
-      cudaMalloc(&vhxc, npts * 8) != cudaSuccess || cudaMalloc(&bmax, nblk * 8) != cudaSuccess ||
-      cudaMalloc(&occ, nb * 8) != cudaSuccess || cudaMalloc(&X, (size_t)npw * nb * 16) != cudaSuccess) {
+  if (pw_cuda_malloc(&nin, npts * 8) != cudaSuccess || pw_cuda_malloc(&nout, npts * 8) != cudaSuccess ||
+      pw_cuda_malloc(&vhxc, npts * 8) != cudaSuccess || pw_cuda_malloc(&bmax, nblk * 8) != cudaSuccess ||
+      pw_cuda_malloc(&occ, nb * 8) != cudaSuccess || pw_cuda_malloc(&X, (size_t)npw * nb * 16) != cudaSuccess) {
     cudaGetLastError();
     cleanup();
     return PW_ERR_OOM;

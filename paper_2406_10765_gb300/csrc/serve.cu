@@ -332,6 +332,7 @@ extern "C" pw_status pw_serve(const pw_serve_opts *opts, const pw_request *req, 
   PW_CUDA(cudaGetDevice(&device));
   size_t budget = opts->hbm_budget;
   if (budget == 0) {
+    pw_pool_trim();
     size_t fr = 0, tot = 0;
     PW_CUDA(cudaMemGetInfo(&fr, &tot));
     budget = fr / 10 * 8;

@@ -57,7 +57,7 @@ pw_status pw_ensure(void **ptr, size_t *cur, size_t need) {
   *ptr = nullptr;
   *cur = 0;
   if (need == 0) return PW_OK;
-  if (cudaMalloc(ptr, need) != cudaSuccess) {
+  if (pw_cuda_malloc(ptr, need) != cudaSuccess) {
     cudaGetLastError();
     *ptr = nullptr;
     return PW_ERR_OOM;
@@ -107,7 +107,7 @@ static bool fft_plan(int n, pw_fft_axis &ax) {
 // kernels on a non-blocking stream are not ordered after it
 static pw_status upload(void **dst, const void *src, size_t bytes, size_t *acc, cudaStream_t st) {
   if (bytes == 0) { *dst = nullptr; return PW_OK; }
-  if (cudaMalloc(dst, bytes) != cudaSuccess) { cudaGetLastError(); *dst = nullptr; return PW_ERR_OOM; }
+  if (pw_cuda_malloc(dst, bytes) != cudaSuccess) { cudaGetLastError(); *dst = nullptr; return PW_ERR_OOM; }
   *acc += bytes;
   PW_CUDA(cudaMemcpyAsync(*dst, src, bytes, cudaMemcpyHostToDevice, st));
   return PW_OK;
@@ -342,8 +342,8 @@ extern "C" pw_status pw_setup_cell(const pw_cell_desc *d, void *stream, pw_cell 
   c->dkb_host.assign(d->dkb, d->dkb + 4 * (size_t)d->natom);
   {
     const long ng = (long)Nx * Ny * Nz;
-    if (cudaMalloc(&c->d_V, ng * sizeof(double)) != cudaSuccess ||
-        cudaMalloc(&c->d_Vf, ng * sizeof(float)) != cudaSuccess) {
+    if (pw_cuda_malloc(&c->d_V, ng * sizeof(double)) != cudaSuccess ||
+        pw_cuda_malloc(&c->d_Vf, ng * sizeof(float)) != cudaSuccess) {
       cudaGetLastError(); pw_destroy_cell(c); return PW_ERR_OOM;
     }
     acc += ng * (sizeof(double) + sizeof(float));
@@ -391,7 +391,7 @@ extern "C" pw_status pw_setup_cell(const pw_cell_desc *d, void *stream, pw_cell 
     std::vector<double> D(d->dkb, d->dkb + 4 * (size_t)d->natom);
     UP(c->d_D, D);
     size_t nbeta = (size_t)c->npw * c->nproj;
-    if (cudaMalloc(&c->d_beta, nbeta * sizeof(double2)) != cudaSuccess) {
+    if (pw_cuda_malloc(&c->d_beta, nbeta * sizeof(double2)) != cudaSuccess) {
       cudaGetLastError(); pw_destroy_cell(c); return PW_ERR_OOM;
     }
     acc += nbeta * sizeof(double2);
@@ -467,7 +467,7 @@ extern "C" pw_status pw_cell_set_projectors(pw_cell *c, int onthefly, void *stre
     c->proj_onthefly = 1;
     return PW_OK;
   }
-  if (cudaMalloc(&c->d_beta, (size_t)c->npw * c->nproj * sizeof(double2)) != cudaSuccess) {
+  if (pw_cuda_malloc(&c->d_beta, (size_t)c->npw * c->nproj * sizeof(double2)) != cudaSuccess) {
     cudaGetLastError();
     c->d_beta = nullptr;
     return PW_ERR_OOM;

@@ -1008,9 +1008,8 @@ pw_status pw_tc_operand_alloc(pw_tc_operand *op, int rows, int kreal, cudaStream
     return PW_OK;
   }
   pw_tc_operand_free(op);
-  if (cudaMalloc(&op->data, bytes) != cudaSuccess ||
-      cudaMalloc(&op->inv_scale, (size_t)rows_pad * sizeof(float)) != cudaSuccess) {
-    cudaGetLastError();
+  if (pw_mem_alloc(op->mem, (void **)&op->data, bytes) != cudaSuccess ||
+      pw_mem_alloc(op->mem, (void **)&op->inv_scale, (size_t)rows_pad * sizeof(float)) != cudaSuccess) {
     pw_tc_operand_free(op);
     return PW_ERR_OOM;
   }
@@ -1026,9 +1025,11 @@ pw_status pw_tc_operand_alloc(pw_tc_operand *op, int rows, int kreal, cudaStream
 }
 
 void pw_tc_operand_free(pw_tc_operand *op) {
-  if (op->data) cudaFree(op->data);
-  if (op->inv_scale) cudaFree(op->inv_scale);
+  const pw_mem m = op->mem;
+  pw_mem_free(m, op->data);
+  pw_mem_free(m, op->inv_scale);
   *op = pw_tc_operand();
+  op->mem = m;
 }
 
 extern "C" pw_status pw_zgemm_tc(char opA, int m, int n, int k, const void *A, int lda, const void *B,
@@ -1038,12 +1039,14 @@ extern "C" pw_status pw_zgemm_tc(char opA, int m, int n, int k, const void *A, i
     return PW_ERR_ARG;
   if (opA == 'C' ? (lda < k || ldb < k) : (lda < m || ldb < k)) return PW_ERR_ARG;
   cudaStream_t st = (cudaStream_t)stream;
+  const pw_mem mem{true, st};
   pw_tc_operand a, b;
+  a.mem = b.mem = mem;
   int *err = nullptr;
   float *rmax = nullptr;
   pw_status r = PW_OK;
   const double2 *Ad = (const double2 *)A, *Bd = (const double2 *)B;
-  if (cudaMalloc(&err, sizeof(int)) != cudaSuccess) { cudaGetLastError(); return PW_ERR_OOM; }
+  if (pw_mem_alloc(mem, (void **)&err, sizeof(int)) != cudaSuccess) return PW_ERR_OOM;
   cudaMemsetAsync(err, 0, sizeof(int), st);
   if (opA == 'C') {
     if ((r = pw_tc_operand_alloc(&a, 2 * m, 2 * k, st)) == PW_OK &&
@@ -1052,7 +1055,7 @@ extern "C" pw_status pw_zgemm_tc(char opA, int m, int n, int k, const void *A, i
         (r = pw_tc_split_rows(Bd, ldb, k, n, 0, nullptr, &b, st)) == PW_OK)
       r = pw_tc_gemm(&a, 2 * m, &b, n, (double2 *)C, ldc, 0, beta != 0.0, 0, err, st);
   } else {
-    if (cudaMalloc(&rmax, (size_t)m * sizeof(float)) != cudaSuccess) { cudaGetLastError(); r = PW_ERR_OOM; }
+    if (pw_mem_alloc(mem, (void **)&rmax, (size_t)m * sizeof(float)) != cudaSuccess) r = PW_ERR_OOM;
     if (r == PW_OK && (r = pw_tc_operand_alloc(&a, m, 2 * k, st)) == PW_OK &&
         (r = pw_tc_operand_alloc(&b, 2 * n, 2 * k, st)) == PW_OK &&
         (r = pw_tc_split_trans(Ad, lda, m, k, rmax, &a, st)) == PW_OK &&
@@ -1064,8 +1067,8 @@ extern "C" pw_status pw_zgemm_tc(char opA, int m, int n, int k, const void *A, i
       cudaStreamSynchronize(st) != cudaSuccess)
     r = PW_ERR_CUDA;
   if (r == PW_OK && herr) r = PW_ERR_TIMEOUT;
-  cudaFree(err);
-  if (rmax) cudaFree(rmax);
+  pw_mem_free(mem, err);
+  pw_mem_free(mem, rmax);
   pw_tc_operand_free(&a);
   pw_tc_operand_free(&b);
   return r;

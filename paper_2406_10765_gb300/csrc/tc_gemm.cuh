@@ -12,6 +12,7 @@ struct pw_tc_operand {
   int rows_total = 0, kpad = 0;
   size_t cap_bytes = 0;
   int scale_cap = 0;
+  pw_mem mem;                 // where the buffers come from
 };
 
 int pw_tc_kpad(int kreal);

@@ -117,7 +117,7 @@ extern "C" pw_status pw_cell_autotune_fft(pw_cell *c, int nb, int precision, voi
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   pw_status s = PW_OK;
   const size_t bytes = (size_t)npw * nb * sizeof(double2);
-  if (cudaMalloc((void **)&psi, bytes) != cudaSuccess || cudaMalloc((void **)&hpsi, bytes) != cudaSuccess) {
+  if (pw_cuda_malloc((void **)&psi, bytes) != cudaSuccess || pw_cuda_malloc((void **)&hpsi, bytes) != cudaSuccess) {
     cudaGetLastError();
     s = PW_ERR_OOM;
   }
