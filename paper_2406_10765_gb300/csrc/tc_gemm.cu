@@ -495,11 +495,22 @@ __device__ __forceinline__ float d2f_pow2(double x, int sh) {
   return __uint_as_float(sign | ((unsigned)e << 23) | m);
 }
 
-// hi = fp16(x), lo = fp16(x - hi); x - hi is exact in FP32
-__device__ __forceinline__ void split2f(float x, __half &hi, __half &lo) {
-  hi = __float2half_rn(x);
-  lo = __float2half_rn(x - __half2float(hi));
+// Slices of (a, b): hi = fp16(x), lo = fp16(x - hi), x - hi exact in FP32, as
+// packed pairs (a low)
+__device__ __forceinline__ void split2f(float a, float b, uint32_t &hi, uint32_t &lo) {
+  const __half2 h = __floats2half2_rn(a, b);
+  const float2 f = __half22float2(h);
+  const __half2 l = __floats2half2_rn(a - f.x, b - f.y);
+  hi = *reinterpret_cast<const uint32_t *>(&h);
+  lo = *reinterpret_cast<const uint32_t *>(&l);
 }
+template <int V>
+__device__ __forceinline__ void store_pairs(__half *o, const uint32_t *w) {
+  if (V == 2) *(uint2 *)o = make_uint2(w[0], w[V - 1]);
+  else *(uint32_t *)o = w[0];
+}
+// pair (re, im) -> (-im, re)
+__device__ __forceinline__ uint32_t times_i(uint32_t h) { return __byte_perm(h, 0, 0x1032) ^ 0x8000u; }
 
 __device__ __forceinline__ unsigned long long warp_maxu(unsigned long long v) {
   for (int o = 16; o > 0; o >>= 1) {
@@ -534,15 +545,25 @@ __device__ __forceinline__ int pow2_shift(double mx, float *inv) {
 //   conj=0:  row c       = (re, im) interleaved over g
 //   conj=1:  row 2c      = (re, im),   row 2c + 1 = (-im, re)
 // out: slices [2][rows_total][kpad] (hi then lo), inv scale per row.
-__global__ void __launch_bounds__(256) k_split_rows(const double2 *__restrict__ X, int ld, int npw,
-                                                    int ncols, int conj, int kpad, int rows_total,
-                                                    __half *__restrict__ out,
-                                                    float *__restrict__ inv_scale,
-                                                    const double *__restrict__ colscale) {
+// Bound: memory, 40 bytes per element (48 with conj): the column is read for its
+// maximum and again for the slices, the columns in flight being more than L2
+// holds.  (Held in the registers of a cluster per column instead, read once:
+// 1.2 to 1.9 times slower, the clusters' barriers and occupancy cost more than
+// the pass.)  V = 2 entries per thread and 8-byte stores; with 2-byte stores the
+// stores bounded it.  One entry per thread for columns short enough that the
+// time is one thread's.  43,819 x 1,458, both operands of a Gram product: 1.25 ->
+// 0.97 ms; 104,415 x 383: 1.16 -> 0.47 ms.
+template <int V>
+__global__ void __launch_bounds__(512) k_split_rows(const double2 *__restrict__ X, int ld, int npw,
+                                                        int ncols, int conj, int kpad, int rows_total,
+                                                        __half *__restrict__ out,
+                                                        float *__restrict__ inv_scale,
+                                                        const double *__restrict__ colscale) {
   const int c = blockIdx.x;
   const double2 *x = X + (long)c * ld;
   const double cs = colscale ? colscale[c] : 1.0;
   unsigned long long mb = 0;
+#pragma unroll 4
   for (int g = threadIdx.x; g < npw; g += blockDim.x) {
     const double2 v = x[g];
     const unsigned long long a = abs_bits(v.x), b = abs_bits(v.y);
@@ -556,21 +577,25 @@ __global__ void __launch_bounds__(256) k_split_rows(const double2 *__restrict__ 
   const int r0 = conj ? 2 * c : c;
   if (threadIdx.x == 0) { inv_scale[r0] = inv; if (conj) inv_scale[r0 + 1] = inv; }
   __half *o0 = out + (long)r0 * kpad;
-  for (int g = threadIdx.x; g < kpad / 2; g += blockDim.x) {
-    float re = 0.0f, im = 0.0f;
-    if (g < npw) {
-      double2 v = x[g];
-      if (colscale) { v.x *= cs; v.y *= cs; }
-      re = d2f_pow2(v.x, sh);
-      im = d2f_pow2(v.y, sh);
+#pragma unroll 2
+  for (int g = V * threadIdx.x; g < kpad / 2; g += V * blockDim.x) {   // kpad / 2 is a multiple of 32
+    double2 v[V];
+    uint32_t h[V], l[V];
+#pragma unroll
+    for (int q = 0; q < V; ++q) v[q] = g + q < npw ? x[g + q] : make_double2(0.0, 0.0);
+    if (colscale) {
+#pragma unroll
+      for (int q = 0; q < V; ++q) { v[q].x *= cs; v[q].y *= cs; }
     }
-    __half h, l;
-    split2f(re, h, l); o0[2 * g] = h; o0[slice + 2 * g] = l;
-    split2f(im, h, l); o0[2 * g + 1] = h; o0[slice + 2 * g + 1] = l;
+#pragma unroll
+    for (int q = 0; q < V; ++q) split2f(d2f_pow2(v[q].x, sh), d2f_pow2(v[q].y, sh), h[q], l[q]);
+    store_pairs<V>(o0 + 2 * g, h);
+    store_pairs<V>(o0 + slice + 2 * g, l);
     if (conj) {
-      __half *o1 = o0 + kpad;
-      split2f(-im, h, l); o1[2 * g] = h; o1[slice + 2 * g] = l;
-      split2f(re, h, l); o1[2 * g + 1] = h; o1[slice + 2 * g + 1] = l;
+#pragma unroll
+      for (int q = 0; q < V; ++q) { h[q] = times_i(h[q]); l[q] = times_i(l[q]); }
+      store_pairs<V>(o0 + kpad + 2 * g, h);
+      store_pairs<V>(o0 + kpad + slice + 2 * g, l);
     }
   }
 }
@@ -623,9 +648,10 @@ __global__ void __launch_bounds__(256) k_split_trans(const double2 *__restrict__
       const int t = t0 + tt;
       if (2 * t >= kpad) continue;
       const double2 v = tileS[tt][gg];
-      __half h, l;
-      split2f(d2f_pow2(v.x, sh), h, l); o[2 * t] = h; o[slice + 2 * t] = l;
-      split2f(d2f_pow2(v.y, sh), h, l); o[2 * t + 1] = h; o[slice + 2 * t + 1] = l;
+      uint32_t h, l;
+      split2f(d2f_pow2(v.x, sh), d2f_pow2(v.y, sh), h, l);
+      *(uint32_t *)(o + 2 * t) = h;
+      *(uint32_t *)(o + slice + 2 * t) = l;
     }
   }
 }
@@ -662,11 +688,13 @@ __global__ void __launch_bounds__(256) k_split_coef(const double2 *__restrict__ 
       re = d2f_pow2(v.x, sh);
       im = d2f_pow2(v.y, sh);
     }
-    __half h, l;
-    split2f(re, h, l); o0[2 * t] = h; o0[slice + 2 * t] = l;
-    split2f(-im, h, l); o0[2 * t + 1] = h; o0[slice + 2 * t + 1] = l;
-    split2f(im, h, l); o1[2 * t] = h; o1[slice + 2 * t] = l;
-    split2f(re, h, l); o1[2 * t + 1] = h; o1[slice + 2 * t + 1] = l;
+    uint32_t h, l;
+    split2f(re, -im, h, l);
+    *(uint32_t *)(o0 + 2 * t) = h;
+    *(uint32_t *)(o0 + slice + 2 * t) = l;
+    split2f(im, re, h, l);
+    *(uint32_t *)(o1 + 2 * t) = h;
+    *(uint32_t *)(o1 + slice + 2 * t) = l;
   }
 }
 
@@ -742,8 +770,9 @@ pw_status pw_tc_split_rows(const double2 *X, int ld, int npw, int ncols, int con
                            pw_tc_operand *op, cudaStream_t st) {
   if (op->rows_total < (conj ? 2 : 1) * ncols || op->kpad < 2 * npw) return PW_ERR_ARG;
   pw_count_launch();
-  k_split_rows<<<ncols, 256, 0, st>>>(X, ld, npw, ncols, conj, op->kpad, op->rows_total, op->data,
-                                      op->inv_scale, colscale);
+  const bool wide = npw > 4096;
+  (wide ? k_split_rows<2> : k_split_rows<1>)<<<ncols, wide ? 512 : 256, 0, st>>>(
+      X, ld, npw, ncols, conj, op->kpad, op->rows_total, op->data, op->inv_scale, colscale);
   return pw_check_launch("split_rows");
 }
 
@@ -1013,10 +1042,8 @@ pw_status pw_tc_operand_alloc(pw_tc_operand *op, int rows, int kreal, cudaStream
     pw_tc_operand_free(op);
     return PW_ERR_OOM;
   }
-  // padded rows and K must read as zeros: cleared on the caller's stream so
-  // the clearing is ordered before the kernels that fill the operand
-  PW_CUDA(cudaMemsetAsync(op->data, 0, bytes, st));
-  PW_CUDA(cudaMemsetAsync(op->inv_scale, 0, (size_t)rows_pad * sizeof(float), st));
+  // not cleared: the split kernels write every K of a row, its padding too, and
+  // rows past the operand's own only feed outputs that are not stored
   op->cap_bytes = bytes;
   op->scale_cap = rows_pad;
   op->rows_total = rows_pad;

@@ -16,7 +16,7 @@ struct pw_tc_operand {
 };
 
 int pw_tc_kpad(int kreal);
-// (re)allocates when larger; new storage is cleared on `st`
+// (re)allocates when larger
 pw_status pw_tc_operand_alloc(pw_tc_operand *op, int rows, int kreal, cudaStream_t st);
 void pw_tc_operand_free(pw_tc_operand *op);
 
