@@ -664,6 +664,7 @@ __device__ int block_excl_scan(int v, int *s_scan, int *total) {
 // of the two sorted halves places each value by its rank in the other half
 // (ties: left first); the deflating rotations are recorded in order, and the
 // block then applies them; the compactions are block-wide prefix sums.
+template <bool FIXED>
 __global__ void __launch_bounds__(256) k_dc_deflate(const int *nodes, int n, const double *e,
                                                     DcArrays a) {
   __shared__ double sh[32];
@@ -739,6 +740,10 @@ __global__ void __launch_bounds__(256) k_dc_deflate(const int *nodes, int n, con
   auto pair_rotates = [&](int q) {   // survivors q - 1 and q
     const int j = lo + surv[q - 1], p = lo + surv[q];
     const double zj = a.zs[j], zp = a.zs[p];
+    if (FIXED) {               // with the rotation's own rounding
+      const double r = hypot(zp, zj), c = zp / r, s = -zj / r;
+      return fabs(c * s * (a.Ds[p] - a.Ds[j])) <= tol;
+    }
     return fabs(zj * zp * (a.Ds[p] - a.Ds[j])) <= tol * fma(zj, zj, zp * zp);
   };
   const int sch = (ns + blockDim.x - 1) / blockDim.x;
@@ -923,7 +928,87 @@ __global__ void __launch_bounds__(256) k_dc_roots(const int *nodes, DcArrays a) 
   }
 }
 
+// The same in the fixed order (pw_dense_ws::fixed): until the bracket closes
+__global__ void __launch_bounds__(256) k_dc_roots_fixed(const int *nodes, DcArrays a) {
+  const int node = blockIdx.y;
+  const int lo = nodes[3 * node];
+  const int k = a.knode[node];
+  const int t = blockIdx.x * 8 + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (t >= k) return;
+  const double rho = a.rhonode[node];
+  const double *D = a.DK + lo, *z = a.zK + lo;
+  int o;
+  double blo, bhi;
+  if (t < k - 1) {
+    const double half = 0.5 * (D[t + 1] - D[t]);
+    double s = 0.0;
+    for (int i = lane; i < k; i += 32) s += z[i] * z[i] / ((D[i] - D[t]) - half);
+    s = warp_sum(s);
+    if (1.0 + rho * s >= 0.0) { o = t; blo = 0.0; bhi = half; }
+    else { o = t + 1; blo = -half; bhi = 0.0; }
+  } else {
+    double s = 0.0;
+    for (int i = lane; i < k; i += 32) s += z[i] * z[i];
+    s = warp_sum(s);
+    o = t; blo = 0.0; bhi = rho * s;
+  }
+  const double Do = D[o];
+  const double da = D[t] - Do;                          // left pole
+  const double db = (t < k - 1) ? D[t + 1] - Do : 0.0;  // right pole (if any)
+  double tau = 0.5 * (blo + bhi);
+  for (int it = 0; it < 100; ++it) {
+    double psi = 0.0, dpsi = 0.0, phi = 0.0, dphi = 0.0;
+    for (int i = lane; i < k; i += 32) {
+      // one reciprocal per term (FP64 divisions are the costly part here)
+      const double r = __drcp_rn((D[i] - Do) - tau);
+      const double term = z[i] * z[i] * r;
+      if (i <= t) { psi += term; dpsi = fma(term, r, dpsi); }
+      else { phi += term; dphi = fma(term, r, dphi); }
+    }
+    psi = rho * warp_sum(psi);
+    dpsi = rho * warp_sum(dpsi);
+    phi = rho * warp_sum(phi);
+    dphi = rho * warp_sum(dphi);
+    const double f = 1.0 + psi + phi;
+    if (f < 0.0) blo = fmax(blo, tau); else bhi = fmin(bhi, tau);
+    if (f == 0.0 || bhi - blo <= 4.0 * kEps * fmax(fabs(blo), fabs(bhi))) break;
+    const double q = dpsi * (da - tau) * (da - tau);
+    const double pp = psi - dpsi * (da - tau);
+    double x;
+    if (t < k - 1) {
+      const double s = dphi * (db - tau) * (db - tau);
+      const double r = phi - dphi * (db - tau);
+      const double Cc = 1.0 + pp + r;
+      const double A2 = Cc, B2 = -(Cc * (da + db) + q + s), C2 = Cc * da * db + q * db + s * da;
+      x = 0.5 * (blo + bhi);
+      if (A2 == 0.0) {
+        if (B2 != 0.0) x = -C2 / B2;
+      } else {
+        const double disc = fmax(B2 * B2 - 4.0 * A2 * C2, 0.0);
+        const double sq = sqrt(disc);
+        const double r1 = (B2 >= 0.0) ? (-B2 - sq) / (2.0 * A2) : (-B2 + sq) / (2.0 * A2);
+        const double r2 = (r1 != 0.0) ? C2 / (A2 * r1) : r1;
+        if (r1 > da && r1 < db) x = r1;
+        else if (r2 > da && r2 < db) x = r2;
+      }
+    } else {
+      const double Cc = 1.0 + pp + phi;
+      x = (Cc > 0.0) ? da + q / Cc : 0.5 * (blo + bhi);
+    }
+    if (!(x > blo && x < bhi)) x = 0.5 * (blo + bhi);
+    if (fabs(x - tau) <= 2.0 * kEps * fabs(x)) { tau = x; break; }
+    tau = x;
+  }
+  if (lane == 0) {
+    a.orig[lo + t] = o;
+    a.tauK[lo + t] = tau;
+    a.lamK[lo + t] = Do + tau;
+  }
+}
+
 // Lowner: rho zh_i^2 = prod_j (lam_j - D_i) / prod_{j != i} (D_j - D_i)
+template <bool FIXED>
 __global__ void __launch_bounds__(256) k_dc_zhat(const int *nodes, DcArrays a) {
   const int node = blockIdx.y;
   const int lo = nodes[3 * node];
@@ -936,7 +1021,7 @@ __global__ void __launch_bounds__(256) k_dc_zhat(const int *nodes, DcArrays a) {
   double prod = 1.0;
   for (int j = lane; j < k; j += 32) {
     const double num = (D[a.orig[lo + j]] - Di) + a.tauK[lo + j];
-    prod *= (j == i) ? num : div_newton(num, D[j] - Di);
+    prod *= (j == i) ? num : FIXED ? num / (D[j] - Di) : div_newton(num, D[j] - Di);
   }
   prod = warp_prod(prod);
   if (lane == 0) {
@@ -946,6 +1031,7 @@ __global__ void __launch_bounds__(256) k_dc_zhat(const int *nodes, DcArrays a) {
 }
 
 // eigenvectors of the secular problem: u_t[i] = zh_i / (D_i - lam_t), normalised
+template <bool FIXED>
 __global__ void __launch_bounds__(256) k_dc_vectors(const int *nodes, int n, DcArrays a) {
   const int node = blockIdx.y;
   const int lo = nodes[3 * node];
@@ -957,6 +1043,15 @@ __global__ void __launch_bounds__(256) k_dc_vectors(const int *nodes, int n, DcA
   const double Do = D[a.orig[lo + t]], tau = a.tauK[lo + t];
   double s = 0.0;
   double *Ucol = a.U + (long)(lo + t) * n + lo;
+  if (FIXED) {
+    for (int i = lane; i < k; i += 32) {
+      const double u = a.zh[lo + i] / ((D[i] - Do) - tau);
+      s += u * u;
+    }
+    const double inv = 1.0 / sqrt(warp_sum(s));
+    for (int i = lane; i < k; i += 32) Ucol[i] = inv * a.zh[lo + i] / ((D[i] - Do) - tau);
+    return;
+  }
   for (int i = lane; i < k; i += 32) {
     const double u = div_newton(a.zh[lo + i], (D[i] - Do) - tau);
     Ucol[i] = u;
@@ -1193,6 +1288,52 @@ __global__ void __launch_bounds__(32 * BT_WARPS) k_build_T(const double2 *G, con
   }
 }
 
+// The same in the fixed order: dot products, the lanes splitting the sum, the row
+// in shared memory, the next column of G fetched while the current one is reduced
+__global__ void __launch_bounds__(32 * BT_WARPS) k_build_T_fixed(const double2 *G, const double2 *tau, int j0, int b,
+                                                           double2 *T) {
+  __shared__ double2 trow[BT_WARPS][BTB];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int r = blockIdx.x * BT_WARPS + w;
+  if (r >= b) return;
+  double2 *tr = trow[w];
+  constexpr int KMAX = BTB / 32;
+  double2 gnext[KMAX];
+  auto fetch = [&](int col) {
+#pragma unroll
+    for (int k = 0; k < KMAX; ++k) {
+      const int m = r + lane + 32 * k;
+      gnext[k] = (col < b && m < col) ? G[m + (long)col * b] : make_double2(0.0, 0.0);
+    }
+  };
+  if (lane == 0) tr[r] = tau[j0 + r];
+  fetch(r + 1);
+  __syncwarp();
+  for (int c = r + 1; c < b; ++c) {
+    double2 g[KMAX];
+#pragma unroll
+    for (int k = 0; k < KMAX; ++k) g[k] = gnext[k];
+    fetch(c + 1);
+    double2 s = make_double2(0.0, 0.0);
+#pragma unroll
+    for (int k = 0; k < KMAX; ++k) {
+      const int m = r + lane + 32 * k;
+      if (m < c) cmac(s, tr[m], g[k]);
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      s.x += __shfl_xor_sync(0xffffffffu, s.x, off);
+      s.y += __shfl_xor_sync(0xffffffffu, s.y, off);
+    }
+    if (lane == 0) {
+      const double2 t = cmul(tau[j0 + c], s);
+      tr[c] = make_double2(-t.x, -t.y);
+    }
+    __syncwarp();
+  }
+  for (int c = lane; c < b; c += 32) T[r + (long)c * b] = c >= r ? tr[c] : make_double2(0.0, 0.0);
+}
+
 void build_tree(pw_dense_ws *ws, int n, cudaStream_t st) {
   ws->levels.clear();
   std::function<void(int, int, int)> rec = [&](int lo, int hi, int depth) {
@@ -1234,6 +1375,7 @@ pw_status pw_dense_gemm(pw_dense_ws *ws, char opA, char opB, int m, int n, int k
                         const double2 *A, int lda, const double2 *B, int ldb, double2 beta, double2 *C,
                         int ldc, cudaStream_t st, int herm) {
   if (m <= 0 || n <= 0) return PW_OK;
+  ws->oz.fixed = ws->fixed;
   if (pw_use_oz(m, n, k)) {
     if (ws->oz.bytes == 0) {
       // reserve the largest product of an order-nmax solve at once (the
@@ -1247,7 +1389,7 @@ pw_status pw_dense_gemm(pw_dense_ws *ws, char opA, char opB, int m, int n, int k
     return pw_zgemm_oz(&ws->oz, opA, opB, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, st, herm);
   }
   return pw_zgemm_ex(opA, opB, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, ws->gemm_ws, ws->gemm_ws_elems,
-                     st, herm);
+                     st, herm, ws->fixed);
 }
 
 // ======================================================================
@@ -1288,7 +1430,7 @@ pw_status pw_dense_alloc(pw_dense_ws *ws, int nmax, int nbmax) {
        get((void **)&ws->ucorr, 2 * TPB * HH_CHUNKS * 16) && get((void **)&ws->hscal, 16) && get((void **)&ws->Li, CB * CB * 16) &&
        get((void **)&ws->nrm_part, (size_t)(nmax / 32 + 2) * 8) &&
        get((void **)&ws->hsmax, (size_t)(nmax / TPB + 2) * 8) && get((void **)&ws->xcol, (size_t)nmax * 16) &&
-       get((void **)&ws->acol, (size_t)nmax * 16) && get((void **)&ws->hpart, 2 * pw_house_parts(nmax) * 8);
+       get((void **)&ws->acol, (size_t)nmax * 16) && get((void **)&ws->hpart, 2 * pw_house_parts(nmax) * 8) && get((void **)&ws->ticket, 64);
   // a slice tile is only read where the panel's slicing wrote it
   if (pw_hs_bytes(nmax)) ok = ok && get(&ws->hsl, pw_hs_bytes(nmax));
   ok = ok && get((void **)&ws->Vb, (size_t)nmax * BTB * 16) && get((void **)&ws->Gv, BTB * BTB * 16) &&
@@ -1440,7 +1582,8 @@ pw_status stage_tridiag(pw_dense_ws *ws, int n, double2 *A, cudaStream_t st) {
                   n - 1 >= PW_HS_MIN_ORDER;
   const int hgrid = hs && mode == 3 ? pw_hs_panel_grid() : 0;
   // the last columns (all of a small matrix) in one cluster
-  const int ncl = pw_house_cluster_max();
+  const int ncl = ws->fixed ? 0 : pw_house_cluster_max();
+  if (ws->fixed) PW_CUDA(cudaMemsetAsync(ws->ticket, 0, sizeof(unsigned), st));
   if (n <= ncl) return pw_house_cluster(ws, A, n, 0, st);
   // 1. Householder tridiagonalisation: panels of TPB columns (lower triangle)
   if (hs) PW_CUDA(cudaMemsetAsync(ws->hsmax, 0, (size_t)(n / TPB + 2) * 8, st));
@@ -1463,7 +1606,7 @@ pw_status stage_tridiag(pw_dense_ws *ws, int n, double2 *A, cudaStream_t st) {
                                n, one, A + t + (long)t * n, n, st, 2));
         continue;
       }
-      PW_TRY(pw_house_panel(ws, A, n, j0, b, ptc, st));
+      PW_TRY(ws->fixed ? pw_house_panel_fixed(ws, A, n, j0, b, ptc, st) : pw_house_panel(ws, A, n, j0, b, ptc, st));
       const int t = j0 + b, m2 = n - t;
       if (m2 > 0)
         PW_TRY(pw_dense_gemm(ws, 'N', 'C', m2, m2, 2 * b, mone, ws->panel + t, n, ws->panel + (long)b * n + t,
@@ -1493,14 +1636,14 @@ pw_status stage_dc(pw_dense_ws *ws, int n, int nb, double *lam, cudaStream_t st)
     int maxsize = 0;
     for (int q = 0; q < nn; ++q) maxsize = std::max(maxsize, ws->levels[l][3 * q + 2] - ws->levels[l][3 * q]);
     pw_count_launch();
-    k_dc_deflate<<<nn, 256, 0, st>>>(nodes, n, ws->e, a);
+    (ws->fixed ? k_dc_deflate<true> : k_dc_deflate<false>)<<<nn, 256, 0, st>>>(nodes, n, ws->e, a);
     const dim3 gw((maxsize + 7) / 8, nn);
     pw_count_launch();
-    k_dc_roots<<<gw, 256, 0, st>>>(nodes, a);
+    (ws->fixed ? k_dc_roots_fixed : k_dc_roots)<<<gw, 256, 0, st>>>(nodes, a);
     pw_count_launch();
-    k_dc_zhat<<<gw, 256, 0, st>>>(nodes, a);
+    (ws->fixed ? k_dc_zhat<true> : k_dc_zhat<false>)<<<gw, 256, 0, st>>>(nodes, a);
     pw_count_launch();
-    k_dc_vectors<<<gw, 256, 0, st>>>(nodes, n, a);
+    (ws->fixed ? k_dc_vectors<true> : k_dc_vectors<false>)<<<gw, 256, 0, st>>>(nodes, n, a);
     // the root merge keeps only the nb lowest eigenpairs
     const int keep = l == 0 ? nb : n;
     pw_count_launch();
@@ -1529,6 +1672,7 @@ pw_status stage_dc(pw_dense_ws *ws, int n, int nb, double *lam, cudaStream_t st)
           pw_count_launch();
           k_dc_gather_u<<<(unsigned)(((long)kmax * tmax + 255) / 256), 256, 0, st>>>(lo, node, half, n, a, kmax,
                                                                                      tmax, Ug);
+          ws->oz.fixed = ws->fixed;
           PW_TRY(pw_dgemm_oz(&ws->oz, rows, tmax, kmax, Zg, rows, Ug, kmax, Wt, rows, st));
           pw_count_launch();
           k_dc_scatter_w<<<(unsigned)(((long)rows * tmax + 255) / 256), 256, 0, st>>>(lo, mid, hi, node, half, n,
@@ -1568,7 +1712,7 @@ pw_status stage_backtransform(pw_dense_ws *ws, int n, int nb, const double2 *A, 
       k_copy_panel<<<(unsigned)(((long)mb * b + 255) / 256), 256, 0, st>>>(A, n, j0, b, ws->Vb, mb);
       PW_TRY(pw_dense_gemm(ws, 'C', 'N', b, b, mb, one, ws->Vb, mb, ws->Vb, mb, zero, ws->Gv, b, st));
       pw_count_launch();
-      k_build_T<<<(b + BT_WARPS - 1) / BT_WARPS, 32 * BT_WARPS, 0, st>>>(ws->Gv, ws->tau, j0, b, ws->Tb);
+      (ws->fixed ? k_build_T_fixed : k_build_T)<<<(b + BT_WARPS - 1) / BT_WARPS, 32 * BT_WARPS, 0, st>>>(ws->Gv, ws->tau, j0, b, ws->Tb);
       double2 *Yb = Y + (j0 + 1);
       PW_TRY(pw_dense_gemm(ws, 'C', 'N', b, nb, mb, one, ws->Vb, mb, Yb, n, zero, ws->Wk, b, st));
       PW_TRY(pw_dense_gemm(ws, 'N', 'N', b, nb, b, one, ws->Tb, b, ws->Wk, b, zero, ws->Wk2, b, st));
@@ -1582,9 +1726,10 @@ pw_status stage_backtransform(pw_dense_ws *ws, int n, int nb, const double2 *A, 
 std::atomic<int> g_graphs{1};
 
 // what a captured stage depends on besides its key: the product buffers'
-// generation, the product mode and the panel mode
+// generation, the product mode, the panel mode and the order of operations
 unsigned stage_gen(const pw_dense_ws *ws) {
-  return (2 * ws->oz.gen + (unsigned)pw_dense_products_mode()) * 4 + (unsigned)g_coop.load();
+  return ((2 * ws->oz.gen + (unsigned)pw_dense_products_mode()) * 4 + (unsigned)g_coop.load()) * 2 +
+         (unsigned)ws->fixed;
 }
 
 // A stage through the workspace's graph cache: the first call of a key runs
@@ -1736,10 +1881,10 @@ pw_status trinv(pw_dense_ws *ws, const double2 *L, double2 *X, int n, cudaStream
       } else {
         // T_p = L21 X11 (w x w, ld w)
         PW_TRY(pw_zgemm_batched('N', 'N', w, w, w, one, L + w, n, s2, X, n, s2, zero, T, w, (long)w * w,
-                                full, st, 4));
+                                full, st, 4, ws->fixed));
         // X21 = -X22 T_p
         PW_TRY(pw_zgemm_batched('N', 'N', w, w, w, mone, X + w * dstep, n, s2, T, w, (long)w * w, zero,
-                                X + w, n, s2, full, st, 5));
+                                X + w, n, s2, full, st, 5, ws->fixed));
       }
     }
     const int off = full * 2 * w;
@@ -1759,6 +1904,7 @@ pw_status pw_rayleigh_ritz(pw_dense_ws *ws, int n, int nb, const double2 *G, int
                            const double2 *A, int lda, double *theta, double2 *C, int ldc,
                            int *chol_ok, cudaStream_t st, double piv_tol) {
   if (n > ws->nmax || nb > ws->nbmax || nb > n) return PW_ERR_ARG;
+  ws->fixed = false;
   *chol_ok = 1;
   cudaEventRecord(ws->ev[0], st);
   PW_CUDA(cudaMemsetAsync(ws->flag, 0, 16, st));
@@ -1837,6 +1983,7 @@ __global__ void k_make_M(const double2 *Linv, int n, const double *d, double2 *M
 pw_status pw_rr_factor(pw_dense_ws *ws, int n, const double2 *G, int ldg, double2 *M, int ldm,
                        int *chol_ok, cudaStream_t st, double piv_tol) {
   if (n > ws->nmax) return PW_ERR_ARG;
+  ws->fixed = true;
   *chol_ok = 1;
   cudaEventRecord(ws->ev[0], st);
   PW_CUDA(cudaMemsetAsync(ws->flag, 0, 16, st));
@@ -1864,6 +2011,7 @@ pw_status pw_rr_factor(pw_dense_ws *ws, int n, const double2 *G, int ldg, double
 pw_status pw_rr_finish_tall(pw_dense_ws *ws, int n, int nb, const double2 *At, int lda, const double2 *M,
                             int ldm, double *theta, double2 *Cp, int ldc, cudaStream_t st) {
   if (n > ws->nmax || nb > ws->nbmax || nb > n) return PW_ERR_ARG;
+  ws->fixed = true;
   pw_count_launch();
   const dim3 g2((n + 31) / 32, (n + 31) / 32), b2(32, 32);
   k_copy_herm<<<g2, b2, 0, st>>>(At, lda, n, ws->A);

@@ -68,6 +68,14 @@ struct pw_dense_ws {
   void *arena = nullptr;      // every buffer above, one allocation from mem
   pw_mem mem;
   bool timed = true;          // with the events below
+  // One fixed order of operations in the dense solves of the mixed iteration
+  // (set by pw_rr_factor and pw_rr_finish_tall): the iteration multiplies a
+  // difference of rounding (1e-15) through its FP16 splits and FP32 FFTs to
+  // 1e-7 in the Ritz values of an unconverged block, so another order is
+  // another trajectory.  Its kernels keep the sums they had; the FP64 solves
+  // take the faster ones.
+  bool fixed = false;
+  unsigned *ticket = nullptr;   // last-block-done counter of house_chain.cu
   // sub-stage timing of the last Rayleigh-Ritz: events at the boundaries of
   // scale+Cholesky+L^-1 | L^-1 A L^-H | tridiagonal | divide & conquer |
   // back-transform + coefficients
@@ -106,9 +114,15 @@ pw_status pw_hs_panel(pw_dense_ws *ws, double2 *A, int n, int j0, int b, int gri
 // All columns of the panel at j0 (width b) as chained kernels (house_cols.cu),
 // with the Hermitian products on the tensor cores (tc: the panel's slices are
 // written) or on the FP64 pipe; leaves the panel, tau, d, e as above.
+// pw_house_panel_fixed: the same in the fixed order (three kernels per column,
+// house_chain.cu).
 // pw_house_parts: blocks its arrays of partials hold.
 size_t pw_house_parts(int nmax);
 pw_status pw_house_panel(pw_dense_ws *ws, double2 *A, int n, int j0, int b, bool tc, cudaStream_t st);
+pw_status pw_house_panel_fixed(pw_dense_ws *ws, double2 *A, int n, int j0, int b, bool tc, cudaStream_t st);
+// its column product on the slices, v = x s (scale in ws->hscal)
+pw_status pw_hs_hemv_fixed(pw_dense_ws *ws, const double2 *A, int n, int c, int i, int b, int j0, int *nslots,
+                           cudaStream_t st);
 // The reduction from column j0 on (order n - j0 <= pw_house_cluster_max(), the
 // trailing matrix up to date) in one thread-block cluster, leaving reflectors,
 // tau, d (to the last entry) and e as the chained kernels do.

@@ -275,6 +275,14 @@ __host__ __device__ __forceinline__ int hs_pieces(int ntp, int grid, int slots) 
   return ks;
 }
 
+// the same for the products of the reflector (fixed order, cooperative panel):
+// enough units for the grid
+__host__ __device__ __forceinline__ int hs_pieces_v(int ntp, int grid, int slots) {
+  int ks = 1;
+  while (ks < S && ntp * (ntp + 1) * ks < grid && 2 * ntp * ks * 2 <= slots) ks *= 2;
+  return ks;
+}
+
 // an error word another role of the CTA (or another CTA) may have set
 __device__ __forceinline__ bool hs_failed(const int *err) { return *(const volatile int *)err != 0; }
 
@@ -366,14 +374,17 @@ __device__ __forceinline__ double2 refl_v(const double2 *xcol, int x, int m, dou
   return x == 0 ? make_double2(1.0, 0.0) : cmul(__ldcg(&xcol[x]), s);
 }
 
-// The vector of a product: entry(row), zero before row c + 1
-struct VecRefl {                       // the reflector v = x s below its unit head
+// The vector of a product: entry(row), zero before row c + 1; scaled per block of
+// 128 entries by the block's largest one, or by 1/2 throughout
+struct VecRefl {                       // the reflector v = x s below its unit head (|v| <= 1)
+  static constexpr bool block_scale = false;
   const double2 *xk;
   int o, mm;
   double2 scal;
   __device__ double2 entry(int r) const { return refl_v(xk, r - o, mm, scal); }
 };
 struct VecCol {                        // the column x
+  static constexpr bool block_scale = true;
   const HhCol &h;
   double k2;
   __device__ double2 entry(int r) const {
@@ -383,8 +394,8 @@ struct VecCol {                        // the column x
 
 // Warps 2..5 (et = threadIdx.x - 64, the K entry of the B operands):
 // digits of the vector over unit u's tile columns (dir 0, A v) and rows (dir
-// 1, A^H v) into buffer ug & 1, rows 14..29 of the window layout, each block of
-// 128 entries scaled by its own largest one; ev: the blocks' exponents
+// 1, A^H v) into buffer ug & 1, rows 14..29 of the window layout; ev: the blocks'
+// exponents, |entry| 2^ev <= 1
 template <int NS, class Vec>
 __device__ void hs_build(const HsCol &w, const HsSmem<NS> &m, int u, int ug, const Vec &vec, int (&ev)[2]) {
   const int et = threadIdx.x - 64;
@@ -396,17 +407,22 @@ __device__ void hs_build(const HsCol &w, const HsSmem<NS> &m, int u, int ug, con
   v[1] = diag ? v[0] : vec.entry(I * HT + et);
   // the exponents, from the high words of the largest entries of both blocks
   uint32_t *mx = m.vmax + (ug & 1) * 8;
+  if (Vec::block_scale) {
 #pragma unroll
-  for (int dir = 0; dir < 2; ++dir) {
-    const uint32_t hb = (uint32_t)(max(abs_bits(v[dir].x), abs_bits(v[dir].y)) >> 32);
-    const uint32_t wm = __reduce_max_sync(0xffffffffu, hb);
-    if ((et & 31) == 0) mx[dir * 4 + (et >> 5)] = wm;
+    for (int dir = 0; dir < 2; ++dir) {
+      const uint32_t hb = (uint32_t)(max(abs_bits(v[dir].x), abs_bits(v[dir].y)) >> 32);
+      const uint32_t wm = __reduce_max_sync(0xffffffffu, hb);
+      if ((et & 31) == 0) mx[dir * 4 + (et >> 5)] = wm;
+    }
+    named_sync(3, 128);
   }
-  named_sync(3, 128);
 #pragma unroll
   for (int dir = 0; dir < 2; ++dir) {
-    const uint32_t hb = max(max(mx[dir * 4], mx[dir * 4 + 1]), max(mx[dir * 4 + 2], mx[dir * 4 + 3]));
-    ev[dir] = row_exp((unsigned long long)hb << 32);
+    ev[dir] = -1;
+    if (Vec::block_scale) {
+      const uint32_t hb = max(max(mx[dir * 4], mx[dir * 4 + 1]), max(mx[dir * 4 + 2], mx[dir * 4 + 3]));
+      ev[dir] = row_exp((unsigned long long)hb << 32);
+    }
     if (dir == 1 && diag) break;
     uint32_t d[S];
     digit_pairs(v[dir].x, v[dir].y, ev[dir], d);
@@ -614,6 +630,77 @@ __global__ void __launch_bounds__(NTHR, 1) k_hemv_tc(const __grid_constant__ HsA
   }
 }
 
+// One column of the fixed order: the reflector's product, its sides in warps 6, 7
+struct HsArgsV {
+  HsSide side;
+  const unsigned char *hsl;    // slices of the panel's trailing tiles
+  const unsigned long long *slot;   // max bits of the trailing matrix (its scale)
+  const double2 *hscal;        // reflector scale s (v = x s below the unit head)
+  double2 *part;               // tile partials [slot][nmax]
+  int nmax;
+  int J0, ks, units;           // first trailing tile, pieces per (tile, part), units
+  int *err;
+};
+
+__global__ void __launch_bounds__(NTHR_PANEL, 1) k_hemv_tc_fixed(const __grid_constant__ HsArgsV a) {
+  constexpr int NS = NST_HEMV;
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  const HsSmem<NS> m((unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023));
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  HsCol w;
+  w.n = a.side.n;
+  w.c = a.side.c;
+  hs_range(a.units, w.ub, w.nunit);
+  w.J0 = a.J0;
+  w.ks = a.ks;
+  w.hsl = a.hsl;
+  w.part = a.part;
+  w.nmax = a.nmax;
+  w.err = a.err;
+
+  hs_setup(m);
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = *m.tmem_slot;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      // the slices were written before the panel's first column, two or more
+      // launches back, so the producer needs no dependency wait
+      int k = 0;
+      uint32_t issued = 0, last_ph = 0;
+      hs_produce(w, m, 0, hs_subtiles(w), k, issued, last_ph);
+      hs_produce_drain(m, issued, last_ph, w.err);
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      int k = 0, ug = 0;
+      hs_mma(w, m, tmem, k, ug);
+      hs_mma_finish(m, w.err);
+    }
+  } else if (warp < 6) {
+    pdl_wait();
+    pdl_trigger();
+    const double2 scal = *a.hscal;
+    const int eA = row_exp(*a.slot);
+    int ug = 0;
+    const int o = w.c + 1;
+    const VecRefl vec{a.side.A + o + (long)w.c * w.n, o, w.n - o, scal};
+    hs_epi(w, m, tmem, vec, eA, ug);
+  } else {
+    pdl_wait();
+    pdl_trigger();
+    hs_side(a.side, *a.hscal, m.red, 1, 64, threadIdx.x - 192);
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0) {
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS));
+  }
+}
+
 // --------------------------------------------- one cooperative panel ----
 // All the columns of a panel (32 from j0) in one cooperative launch, one CTA
 // per SM, the phases of each column separated by grid-wide barriers:
@@ -677,7 +764,7 @@ __global__ void __launch_bounds__(NTHR_PANEL, 1) k_panel_tc(const __grid_constan
     w.c = c;
     w.J0 = o / HT;
     const int ntp = nT - w.J0;
-    w.ks = hs_pieces(ntp, nblk, a.slots);
+    w.ks = hs_pieces_v(ntp, nblk, a.slots);
     hs_range(ntp * (ntp + 1) * w.ks, w.ub, w.nunit);
     w.hsl = a.hsl;
     w.part = a.part;
@@ -868,6 +955,8 @@ pw_status allow_smem() {
   std::lock_guard<std::mutex> lk(mu);
   if (!done[dev]) {
     PW_CUDA(cudaFuncSetAttribute(k_hemv_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, HsL<NST_HEMV>::SMEM));
+    PW_CUDA(
+        cudaFuncSetAttribute(k_hemv_tc_fixed, cudaFuncAttributeMaxDynamicSharedMemorySize, HsL<NST_HEMV>::SMEM));
     PW_CUDA(cudaFuncSetAttribute(k_panel_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, HsL<NST_PANEL>::SMEM));
     done[dev] = true;
   }
@@ -923,6 +1012,47 @@ pw_status pw_hs_hemv(pw_dense_ws *ws, const HhCol &h, int j0, int *nslots, int *
   cfg.numAttrs = h.i > 0 ? 1 : 0;      // the panel's first column: after the slicing
   pw_count_launch();
   PW_CUDA(cudaLaunchKernelEx(&cfg, k_hemv_tc, a));
+  return PW_OK;
+}
+
+pw_status pw_hs_hemv_fixed(pw_dense_ws *ws, const double2 *A, int n, int c, int i, int b, int j0, int *nslots,
+                           cudaStream_t st) {
+  PW_TRY(allow_smem());
+  HsArgsV a;
+  a.side.A = A;
+  a.side.n = n;
+  a.side.c = c;
+  a.side.i = i;
+  a.side.b = b;
+  a.side.P = ws->panel;
+  a.side.ucorr = ws->ucorr;
+  a.hsl = (const unsigned char *)ws->hsl;
+  a.slot = ws->hsmax + j0 / 32;
+  a.hscal = ws->hscal;
+  a.part = ws->part;
+  a.nmax = ws->nmax;
+  a.J0 = (c + 1) / HT;
+  const int ntp = (n + HT - 1) / HT - a.J0;
+  // pieces per (tile, part): enough units for every SM, within the partial
+  // slots ws->part holds ((nmax + 31) / 32)
+  const int sms = sm_count();
+  a.ks = hs_pieces_v(ntp, sms, (ws->nmax + 31) / 32);
+  a.units = ntp * (ntp + 1) * a.ks;
+  a.err = ws->oz.err;
+  *nslots = 2 * ntp * a.ks;
+  const int grid = std::min(a.units, sms);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(NTHR_PANEL);
+  cfg.dynamicSmemBytes = HsL<NST_HEMV>::SMEM;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  pw_count_launch();
+  PW_CUDA(cudaLaunchKernelEx(&cfg, k_hemv_tc_fixed, a));
   return PW_OK;
 }
 

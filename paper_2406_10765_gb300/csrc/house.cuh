@@ -1,5 +1,5 @@
 // Device helpers of the blocked Householder reduction shared by its kernels
-// (house_cols.cu: the chained column kernels; hemv_tc.cu: their tensor-core
+// (house_cols.cu and house_chain.cu: the chained column kernels; hemv_tc.cu: their tensor-core
 // Hermitian product and the cooperative tensor-core panel; dense.cu: the
 // cooperative FP64 panel; house_cluster.cu: the last columns): warp and block
 // sums, complex multiply-adds written as four FMAs, the reflector scalars, a

@@ -77,9 +77,11 @@ constexpr int STAGE = OFF_B + S * B_T;   // 108 KB
 constexpr int STAGE_LOAD = S * (A_T + B_T);   // of which TMA writes 96 KB
 constexpr int NSTAGE = 2;
 constexpr int NG = S;                 // accumulator groups g = 2..S+1
-constexpr int CHUNK_KB = 3;           // K blocks per exact accumulation chunk (96 real K)
+// K blocks per exact accumulation chunk: 96 real K, or in a fixed order of
+// operations (pw_oz_ws::fixed) 64, after which every group is rounded to the
+// sum's binary point
+constexpr int CHUNK_KB = 3, CHUNK_KB_FIXED = 2;
 constexpr int STEPS_KB = BK / 16;     // MMA steps (16 real K) per K block
-constexpr int CHUNK = CHUNK_KB * STEPS_KB;
 constexpr int NH = 2;
 constexpr int SMEM_BYTES = NSTAGE * STAGE + 1024 + 512;
 static_assert(SMEM_BYTES <= 232448, "shared memory per CTA");
@@ -99,8 +101,11 @@ __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, u
 __device__ __forceinline__ uint64_t smem_desc_sw64(uint32_t addr) { return smem_desc(addr, 16, 512, 4); }
 
 // whether half h (0: groups 2..5, 1: groups 6..9) is emptied after MMA step t
-// of nsteps: every CHUNK steps, the halves CHUNK / 2 apart, and at the end
+// of nsteps: every chunk (CKB blocks), the halves half a chunk apart, and at the
+// end
+template <int CKB>
 __device__ __forceinline__ bool oz_flush(int h, int t, int nsteps) {
+  constexpr int CHUNK = CKB * STEPS_KB;
   return (t + 1 + (h == 0 ? CHUNK / 2 : 0)) % CHUNK == 0 || t == nsteps - 1;
 }
 
@@ -125,6 +130,7 @@ __device__ __forceinline__ uint32_t biased(uint32_t v) {
   return __float_as_uint(__uint_as_float(v) + 12582912.0f);
 }
 
+template <int CKB>
 __global__ void __launch_bounds__(NTHREADS, 1)
     k_oz_gemm(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
               int a_slice_rows, int b_slice_rows, int m, int n, int kblocks, int mtiles, int ntiles,
@@ -159,11 +165,11 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   if (herm == 5) kb_hi = min(kblocks, (2 * (gm0 + BM) + BK - 1) / BK);
   // K split: part z of gridDim.y takes an equal share, in whole chunks
   const int ntot = max(0, kb_hi - kb_lo);
-  const int nch = (ntot + CHUNK_KB - 1) / CHUNK_KB;
+  const int nch = (ntot + CKB - 1) / CKB;
   const int per = (nch + (int)gridDim.y - 1) / (int)gridDim.y;
   const int c0 = min(nch, (int)blockIdx.y * per), c1 = min(nch, c0 + per);
-  const int kb_beg = kb_lo + c0 * CHUNK_KB;
-  const int nkb = max(0, min(kb_hi, kb_lo + c1 * CHUNK_KB) - kb_beg);
+  const int kb_beg = kb_lo + c0 * CKB;
+  const int nkb = max(0, min(kb_hi, kb_lo + c1 * CKB) - kb_beg);
   const int nsteps = nkb * STEPS_KB;
   // binary point of the fixed-point sum: |sum| <= K' (scaled entries < 1)
   int lg = 0;
@@ -232,14 +238,14 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           }
           oz_mmas<1>(tmem, da0 + off, db0 + off, first1);
-          first1 = oz_flush(1, t, nsteps);
+          first1 = oz_flush<CKB>(1, t, nsteps);
           if (first1) { mma_commit(&accf[1]); ++nfl1; }
           if (first0) {
             if (!mbar_wait(&acce[0], (nfl0 & 1) ^ 1)) { atomicOr(err, 8); ok = false; break; }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           }
           oz_mmas<0>(tmem, da0 + off, db0 + off, first0);
-          first0 = oz_flush(0, t, nsteps);
+          first0 = oz_flush<CKB>(0, t, nsteps);
           if (first0) { mma_commit(&accf[0]); ++nfl0; }
         }
         if (!ok) break;
@@ -255,9 +261,10 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     unsigned long long acc[32];
 #pragma unroll
     for (int i = 0; i < 32; ++i) acc[i] = 0;
-    // the two lowest groups, weights 2^-56 and 2^-63, are added in units of
+    // CARRY: the two lowest groups, weights 2^-56 and 2^-63, are added in units of
     // 2^-63, and what lies below the sum's binary point stays in rem until the
     // end: one rounding instead of two per chunk
+    constexpr bool CARRY = CKB == CHUNK_KB;
     uint32_t rem[32];
 #pragma unroll
     for (int i = 0; i < 32; ++i) rem[i] = 0;
@@ -269,19 +276,19 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     for (int t = 0; t < nsteps && ok; ++t) {
 #pragma unroll
       for (int hh = NH - 1; hh >= 0; --hh) {
-        if (!ok || !oz_flush(hh, t, nsteps)) continue;
+        if (!ok || !oz_flush<CKB>(hh, t, nsteps)) continue;
         if (!mbar_wait(&accf[hh], nfl[hh] & 1)) { atomicOr(err, 4); ok = false; continue; }
         ++nfl[hh];
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const int gend = hh == NH - 1 ? NG - 2 : (hh + 1) * HG;
+        const int gend = CARRY && hh == NH - 1 ? NG - 2 : (hh + 1) * HG;
 #pragma unroll 1
         for (int g = hh * HG; g < gend; ++g) {
           uint32_t v[32];
           tmem_ld32(tmem + lanes + (uint32_t)(g * BN + h * 32), v);
-          if (g == HG - 1) {
+          if (g == HG - 1 || (!CARRY && g == NG - 1)) {
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
-            if (lane == 0) mbar_arrive(&acce[0]);
+            if (lane == 0) mbar_arrive(&acce[hh]);
           }
           const int sh = Lfix - BETA * (g + 2);
           if (sh >= 32) {
@@ -292,7 +299,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 #pragma unroll
             for (int i = 0; i < 32; ++i) acc[i] += (unsigned long long)biased(v[i]) * f;
           } else {
-            // rounded to nearest (the third lowest group of very long sums)
+            // rounded to nearest (with CARRY the third lowest group of very long sums)
             const int half = 1 << (-sh - 1);
 #pragma unroll
             for (int i = 0; i < 32; ++i)
@@ -300,7 +307,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           }
           if (sh >= 0) bias += (unsigned long long)kBias << sh;
         }
-        if (hh == NH - 1) {
+        if (CARRY && hh == NH - 1) {
           const uint32_t tv = tmem + lanes + (uint32_t)((NG - 2) * BN + h * 32), tu = tv + BN;
 #pragma unroll
           for (int c = 0; c < 32; c += 16) {
@@ -322,8 +329,10 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         }
       }
     }
+    if (CARRY) {
 #pragma unroll
-    for (int i = 0; i < 32; ++i) acc[i] += (rem[i] + (1u << (slow - 1))) >> slow;
+      for (int i = 0; i < 32; ++i) acc[i] += (rem[i] + (1u << (slow - 1))) >> slow;
+    }
 #pragma unroll
     for (int i = 0; i < 32; ++i) acc[i] -= bias;
     const int i = m0 + q * 32 + lane;              // complex output row
@@ -652,7 +661,8 @@ pw_status allow_smem() {
   if (dev < 0 || dev >= 64) return PW_ERR_ARG;
   std::lock_guard<std::mutex> g(mu);
   if (!done[dev]) {
-    PW_CUDA(cudaFuncSetAttribute(k_oz_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
+    PW_CUDA(cudaFuncSetAttribute(k_oz_gemm<CHUNK_KB>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
+    PW_CUDA(cudaFuncSetAttribute(k_oz_gemm<CHUNK_KB_FIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
     done[dev] = true;
   }
   return PW_OK;
@@ -728,11 +738,13 @@ pw_status oz_block(pw_oz_ws *w, char opA, char opB, int mb, int nb, int k, doubl
   // what its start and its share of the reduction cost; a tile alone on its SM
   // takes ~1.1 us a step (S^H S of the 8-atom cell, 72 x 72 x 1,647: 227 us in
   // one part, 28 us split).
-  const int nch = (kblocks + CHUNK_KB - 1) / CHUNK_KB;
-  const int act = herm == 1 ? (tiles + 1) / 2 : tiles;
+  const int ckb = w->fixed ? CHUNK_KB_FIXED : CHUNK_KB;
+  const int nch = (kblocks + ckb - 1) / ckb;
+  const int act = herm == 1 && !w->fixed ? (tiles + 1) / 2 : tiles;
   int parts = 1;
-  if (herm <= 1 && act < 152) {
-    parts = std::min({(2 * 152 + act - 1) / act, std::max(1, nch / 2), g_max_parts});
+  if (herm <= (w->fixed ? 0 : 1) && act < 152) {
+    // (a fixed order of operations keeps parts of eight chunks)
+    parts = std::min({(2 * 152 + act - 1) / act, std::max(1, nch / (w->fixed ? 8 : 2)), g_max_parts});
     const size_t pbytes = (size_t)parts * mb * nb * 16;
     if (parts > 1 && pbytes > w->part_bytes) {
       pw_mem_free(w->mem, w->part);
@@ -744,7 +756,8 @@ pw_status oz_block(pw_oz_ws *w, char opA, char opB, int mb, int nb, int k, doubl
     }
   }
   pw_count_launch();
-  k_oz_gemm<<<dim3(tiles, parts), NTHREADS, SMEM_BYTES, st>>>(ma, mbm, arows, brows, mb, nb, kblocks, mtiles,
+  const auto kern = w->fixed ? k_oz_gemm<CHUNK_KB_FIXED> : k_oz_gemm<CHUNK_KB>;
+  kern<<<dim3(tiles, parts), NTHREADS, SMEM_BYTES, st>>>(ma, mbm, arows, brows, mb, nb, kblocks, mtiles,
                                                                ntiles, ea, eb, alpha, beta, C, ldc, herm, ioff,
                                                                joff, parts > 1 ? w->part : nullptr, w->err, 0);
   PW_TRY(pw_check_launch("oz gemm"));
@@ -806,7 +819,8 @@ pw_status pw_dgemm_oz(pw_oz_ws *w, int m, int n, int k, const double *A, int lda
   PW_TRY(allow_smem());
   const int mtiles = arows / BM, ntiles = brows / BN;
   pw_count_launch();
-  k_oz_gemm<<<dim3(mtiles * ntiles, 1), NTHREADS, SMEM_BYTES, st>>>(
+  const auto kern = w->fixed ? k_oz_gemm<CHUNK_KB_FIXED> : k_oz_gemm<CHUNK_KB>;
+  kern<<<dim3(mtiles * ntiles, 1), NTHREADS, SMEM_BYTES, st>>>(
       ma, mbm, arows, brows, m, n, kblocks, mtiles, ntiles, ea, eb, make_double2(1.0, 0.0), make_double2(0.0, 0.0),
       (double2 *)C, ldc, 0, 0, 0, nullptr, w->err, 1);
   return pw_check_launch("oz gemm (real)");

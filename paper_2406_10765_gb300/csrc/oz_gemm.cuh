@@ -17,6 +17,7 @@ struct pw_oz_ws {
   int *err = nullptr;         // device error word (a bounded wait ran out)
   unsigned gen = 0;           // bumped whenever buf or part is reallocated
   pw_mem mem;                 // where the buffers come from
+  bool fixed = false;         // fixed order of operations (pw_dense_ws::fixed)
 };
 
 // C = alpha op(A) op(B) + beta C, column-major complex128, op in {N, C};

@@ -146,19 +146,15 @@ __device__ __forceinline__ int row_exp(unsigned long long mb) {
   return 1022 - ex;                      // max in [2^(ex-1023), 2^(ex-1022)) -> [1/2, 1)
 }
 // The S digits of x0 2^e and x1 2^e (|x 2^e| <= 1) as FP16 pairs (x0 low): the
-// fixed-point value F = round(x 2^(e + 56)) with -64 <= d_p < 64 for p > 1 and
-// |d_1| <= 2^BETA, x 2^e = sum_p d_p 2^(-BETA p) to 2^-57.  Adding 64 to every
-// digit but the first at once (kDigitBias) makes them plain bit fields; a field
-// f under the exponent of 1024 is the half 1024 + f, and one packed subtraction
-// takes the offset off.  About 30 integer instructions per value against 120
-// for peeling the digits from the top and converting each.
-constexpr long long digit_bias() {
-  long long k = 0;
-  for (int p = 2; p <= S; ++p) k += 1ll << (BETA * (S - p) + BETA - 1);
-  return k;
-}
-// F + the bias of x 2^e
-__device__ __forceinline__ long long biased_digits(double x, int e) {
+// fixed-point value F = round(x 2^(e + 56)) is cut from the top, BETA bits at a
+// time, each digit rounded to nearest; |d_1| <= 2^BETA, |d_p| <= 2^(BETA-1)
+// after it, and x 2^e = sum_p d_p 2^(-BETA p) to 2^-57.  The digits up to p add
+// up to F rounded at digit p, R_p = (F + half) >> shift, so d_p = R_p - 2^BETA
+// R_(p-1) needs no remainder; d + 64 (d_1 + 128) under the exponent of 1024 is
+// the half 1024 + that, and one packed subtraction takes the offset off.  About
+// 60 integer instructions per value against 120 for peeling remainders and
+// converting each digit.
+__device__ __forceinline__ long long fixed_point56(double x, int e) {
   const long long b = __double_as_longlong(x);
   const int ex = (int)((b >> 52) & 0x7FF);
   // mantissa (53 bits) times 2^4, shifted right by r >= 0 to the unit 2^-56
@@ -166,20 +162,25 @@ __device__ __forceinline__ long long biased_digits(double x, int e) {
   const int r = max(0, 1023 - ex - e);
   long long F = 0;
   if (ex != 0 && r < 62) F = (mant + ((1ll << r) >> 1)) >> r;
-  return (b < 0 ? -F : F) + digit_bias();
+  return b < 0 ? -F : F;
 }
 __device__ __forceinline__ void digit_pairs(double x0, double x1, int e, uint32_t *out) {
   static_assert(BETA * S == 56, "unit of the fixed-point value");
-  const long long u0 = biased_digits(x0, e), u1 = biased_digits(x1, e);
+  const long long F0 = fixed_point56(x0, e), F1 = fixed_point56(x1, e);
+  uint32_t q0 = 0, q1 = 0;             // R_(p-1), low words
 #pragma unroll
   for (int p = 1; p <= S; ++p) {
     const int sh = BETA * (S - p);
+    const long long half = sh > 0 ? 1ll << (sh - 1) : 0;
+    const uint32_t r0 = (uint32_t)((F0 + half) >> sh), r1 = (uint32_t)((F1 + half) >> sh);
     // the first digit with an offset of 2^BETA, the others with 2^(BETA-1)
-    const uint32_t f0 = p == 1 ? (uint32_t)(u0 >> sh) + (1u << BETA) : (uint32_t)(u0 >> sh) & ((1u << BETA) - 1u);
-    const uint32_t f1 = p == 1 ? (uint32_t)(u1 >> sh) + (1u << BETA) : (uint32_t)(u1 >> sh) & ((1u << BETA) - 1u);
+    const uint32_t off = p == 1 ? 1u << BETA : 1u << (BETA - 1);
+    const uint32_t f0 = r0 - (q0 << BETA) + off, f1 = r1 - (q1 << BETA) + off;
+    q0 = r0;
+    q1 = r1;
     const uint32_t w = (f0 | (f1 << 16)) | 0x64006400u;
-    const uint32_t off = (0x6400u + (p == 1 ? 1u << BETA : 1u << (BETA - 1))) * 0x10001u;
-    const __half2 d = __hsub2(*reinterpret_cast<const __half2 *>(&w), *reinterpret_cast<const __half2 *>(&off));
+    const uint32_t o2 = (0x6400u + off) * 0x10001u;
+    const __half2 d = __hsub2(*reinterpret_cast<const __half2 *>(&w), *reinterpret_cast<const __half2 *>(&o2));
     out[p - 1] = *reinterpret_cast<const uint32_t *>(&d);
   }
 }

@@ -280,7 +280,7 @@ pw_status pw_zgemm(char opA, char opB, int m, int n, int k, double2 alpha, const
 
 pw_status pw_zgemm_ex(char opA, char opB, int m, int n, int k, double2 alpha, const double2 *A, int lda,
                       const double2 *B, int ldb, double2 beta, double2 *C, int ldc, double2 *ws,
-                      size_t ws_elems, cudaStream_t st, int herm) {
+                      size_t ws_elems, cudaStream_t st, int herm, bool fixed) {
   if (m <= 0 || n <= 0) return PW_OK;
   if (k <= 0) {
     // C = beta C
@@ -295,7 +295,7 @@ pw_status pw_zgemm_ex(char opA, char opB, int m, int n, int k, double2 alpha, co
   if ((size_t)splits * m * n > ws_elems || !ws) splits = 1;
   // few 64 x 64 tiles even when split: 8 x 8 tiles, with no more parts (each
   // part costs a pass over C) than give the SMs four CTAs each
-  const bool small = small_tiles(m, n, splits);
+  const bool small = !fixed && small_tiles(m, n, splits);
   const int tiles8 = ((m + T8 - 1) / T8) * ((n + T8 - 1) / T8);
   if (small) splits = std::min(splits, (4 * 152 + tiles8 - 1) / tiles8);
   int kchunk = (k + splits - 1) / splits;
@@ -327,10 +327,10 @@ pw_status pw_zgemm_ex(char opA, char opB, int m, int n, int k, double2 alpha, co
 
 pw_status pw_zgemm_batched(char opA, char opB, int m, int n, int k, double2 alpha, const double2 *A,
                            int lda, long sA, const double2 *B, int ldb, long sB, double2 beta,
-                           double2 *C, int ldc, long sC, int batch, cudaStream_t st, int mode) {
+                           double2 *C, int ldc, long sC, int batch, cudaStream_t st, int mode, bool fixed) {
   if (m <= 0 || n <= 0 || batch <= 0) return PW_OK;
   if (k <= 0 || (sA | sB | sC) == 0 || mode == 1) return PW_ERR_ARG;
-  const bool small = small_tiles(m, n, batch);
+  const bool small = !fixed && small_tiles(m, n, batch);
   const int T = small ? T8 : BM;
   dim3 grid((m + T - 1) / T, (n + T - 1) / T, batch);
 #define L(a, b) (small ? k_zgemm8<a, b> : k_zgemm<a, b>)<<<grid, 256, 0, st>>>(m, n, k, k, alpha, A, lda, B, ldb, beta, \
