@@ -6,9 +6,9 @@
 // r < R.  With n = l + L r and k = k2 + R k1:
 //   1. in-lane DFT of length R over r            -> Y[l][k2]
 //   2. twiddle Y[l][k2] *= w_N^(l k2)
-//   3. DFT of length L across the lanes for each k2 (radix-2 decimation in
-//      frequency with warp shuffles), which leaves X[k2 + R k1] in lane
-//      bitrev(k1).
+//   3. DFT of length L across the lanes for each k2 (decimation in frequency
+//      with warp shuffles: radix 2 in FP32, radix 4 in FP64), which leaves
+//      X[k2 + R k1] in lane bitrev(k1).
 // Each pass loads a line from shared memory in the strided order above and
 // stores the result at its natural position, so a whole 1-D transform is one
 // shared-memory read and one write, with no block barrier inside it.
@@ -118,17 +118,29 @@ template <typename C, int R, int N> struct LaneDFT {
   }
 };
 
-// per-lane twiddles of a line: w_N^(l k2) and the shuffle-stage factors
+// per-lane twiddles of a line: w_N^(l k2) and the shuffle-stage factors (FP32:
+// one per radix-2 stage; FP64: one per radix-4 stage, for the lane's output)
 template <typename C, int L, int R> struct LineTw {
   static constexpr int N = L * R, LG = log2c(L);
+  static constexpr bool fp64 = sizeof(C) == sizeof(double2);
+  static constexpr int NS = fp64 ? LG / 2 : LG;
   C lt[R > 1 ? R - 1 : 1];
-  C st[LG > 0 ? LG : 1];
+  C st[NS > 0 ? NS : 1];
   __device__ __forceinline__ void init(const C *tw, int l) {
 #pragma unroll
     for (int k2 = 1; k2 < R; ++k2) lt[k2 - 1] = tw[l * k2];
     int s = 0;
+    if constexpr (fp64) {
 #pragma unroll
-    for (int h = L / 2; h >= 1; h >>= 1, ++s) st[s] = tw[(l & (h - 1)) * (N / (2 * h))];
+      for (int h = L / 2; h >= 2; h >>= 2, ++s) {
+        // output j of the four: w_(2h)^(j n), n = l mod h / 2
+        const int j = ((l & h) ? 1 : 0) + ((l & (h / 2)) ? 2 : 0);
+        st[s] = tw[j * (l & (h / 2 - 1)) * (N / (2 * h))];
+      }
+    } else {
+#pragma unroll
+      for (int h = L / 2; h >= 1; h >>= 1, ++s) st[s] = tw[(l & (h - 1)) * (N / (2 * h))];
+    }
   }
   // natural index of register k2 of lane l after line_fft
   __device__ __forceinline__ int out_index(int k2, int l) const {
@@ -137,6 +149,29 @@ template <typename C, int L, int R> struct LineTw {
   }
 };
 
+// v <- p + sg v in every lane, sg = 1 or -1: a lane's side of the butterfly
+__device__ __forceinline__ double2 bfly(double2 v, double2 p, double sg) {
+  return make_double2(fma(sg, v.x, p.x), fma(sg, v.y, p.y));
+}
+// v times -i (forward) or i (inverse) where sel, by moves and a sign bit
+__device__ __forceinline__ double2 quarter(double2 v, bool sel, bool inv) {
+  const long long sx = __double_as_longlong(inv ? v.y : v.x) ^ (long long)0x8000000000000000ull;
+  const double neg = __longlong_as_double(sx);
+  double2 r;
+  r.x = sel ? (inv ? neg : v.y) : v.x;
+  r.y = sel ? (inv ? v.x : neg) : v.y;
+  return r;
+}
+
+// The DFT across the lanes is what a line costs in FP64, whose pipe issues a
+// warp's instruction in 64 clocks: a radix-2 stage written as a choice between
+// the two sides runs both, 8 FP64 instructions per value.  Here both sides are
+// one signed add (2 instructions), two stages share one twiddle multiplication
+// (radix 4: the inner one is by +-i, moves only), and the last stages need
+// none: 12 instructions per value for 16 lanes instead of 32.  With the in-lane
+// part 21 instead of 41 per value and line at N = 48.  Local part of H psi, 144
+// bands of the 64-atom cell (N = 48): 4.56 -> 2.40 ms; 486 bands of the 216-atom
+// cell (N = 72): 55.3 -> 32.9 ms.  The FP32 stages keep their order (and results).
 template <typename C, int L, int R>
 __device__ __forceinline__ void line_fft(C (&v)[R], const LineTw<C, L, R> &t, const C *tw, int l,
                                          bool inv) {
@@ -144,14 +179,35 @@ __device__ __forceinline__ void line_fft(C (&v)[R], const LineTw<C, L, R> &t, co
 #pragma unroll
   for (int k2 = 1; k2 < R; ++k2) v[k2] = cmul(v[k2], conj_if(t.lt[k2 - 1], inv));
   int s = 0;
+  if constexpr (LineTw<C, L, R>::fp64) {
 #pragma unroll
-  for (int h = L / 2; h >= 1; h >>= 1, ++s) {
-    const C w = conj_if(t.st[s], inv);
-    const bool upper = (l & h) != 0;
+    for (int h = L / 2; h >= 2; h >>= 2, ++s) {
+      const C w = conj_if(t.st[s], inv);
+      const bool up1 = (l & h) != 0, up2 = (l & (h / 2)) != 0;
+      const double s1 = up1 ? -1.0 : 1.0, s2 = up2 ? -1.0 : 1.0;
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const C p = shfl_xor2(v[r], h);
-      v[r] = upper ? cmul(csub(p, v[r]), w) : cadd(v[r], p);
+      for (int r = 0; r < R; ++r) {
+        C a = bfly(v[r], shfl_xor2(v[r], h), s1);
+        a = quarter(a, up1 && up2, inv);
+        a = bfly(a, shfl_xor2(a, h / 2), s2);
+        v[r] = h > 2 ? cmul(a, w) : a;
+      }
+    }
+    if (LineTw<C, L, R>::LG % 2 == 1) {
+      const double s1 = (l & 1) ? -1.0 : 1.0;
+#pragma unroll
+      for (int r = 0; r < R; ++r) v[r] = bfly(v[r], shfl_xor2(v[r], 1), s1);
+    }
+  } else {
+#pragma unroll
+    for (int h = L / 2; h >= 1; h >>= 1, ++s) {
+      const C w = conj_if(t.st[s], inv);
+      const bool upper = (l & h) != 0;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const C p = shfl_xor2(v[r], h);
+        v[r] = upper ? cmul(csub(p, v[r]), w) : cadd(v[r], p);
+      }
     }
   }
 }
