@@ -42,7 +42,7 @@
 // programmatic dependent launch): persistent, one CTA per SM, each CTA a
 // contiguous range of work units (tile, real or imaginary part, and for
 // short trailing orders a piece of its eight slices, so that every SM has
-// work).  Warp 0 = bulk-copy producer (six 32 KB stages), warp 1 = MMA
+// work).  Warp 0 = bulk-copy producer (five 32 KB stages), warp 1 = MMA
 // issuer (one thread), warps 2..5 = B-operand builders and epilogue, warps
 // 6..9 = the finished column and the panel's correction dots on the otherwise
 // idle FP64 pipe; B operands and accumulators are double-buffered, so a unit's
@@ -91,7 +91,14 @@ struct HsL {
   static constexpr int OFF_BAR = OFF_RED + 128;
   static constexpr int SMEM = OFF_BAR + (2 * NS + NBAR_FIXED) * 8 + 16 + 1024;
 };
-constexpr int NST_HEMV = 6;                  // one column per launch
+// One column per launch: five stages, not the six that fit, so that the row
+// kernels (11 KB and less) find room beside a CTA and both kinds start and load
+// while their predecessor runs.  That also takes the same split of L1 and shared
+// memory in every launch of the chain (the launches' carve-out): 198 KB alone
+// would get a split that leaves nothing.  Order-3,456 eigensolve 157.5 -> 145.0 ms
+// (the row kernel's part of a column 16.5 -> 11.7 us at order 3,400, 12 -> 7 us
+// at 1,500); the product itself keeps its speed with five stages.
+constexpr int NST_HEMV = 5;
 constexpr int NST_PANEL = 5;                 // cooperative panel (its column phases need static scratch)
 constexpr int SIDE_WARPS = 4;
 constexpr int NTHR = 192 + 32 * SIDE_WARPS;  // producer, MMA, 4 epilogue warps, side warps
@@ -1005,11 +1012,13 @@ pw_status pw_hs_hemv(pw_dense_ws *ws, const HhCol &h, int j0, int *nslots, int *
   cfg.blockDim = dim3(NTHR);
   cfg.dynamicSmemBytes = HsL<NST_HEMV>::SMEM;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+  attr[0].val.sharedMemCarveout = cudaSharedmemCarveoutMaxShared;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = h.i > 0 ? 1 : 0;      // the panel's first column: after the slicing
+  cfg.numAttrs = h.i > 0 ? 2 : 1;      // the panel's first column: after the slicing
   pw_count_launch();
   PW_CUDA(cudaLaunchKernelEx(&cfg, k_hemv_tc, a));
   return PW_OK;
@@ -1046,11 +1055,13 @@ pw_status pw_hs_hemv_fixed(pw_dense_ws *ws, const double2 *A, int n, int c, int 
   cfg.blockDim = dim3(NTHR_PANEL);
   cfg.dynamicSmemBytes = HsL<NST_HEMV>::SMEM;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+  attr[1].val.sharedMemCarveout = cudaSharedmemCarveoutMaxShared;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   pw_count_launch();
   PW_CUDA(cudaLaunchKernelEx(&cfg, k_hemv_tc_fixed, a));
   return PW_OK;

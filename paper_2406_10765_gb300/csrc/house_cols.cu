@@ -20,7 +20,8 @@
 // rest of the time was chains of FP64 instructions, which the row kernel
 // spreads: RB rows per CTA, the panel's columns over the other threads, the
 // scalars in a warp of their own meanwhile.
-// Measured: order-1,458 eigensolve 49.1 -> 40.6 ms, order 3,456 183 -> 161 ms;
+// Measured: order-1,458 eigensolve 49.1 -> 40.6 ms, order 3,456 183 -> 161 ms
+// (145 ms with the row kernel resident beside k_hemv_tc);
 // a column of trailing order 500 takes 15 us: launches 2, k2 3-4, product 5,
 // scalars 2.5, sums 1, the rows' tail 1.5.
 #include <algorithm>
@@ -293,6 +294,9 @@ int rows_block(int m) { return m <= 152 * 7 ? 8 : m <= 152 * 15 ? 16 : 32; }
 // while its predecessor finishes, waits (griddepcontrol.wait) before it reads
 // anything the predecessor wrote, and only then lets its own successor start.
 // So before its wait it may read what was written two or more launches back.
+// The row kernels ask for the whole of an SM's shared memory, as k_hemv_tc has
+// it: an SM that would have to change the split between L1 and shared memory
+// takes CTAs of the other kernel only once it is empty.
 template <class Arg, class... More>
 cudaError_t launch(void (*kern)(const Arg, More...), int grid, bool overlap, cudaStream_t st, const Arg &arg,
                    More... more) {
@@ -300,11 +304,13 @@ cudaError_t launch(void (*kern)(const Arg, More...), int grid, bool overlap, cud
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(256);
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+  attr[0].val.sharedMemCarveout = cudaSharedmemCarveoutMaxShared;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = overlap ? 1 : 0;
+  cfg.numAttrs = overlap ? 2 : 1;
   pw_count_launch();
   return cudaLaunchKernelEx(&cfg, kern, arg, more...);
 }
