@@ -579,6 +579,50 @@ __global__ void __launch_bounds__(CO_THREADS) k_panel_coop(double2 *A, int n, in
   }
 }
 
+// The trailing updates' product operands hold v (at most 1) and w (of the matrix's
+// size) in one row with one scale, so a matrix far from 1 is brought to it by a
+// power of two before its reduction, and the tridiagonal entries back after it;
+// within 2^+-6 it is left as it is.
+// exponent of the scaling from the largest part's bits (0: none)
+__device__ __forceinline__ int matrix_scale(const unsigned long long *slot) {
+  const int ex = (int)(*slot >> 52);
+  return ex == 0 || ex == 0x7FF || abs(ex - 1023) <= 6 ? 0 : ex - 1023;
+}
+// largest |Re|, |Im| of the lower triangle, as ordered bits (*slot cleared before)
+__global__ void __launch_bounds__(256) k_matrix_max(const double2 *__restrict__ A, int n, unsigned long long *slot) {
+  __shared__ unsigned long long sh[8];
+  const int c = blockIdx.x;
+  unsigned long long mb = 0;
+  for (int r = c + threadIdx.x; r < n; r += 256) {
+    const double2 v = A[r + (long)c * n];
+    mb = max(mb, max((unsigned long long)__double_as_longlong(fabs(v.x)),
+                     (unsigned long long)__double_as_longlong(fabs(v.y))));
+  }
+  for (int o = 16; o > 0; o >>= 1) mb = max(mb, __shfl_xor_sync(0xffffffffu, mb, o));
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = mb;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) mb = max(mb, sh[w]);
+    atomicMax(slot, mb);
+  }
+}
+__global__ void __launch_bounds__(256) k_matrix_scale(double2 *A, int n, const unsigned long long *slot) {
+  const int e = matrix_scale(slot), c = blockIdx.x;
+  if (e == 0) return;
+  for (int r = c + threadIdx.x; r < n; r += 256) {
+    double2 v = A[r + (long)c * n];
+    v.x = scalbn(v.x, -e);
+    v.y = scalbn(v.y, -e);
+    A[r + (long)c * n] = v;
+  }
+}
+__global__ void __launch_bounds__(256) k_tridiag_unscale(double *d, double *e, int n, const unsigned long long *slot) {
+  const int k = matrix_scale(slot), i = blockIdx.x * 256 + threadIdx.x;
+  if (k == 0 || i >= n) return;
+  d[i] = scalbn(d[i], k);
+  if (i + 1 < n) e[i] = scalbn(e[i], k);
+}
+
 __global__ void k_last_diag_plain(const double2 *A, int n, double *d) {
   d[n - 1] = A[(n - 1) + (long)(n - 1) * n].x;
 }
@@ -1427,7 +1471,7 @@ pw_status pw_dense_alloc(pw_dense_ws *ws, int nmax, int nbmax) {
        get((void **)&ws->qL, (size_t)nmax * 4) && get((void **)&ws->qR, (size_t)nmax * 4) &&
        get((void **)&ws->kLR, (size_t)nmax * 8 + 64) && get((void **)&ws->kneed, (size_t)nmax * 4 + 64);
   ok = ok && get((void **)&ws->panel, (size_t)nmax * 3 * TPB * 16) &&
-       get((void **)&ws->ucorr, 2 * TPB * HH_CHUNKS * 16) && get((void **)&ws->hscal, 16) && get((void **)&ws->Li, CB * CB * 16) &&
+       get((void **)&ws->ucorr, 2 * TPB * HH_CHUNKS * 16) && get((void **)&ws->hscal, 128) && get((void **)&ws->Li, CB * CB * 16) &&
        get((void **)&ws->nrm_part, (size_t)(nmax / 32 + 2) * 8) &&
        get((void **)&ws->hsmax, (size_t)(nmax / TPB + 2) * 8) && get((void **)&ws->xcol, (size_t)nmax * 16) &&
        get((void **)&ws->acol, (size_t)nmax * 16) && get((void **)&ws->hpart, 2 * pw_house_parts(nmax) * 8) && get((void **)&ws->ticket, 64);
@@ -1571,7 +1615,7 @@ pw_status tridiag_coop(pw_dense_ws *ws, int n, double2 *A, int grid, cudaStream_
   return pw_check_launch("tridiag (cooperative panels)");
 }
 
-pw_status stage_tridiag(pw_dense_ws *ws, int n, double2 *A, cudaStream_t st) {
+pw_status tridiag_run(pw_dense_ws *ws, int n, double2 *A, cudaStream_t st) {
   const int mode = g_coop.load();
   const int grid = mode == 1 ? coop_grid() : 0;
   if (grid > 0) return tridiag_coop(ws, n, A, grid, st);
@@ -1618,6 +1662,21 @@ pw_status stage_tridiag(pw_dense_ws *ws, int n, double2 *A, cudaStream_t st) {
   PW_TRY(pw_check_launch("tridiag"));
 
   return PW_OK;
+}
+
+pw_status stage_tridiag(pw_dense_ws *ws, int n, double2 *A, cudaStream_t st) {
+  // only where the updates may be digit products, and not in the fixed order
+  if (ws->fixed || pw_dense_products_mode() != 1 || n <= pw_house_cluster_max()) return tridiag_run(ws, n, A, st);
+  unsigned long long *slot = (unsigned long long *)((char *)ws->hscal + 64);
+  PW_CUDA(cudaMemsetAsync(slot, 0, 8, st));
+  pw_count_launch();
+  k_matrix_max<<<n, 256, 0, st>>>(A, n, slot);
+  pw_count_launch();
+  k_matrix_scale<<<n, 256, 0, st>>>(A, n, slot);
+  PW_TRY(tridiag_run(ws, n, A, st));
+  pw_count_launch();
+  k_tridiag_unscale<<<(n + 255) / 256, 256, 0, st>>>(ws->d, ws->e, n, slot);
+  return pw_check_launch("tridiag scale");
 }
 
 pw_status stage_dc(pw_dense_ws *ws, int n, int nb, double *lam, cudaStream_t st) {
