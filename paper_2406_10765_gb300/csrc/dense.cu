@@ -1640,7 +1640,7 @@ pw_status tridiag_run(pw_dense_ws *ws, int n, double2 *A, cudaStream_t st) {
       }
       const int b = std::min(TPB, n - 1 - j0);
       const bool ptc = hs && n - j0 - 1 >= PW_HS_MIN_ORDER;
-      if (ptc) PW_TRY(pw_hs_slice(ws, A, n, j0, st));
+      if (ptc) PW_TRY(pw_hs_slice(ws, A, n, j0, !ws->fixed && hgrid == 0, st));
       if (ptc && hgrid > 0) {
         PW_CUDA(cudaMemsetAsync(ws->panel, 0, (size_t)n * 3 * b * sizeof(double2), st));
         PW_TRY(pw_hs_panel(ws, A, n, j0, b, hgrid, st));

@@ -100,11 +100,12 @@ pw_status pw_dense_alloc(pw_dense_ws *ws, int nmax, int nbmax);
 // (hemv_tc.cu): used for the panels whose trailing order is at least
 // PW_HS_MIN_ORDER when the product mode is 1.  pw_hs_bytes: slice buffer
 // bytes for order nmax (0 below the threshold).  pw_hs_slice: the slices of
-// the trailing matrix of the panel starting at column j0.  The column product
+// the trailing matrix of the panel starting at column j0, in wide digits for
+// pw_hs_hemv, in narrow ones for the other two products.  The column product
 // on them (pw_hs_hemv) is declared in house.cuh.
 #define PW_HS_MIN_ORDER 1024
 size_t pw_hs_bytes(int nmax);
-pw_status pw_hs_slice(pw_dense_ws *ws, const double2 *A, int n, int j0, cudaStream_t st);
+pw_status pw_hs_slice(pw_dense_ws *ws, const double2 *A, int n, int j0, bool wide, cudaStream_t st);
 // All columns of the panel at j0 (width b, trailing order >= PW_HS_MIN_ORDER,
 // its slices written) in one cooperative launch of `grid` CTAs (from
 // pw_hs_panel_grid, 0 when the device cannot hold one per SM), leaving the

@@ -5,24 +5,37 @@
 // Inside a panel of 32 columns the trailing matrix A22 is not updated (the
 // panel's rank-2 corrections are applied through V and W), so it is split
 // once per panel into integer digit slices and every column's product reads
-// the slices instead of the FP64 matrix:
-//   * A22 2^eA = sum_p a_p 2^(-7p) (p = 1..8, the digit split of the
-//     FP64-accurate product, one scale for the whole trailing matrix), and
-//     x 2^ex = sum_q b_q 2^(-7q) for the vector x (the column itself, scaled
-//     by its norm);
-//   * the products a_p b_q with p + q = g (g = 2..9) are summed in one FP32
+// the slices instead of the FP64 matrix.  Two schemes:
+//
+// Wide (k_hemv_tc): A22 2^eA = sum_p a_p 2^(-12p) (p = 1..5, one scale for the
+// whole trailing matrix), x 2^ex = sum_q b_q 2^(-4q) (q = 1..14, a scale per 128
+// entries).  a_p fits FP16 (|a_p| <= 2,048), and the weight of a_p b_q depends on
+// 3p + q only:
+//   * the products with 3p + q = g (g = 4..19) are summed in one FP32
 //     tensor-memory accumulator per g: the B operand for slice p holds the
-//     digit q = g - p of v in its row for g, so all slices p of a tile
-//     accumulate into the same 16 columns (8 groups x real/imaginary part of
-//     v); the eight B operands are 16-row windows of one digit array.  Over
-//     64 K every partial sum is an integer below 2^22 (exact in FP32);
-//   * the epilogue adds the groups into a 64-bit fixed-point sum per output
-//     and writes one FP64 partial per tile, summed with the other tiles'
-//     partials in FP64 by the row kernel of the reduction.
-// The error per output is at most 10 K 2^-55 max|A22| for trailing order K
-// (2K real terms, each off by at most 1.25 2^-55 in scaled units: the
-// digit roundings and the dropped pairs; the scales add a factor of 4):
-// normwise FP64.
+//     digit q = g - 3p of x in its row for g, so all slices p of a tile
+//     accumulate into the same 32 columns (16 groups x real/imaginary part of
+//     x); the five B operands are 32-row windows of one digit array.  Over
+//     128 K every sum is an integer below 128 (4 + 2) 2^14 < 2^24 (exact in
+//     FP32; |b_1| <= 16, the others 8, |a_p b_q| <= 2^14, at most five pairs);
+//   * the epilogue adds the groups exactly and rounds once to a 64-bit
+//     fixed-point sum per output, one FP64 partial per tile, summed with the
+//     other tiles' partials in FP64 by the row kernel of the reduction.
+// The error per term is 2^-57 of the product of the scales (the vector's
+// rounding) and 2^-60 (the matrix's); the dropped pairs are below 2^-62.
+// What bounds the product is not memory: an MMA of M = 128, K = 16 costs about 73
+// clocks at N = 16 and hardly more at N = 32 (each one issued twice, into a spare
+// accumulator, took a unit of 128 from 6.4 to 9.8 us), so fewer slices with more
+// groups each are faster: 80 MMAs and 160 KB a unit instead of 128 and 256 KB.
+// Measured: a unit 6.4 -> 4.0 us, the product at order 3,400 37 -> 27 us, 1,500
+// 17.7 -> 13.7 us; order-3,456 eigensolve 145.0 -> 128.6 ms, 1,458 38.4 -> 35.2 ms.
+//
+// Narrow (the reflector's products in the fixed order of operations and in the
+// cooperative panel): eight 7-bit digits of both, p + q = g (g = 2..9), 16-row
+// windows, sums over 64 K below 2^22.  The error per output is at most 10 K 2^-55
+// max|A22| for trailing order K (2K real terms, each off by at most 1.25 2^-55 in
+// scaled units: the digit roundings and the dropped pairs; the scales add a
+// factor of 4): normwise FP64.
 //
 // Storage: the lower-triangle tiles of 128 x 128 (anchored at row and column
 // 0, so every tile starts on a 256-byte boundary) are written per panel in
@@ -41,8 +54,8 @@
 // Kernel (k_hemv_tc, one column per launch, chained with k_col_rows by
 // programmatic dependent launch): persistent, one CTA per SM, each CTA a
 // contiguous range of work units (tile, real or imaginary part, and for
-// short trailing orders a piece of its eight slices, so that every SM has
-// work).  Warp 0 = bulk-copy producer (five 32 KB stages), warp 1 = MMA
+// short trailing orders a piece of its slices, so that every SM has
+// work).  Warp 0 = bulk-copy producer (four 32 KB stages, five with narrow digits), warp 1 = MMA
 // issuer (one thread), warps 2..5 = B-operand builders and epilogue, warps
 // 6..9 = the finished column and the panel's correction dots on the otherwise
 // idle FP64 pipe; B operands and accumulators are double-buffered, so a unit's
@@ -68,42 +81,56 @@ using namespace pw_umma;
 
 constexpr int HT = 128;                      // tile edge
 constexpr int SUB = HT * HT * 2;             // bytes of one slice of one part of a tile (32 KB)
-constexpr int UNIT = S * SUB;                // one part of a tile, all slices (256 KB)
-// B operand of one direction: 32 rows x 128 K, no swizzle, K-major: 8-row x
-// 16-byte core matrices, rows 16 B apart, the 16 K chunks of 8 elements 512 B
-// apart.  Row 2t (Re v) / 2t + 1 (Im v) holds digit t - 6 of v for t = 7..14
-// and zeros below, so the 16-row window starting at row 14 - 2p is slice
-// p's operand: its row 2j (2j + 1) holds digit j + 1 - p, the partner of
-// slice p + 1 in group g = j + 2.
-constexpr int BROWS = 32;
-constexpr int BKC = BROWS * 16;              // bytes per K chunk (512)
-constexpr int BDIR = (HT / 8) * BKC;         // 8 KB
-constexpr int TMEM_COLS = 128;               // per buffer: D_row[h], D_col[h] (two 64-K halves), 16 columns each
+// The two digit schemes.  B operand of one direction: BROWS rows x 128 K, no
+// swizzle, K-major: 8-row x 16-byte core matrices, rows 16 B apart, the 16 K
+// chunks of 8 elements BKC bytes apart.  Rows 2t and 2t + 1 hold a digit of
+// Re v and Im v, zeros outside the digits, so the N-row window starting at row
+// WIN - WSTEP p is slice p's operand (p = 0..SL-1 here): the partner digits of
+// that slice in the groups' order.
+struct DigNarrow {                           // A: 8 of 7 bits, v: 8 of 7 bits
+  static constexpr bool wide = false;
+  static constexpr int SL = S, N = 16, BROWS = 32, WIN = 14, WSTEP = 2, T0 = 7;   // digit q of v in row 2(q + T0 - 1)
+  static constexpr int BKC = BROWS * 16;     // bytes per K chunk (512)
+  static constexpr int BDIR = (HT / 8) * BKC;   // 8 KB
+  static constexpr int UNIT = SL * SUB;      // one part of a tile, all slices (256 KB)
+};
+struct DigWide {                             // A: 5 of 12 bits, v: 14 of 4 bits
+  static constexpr bool wide = true;
+  static constexpr int SL = 5, N = 32, BROWS = 56, WIN = 24, WSTEP = 6, T0 = 12;
+  static constexpr int VD = 14;              // digits of v
+  static constexpr int BKC = BROWS * 16 + 16;   // 912: the K chunks of a warp's stores in different banks
+  static constexpr int BDIR = (HT / 8) * BKC;   // 14.25 KB
+  static constexpr int UNIT = SL * SUB;      // 160 KB
+};
+constexpr int TMEM_COLS = 128;               // per buffer: 32 columns A v, 32 columns A^H v (narrow: two 64-K halves of 16)
 constexpr int LFIX = 54;                     // binary point of the per-tile fixed-point sums
+constexpr int LFIX_WIDE = 56;
 constexpr int TPB_HS = 32;                   // panel width of the reduction
 constexpr int NBAR_FIXED = 5;                // bready[2], mdone[2], fin
 // dynamic shared memory of a CTA running the product with NS stages of one
 // sub-tile: stages, [buffer 2][dir 2] B operands, block-sum scratch, barriers
-template <int NS>
+template <int NS, class D = DigNarrow>
 struct HsL {
   static constexpr int OFF_B = NS * SUB;
-  static constexpr int OFF_RED = OFF_B + 4 * BDIR;
+  static constexpr int OFF_RED = OFF_B + 4 * D::BDIR;
   static constexpr int OFF_BAR = OFF_RED + 128;
   static constexpr int SMEM = OFF_BAR + (2 * NS + NBAR_FIXED) * 8 + 16 + 1024;
 };
-// One column per launch: five stages, not the six that fit, so that the row
+// One column per launch: fewer stages than fit, so that the row
 // kernels (11 KB and less) find room beside a CTA and both kinds start and load
 // while their predecessor runs.  That also takes the same split of L1 and shared
 // memory in every launch of the chain (the launches' carve-out): 198 KB alone
 // would get a split that leaves nothing.  Order-3,456 eigensolve 157.5 -> 145.0 ms
 // (the row kernel's part of a column 16.5 -> 11.7 us at order 3,400, 12 -> 7 us
-// at 1,500); the product itself keeps its speed with five stages.
-constexpr int NST_HEMV = 5;
+// at 1,500); the product itself keeps its speed.
+constexpr int NST_HEMV = 5;                  // narrow digits
+constexpr int NST_WIDE = 4;                  // wide digits (their B operands are larger)
 constexpr int NST_PANEL = 5;                 // cooperative panel (its column phases need static scratch)
 constexpr int SIDE_WARPS = 4;
 constexpr int NTHR = 192 + 32 * SIDE_WARPS;  // producer, MMA, 4 epilogue warps, side warps
 constexpr int NTHR_PANEL = 256;
 static_assert(HsL<NST_HEMV>::SMEM <= 232448, "shared memory per CTA");
+static_assert(HsL<NST_WIDE, DigWide>::SMEM + 12 * 1024 <= 232448, "room for a row kernel's CTA");
 static_assert(HsL<NST_PANEL>::SMEM + 8 * 1024 <= 232448, "shared memory per CTA");
 
 __device__ __forceinline__ void named_sync(int id, int nthr) {
@@ -122,20 +149,26 @@ __device__ __forceinline__ long tile_index(int I, int J) { return (long)I * (I +
 
 // work unit u: trailing tile (I, J) (relative to the first trailing tile),
 // real (0) or imaginary (1) part of its slices, and the slices p0..p1-1
-// (piece of ks equal shares); its partial sums go to slot
+// (piece of ks shares); its partial sums go to slot
 // (2 tile + part) ks + piece of the row (A v) or column (A^H v) outputs
 struct Unit {
   int I, J, part, piece, p0, p1;
 };
+template <class D>
 __device__ __forceinline__ Unit unit_of(long u, int ks) {
   Unit w;
   w.piece = (int)(u % ks);
   const long r = u / ks;
   w.part = (int)(r & 1);
   tri_decode((int)(r >> 1), w.I, w.J);
-  w.p0 = w.piece * (S / ks);
-  w.p1 = w.p0 + S / ks;
+  w.p0 = w.piece * D::SL / ks;
+  w.p1 = (w.piece + 1) * D::SL / ks;
   return w;
+}
+// slices of the column's units before unit u
+template <class D>
+__device__ __forceinline__ long slices_before(long u, int ks) {
+  return (u / ks) * D::SL + (u % ks) * D::SL / ks;
 }
 
 // byte offset of tile element (r, c) (r in a group of 8 rows r8 = r / 8)
@@ -165,10 +198,50 @@ __global__ void __launch_bounds__(256) k_hs_max(const double2 *__restrict__ A, i
   }
 }
 
+// The five digits of x0 2^e and x1 2^e (|x 2^e| <= 1/2) as FP16 pairs: with an
+// offset of half a digit added at every place, the fields of the 60-bit value
+// are the digits plus 2,048; |d| <= 2,048, all exact in FP16.
+__device__ __forceinline__ void wide_digits(double x0, double x1, int e, uint32_t *out) {
+  constexpr long long OFF = 0x800800800800800ll;
+  const long long u0 = fixed_point<60>(x0, e) + OFF, u1 = fixed_point<60>(x1, e) + OFF;
+#pragma unroll
+  for (int p = 0; p < DigWide::SL; ++p) {
+    const int sh = 12 * (DigWide::SL - 1 - p);
+    const int m = p == 0 ? ~0 : 0xFFF;
+    const int d0 = ((int)(u0 >> sh) & m) - 0x800, d1 = ((int)(u1 >> sh) & m) - 0x800;
+    const __half2 d = __halves2half2(__int2half_rn(d0), __int2half_rn(d1));
+    out[p] = *reinterpret_cast<const uint32_t *>(&d);
+  }
+}
+// the 14 digits of the vector entry (x, y), |x 2^e|, |y 2^e| <= 1: |d_1| <= 16, the
+// others <= 8, the offset again half a digit, taken off as a half
+__device__ __forceinline__ void vector_digits(double x, double y, int e, uint32_t *out) {
+  constexpr long long OFF = 0x88888888888888ll;
+  const long long u0 = fixed_point<56>(x, e) + OFF, u1 = fixed_point<56>(y, e) + OFF;
+#pragma unroll
+  for (int q = 0; q < DigWide::VD; ++q) {
+    const int sh = 4 * (DigWide::VD - 1 - q);
+    // the first digit keeps its sign: 8 more makes it non-negative
+    const uint32_t off = q == 0 ? 16u : 8u;
+    const uint32_t f0 = q == 0 ? (uint32_t)(int)(u0 >> sh) + 8u : (uint32_t)(u0 >> sh) & 15u;
+    const uint32_t f1 = q == 0 ? (uint32_t)(int)(u1 >> sh) + 8u : (uint32_t)(u1 >> sh) & 15u;
+    const uint32_t w = (f0 | (f1 << 16)) | 0x64006400u;
+    const uint32_t o2 = (0x6400u + off) * 0x10001u;
+    const __half2 d = __hsub2(*reinterpret_cast<const __half2 *>(&w), *reinterpret_cast<const __half2 *>(&o2));
+    out[q] = *reinterpret_cast<const uint32_t *>(&d);
+  }
+}
+template <class D>
+__device__ __forceinline__ void matrix_digits(double x0, double x1, int e, uint32_t *out) {
+  if constexpr (D::wide) wide_digits(x0, x1, e, out);
+  else digit_pairs(x0, x1, e, out);
+}
+
 // digit slices of the trailing tiles (I >= J >= J0): block = (tile, 16
 // columns), thread = (column, 8 consecutive rows); entries outside rows and
 // columns [j0, n) are zero, the strict upper part of a diagonal tile is the
 // conjugate of its lower part
+template <class D>
 __global__ void __launch_bounds__(256) k_hs_slice(const double2 *__restrict__ A, int n, int j0, int J0,
                                                   const unsigned long long *__restrict__ slot,
                                                   unsigned char *__restrict__ hsl) {
@@ -176,10 +249,10 @@ __global__ void __launch_bounds__(256) k_hs_slice(const double2 *__restrict__ A,
   tri_decode(blockIdx.x >> 3, I, J);
   I += J0;
   J += J0;
-  const int e = row_exp(*slot);
+  const int e = row_exp(*slot) - (D::wide ? 1 : 0);   // wide digits: |a 2^e| < 1/2
   const int cl = (blockIdx.x & 7) * 16 + (threadIdx.x >> 4), r8 = threadIdx.x & 15;
   const int c = J * HT + cl;
-  uint32_t wr[S][4], wi[S][4];
+  uint32_t wr[D::SL][4], wi[D::SL][4];
 #pragma unroll
   for (int k = 0; k < 8; k += 2) {
     double2 z[2];
@@ -195,27 +268,28 @@ __global__ void __launch_bounds__(256) k_hs_slice(const double2 *__restrict__ A,
         }
       }
     }
-    uint32_t d[S];
-    digit_pairs(z[0].x, z[1].x, e, d);
+    uint32_t d[D::SL];
+    matrix_digits<D>(z[0].x, z[1].x, e, d);
 #pragma unroll
-    for (int p = 0; p < S; ++p) wr[p][k >> 1] = d[p];
-    digit_pairs(z[0].y, z[1].y, e, d);
+    for (int p = 0; p < D::SL; ++p) wr[p][k >> 1] = d[p];
+    matrix_digits<D>(z[0].y, z[1].y, e, d);
 #pragma unroll
-    for (int p = 0; p < S; ++p) wi[p][k >> 1] = d[p];
+    for (int p = 0; p < D::SL; ++p) wi[p][k >> 1] = d[p];
   }
   const uint32_t off = sub_off(r8, cl);
-  unsigned char *base = hsl + (size_t)tile_index(I, J) * 2 * UNIT + off;
+  unsigned char *base = hsl + (size_t)tile_index(I, J) * 2 * D::UNIT + off;
 #pragma unroll
-  for (int p = 0; p < S; ++p) {
+  for (int p = 0; p < D::SL; ++p) {
     *(uint4 *)(base + (size_t)p * SUB) = make_uint4(wr[p][0], wr[p][1], wr[p][2], wr[p][3]);
-    *(uint4 *)(base + UNIT + (size_t)p * SUB) = make_uint4(wi[p][0], wi[p][1], wi[p][2], wi[p][3]);
+    *(uint4 *)(base + D::UNIT + (size_t)p * SUB) = make_uint4(wi[p][0], wi[p][1], wi[p][2], wi[p][3]);
   }
 }
 
 // --------------------------------------------------------- the product ----
 // Shared-memory view of a CTA running the product with NS stages.
-template <int NS>
+template <int NS, class D = DigNarrow>
 struct HsSmem {
+  using L = HsL<NS, D>;
   unsigned char *base;
   uint64_t *full, *empty;      // [NS] stage filled / stage read by the MMAs
   uint64_t *bready, *mdone;    // [2] a unit's B operands built (and its accumulators free) / its MMAs done
@@ -225,29 +299,29 @@ struct HsSmem {
   uint32_t *vmax;              // [2][2][4] largest entries of a unit's two blocks per warp
   __device__ explicit HsSmem(unsigned char *smem) {
     base = smem;
-    full = (uint64_t *)(smem + HsL<NS>::OFF_BAR);
+    full = (uint64_t *)(smem + L::OFF_BAR);
     empty = full + NS;
     bready = empty + NS;
     mdone = bready + 2;
     fin = mdone + 2;
     tmem_slot = (uint32_t *)(fin + 1);
-    red = (double *)(smem + HsL<NS>::OFF_RED);
+    red = (double *)(smem + L::OFF_RED);
     vmax = (uint32_t *)(red + 8);
   }
 };
 
 // barriers, the B operands' zero rows (never rewritten) and the tensor
 // memory (warp 0); the caller synchronises the block afterwards
-template <int NS>
-__device__ void hs_setup(const HsSmem<NS> &m) {
+template <int NS, class D>
+__device__ void hs_setup(const HsSmem<NS, D> &m) {
   if (threadIdx.x == 0) {
     for (int s = 0; s < NS; ++s) { mbar_init(&m.full[s], 1); mbar_init(&m.empty[s], 1); }
     for (int b = 0; b < 2; ++b) { mbar_init(&m.bready[b], 128); mbar_init(&m.mdone[b], 1); }
     mbar_init(m.fin, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  for (int w = threadIdx.x; w < 4 * BDIR / 16; w += blockDim.x)
-    ((uint4 *)(m.base + HsL<NS>::OFF_B))[w] = make_uint4(0u, 0u, 0u, 0u);
+  for (int w = threadIdx.x; w < 4 * D::BDIR / 16; w += blockDim.x)
+    ((uint4 *)(m.base + HsL<NS, D>::OFF_B))[w] = make_uint4(0u, 0u, 0u, 0u);
   if ((threadIdx.x >> 5) == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(m.tmem_slot)),
                  "r"(TMEM_COLS));
@@ -266,7 +340,10 @@ struct HsCol {
   int nmax;
   int *err;
 };
-__device__ __forceinline__ int hs_subtiles(const HsCol &w) { return w.nunit * (S / w.ks); }
+template <class D>
+__device__ __forceinline__ int hs_subtiles(const HsCol &w) {
+  return (int)(slices_before<D>(w.ub + w.nunit, w.ks) - slices_before<D>(w.ub, w.ks));
+}
 
 // the column's units of a CTA: `units` spread over the grid in contiguous ranges
 __device__ __forceinline__ void hs_range(int units, long &ub, int &nunit) {
@@ -278,7 +355,7 @@ __device__ __forceinline__ void hs_range(int units, long &ub, int &nunit) {
 // the partial sums; the host's count of slots uses the same rule
 __host__ __device__ __forceinline__ int hs_pieces(int ntp, int grid, int slots) {
   int ks = 1;
-  while (ks < S && ntp * (ntp + 1) * ks < grid && 2 * ntp * ks * 2 <= slots) ks *= 2;
+  while (ks < 4 && ntp * (ntp + 1) * ks < grid && 2 * ntp * ks * 2 <= slots) ks *= 2;
   return ks;
 }
 
@@ -295,16 +372,18 @@ __device__ __forceinline__ bool hs_failed(const int *err) { return *(const volat
 
 // producer: sub-tiles [pos, end) of the CTA's sequence for the column; k
 // counts every sub-tile the CTA has issued (stage k % NS, phase k / NS)
-template <int NS>
-__device__ bool hs_produce(const HsCol &w, const HsSmem<NS> &m, int pos, int end, int &k, uint32_t &issued,
+template <int NS, class D>
+__device__ bool hs_produce(const HsCol &w, const HsSmem<NS, D> &m, int pos, int end, int &k, uint32_t &issued,
                            uint32_t &last_ph) {
-  const int spu = S / w.ks;
+  const long g0 = slices_before<D>(w.ub, w.ks);
   for (; pos < end; ++pos, ++k) {
-    if (pos % spu == 0 && hs_failed(w.err)) return false;
-    const Unit u = unit_of(w.ub + pos / spu, w.ks);
-    const int p = u.p0 + pos % spu;
+    const long g = g0 + pos, part = g / D::SL;         // (tile, part) and its slice
+    const int p = (int)(g % D::SL);
+    if (p == 0 && hs_failed(w.err)) return false;
+    int I, J;
+    tri_decode((int)(part >> 1), I, J);
     const unsigned char *src =
-        w.hsl + ((size_t)tile_index(u.I + w.J0, u.J + w.J0) * 2 + u.part) * UNIT + (size_t)p * SUB;
+        w.hsl + ((size_t)tile_index(I + w.J0, J + w.J0) * 2 + (part & 1)) * D::UNIT + (size_t)p * SUB;
     const int s = k % NS;
     const uint32_t ph = (uint32_t)(k / NS) & 1;
     if (!mbar_wait(&m.empty[s], ph ^ 1)) { atomicOr(w.err, 1); return false; }
@@ -316,8 +395,8 @@ __device__ bool hs_produce(const HsCol &w, const HsSmem<NS> &m, int pos, int end
   return true;
 }
 // before the CTA leaves: every issued copy has landed
-template <int NS>
-__device__ void hs_produce_drain(const HsSmem<NS> &m, uint32_t issued, uint32_t last_ph, int *err) {
+template <int NS, class D>
+__device__ void hs_produce_drain(const HsSmem<NS, D> &m, uint32_t issued, uint32_t last_ph, int *err) {
   for (int s = 0; s < NS; ++s)
     if (((issued >> s) & 1) && !mbar_wait(&m.full[s], (last_ph >> s) & 1)) atomicOr(err, 1);
 }
@@ -327,39 +406,39 @@ __device__ void hs_produce_drain(const HsSmem<NS> &m, uint32_t issued, uint32_t 
 // descriptors are formed once; K steps, slices and stages only move their
 // start address (16-byte units in the low 14 bits, which cover all of shared
 // memory, so the additions never carry out).
-template <int NS>
-__device__ bool hs_mma(const HsCol &w, const HsSmem<NS> &m, uint32_t tmem, int &k, int &ug) {
-  const uint32_t id_mn = idesc_f16(128, 16, true), id_k = idesc_f16(128, 16, false);
+template <int NS, class D>
+__device__ bool hs_mma(const HsCol &w, const HsSmem<NS, D> &m, uint32_t tmem, int &k, int &ug) {
+  const uint32_t id_mn = idesc_f16(128, D::N, true), id_k = idesc_f16(128, D::N, false);
   // stage 0's A operand: MN-major (64-row atoms 1 KB apart, 8-column groups
   // 2 KB apart) and K-major (8-row groups 2 KB apart)
   const uint64_t dmn0 = smem_desc(smem_u32(m.base), 1024, 2048, 2), dk0 = smem_desc(smem_u32(m.base), 16, 2048, 2);
   for (int u = 0; u < w.nunit; ++u, ++ug) {
     if (hs_failed(w.err)) return false;
-    const Unit un = unit_of(w.ub + u, w.ks);
+    const Unit un = unit_of<D>(w.ub + u, w.ks);
     const bool diag = un.I == un.J;
     const int bf = ug & 1;
     if (!mbar_wait(&m.bready[bf], (uint32_t)(ug >> 1) & 1)) { atomicOr(w.err, 2); return false; }
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint64_t db0 = smem_desc(smem_u32(m.base + HsL<NS>::OFF_B + (2 * bf) * BDIR), BKC, 128, 0);
-    const uint64_t db1 = db0 + (BDIR >> 4);
+    const uint64_t db0 = smem_desc(smem_u32(m.base + HsL<NS, D>::OFF_B + (2 * bf) * D::BDIR), D::BKC, 128, 0);
+    const uint64_t db1 = db0 + (D::BDIR >> 4);
     const uint32_t d0 = tmem + (uint32_t)(bf * 64);
     for (int p = un.p0; p < un.p1; ++p, ++k) {
       const int s = k % NS;
       if (!mbar_wait(&m.full[s], (uint32_t)(k / NS) & 1)) { atomicOr(w.err, 2); return false; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint64_t da_mn = dmn0 + (uint64_t)(s * (SUB >> 4)), da_k = dk0 + (uint64_t)(s * (SUB >> 4));
-      const uint64_t win = (uint64_t)(14 - 2 * p);          // slice p's 16-row window of B
+      const uint64_t win = (uint64_t)(D::WIN - D::WSTEP * p);   // slice p's window of B
 #pragma unroll
       for (int kk = 0; kk < HT / 16; ++kk) {
-        const int h = kk >> 2;
-        const uint32_t acc = (p == un.p0 && (kk & 3) == 0) ? 0u : 1u;
-        const uint64_t bo = (uint64_t)(kk * (2 * BKC >> 4)) + win;
+        const int h = kk >> 2;                      // accumulator: narrow digits have one per 64 K
+        const uint32_t dh = D::wide ? 0u : (uint32_t)(h * 16);
+        const uint32_t acc = (p == un.p0 && (D::wide ? kk : kk & 3) == 0) ? 0u : 1u;
+        const uint64_t bo = (uint64_t)(kk * (2 * D::BKC >> 4)) + win;
         // A v: M = tile rows, K = tile columns (MN-major A)
-        mma_f16(d0 + (uint32_t)(h * 16), da_mn + (uint64_t)(kk * (4096 >> 4)), db0 + bo, id_mn, acc);
+        mma_f16(d0 + dh, da_mn + (uint64_t)(kk * (4096 >> 4)), db0 + bo, id_mn, acc);
         // A^H v: M = tile columns, K = tile rows (K-major A)
         if (!diag)
-          mma_f16(d0 + (uint32_t)(32 + h * 16), da_k + (uint64_t)(h * (1024 >> 4) + (kk & 3) * 2), db1 + bo,
-                  id_k, acc);
+          mma_f16(d0 + 32u + dh, da_k + (uint64_t)(h * (1024 >> 4) + (kk & 3) * 2), db1 + bo, id_k, acc);
       }
       mma_commit(&m.empty[s]);
     }
@@ -368,8 +447,8 @@ __device__ bool hs_mma(const HsCol &w, const HsSmem<NS> &m, uint32_t tmem, int &
   return true;
 }
 // every MMA of the CTA complete before the teardown
-template <int NS>
-__device__ void hs_mma_finish(const HsSmem<NS> &m, int *err) {
+template <int NS, class D>
+__device__ void hs_mma_finish(const HsSmem<NS, D> &m, int *err) {
   mma_commit(m.fin);
   if (!mbar_wait(m.fin, 0)) atomicOr(err, 2);
 }
@@ -401,12 +480,12 @@ struct VecCol {                        // the column x
 
 // Warps 2..5 (et = threadIdx.x - 64, the K entry of the B operands):
 // digits of the vector over unit u's tile columns (dir 0, A v) and rows (dir
-// 1, A^H v) into buffer ug & 1, rows 14..29 of the window layout; ev: the blocks'
+// 1, A^H v) into buffer ug & 1, from row 2 T0 of the window layout; ev: the blocks'
 // exponents, |entry| 2^ev <= 1
-template <int NS, class Vec>
-__device__ void hs_build(const HsCol &w, const HsSmem<NS> &m, int u, int ug, const Vec &vec, int (&ev)[2]) {
+template <int NS, class D, class Vec>
+__device__ void hs_build(const HsCol &w, const HsSmem<NS, D> &m, int u, int ug, const Vec &vec, int (&ev)[2]) {
   const int et = threadIdx.x - 64;
-  const Unit un = unit_of(w.ub + u, w.ks);
+  const Unit un = unit_of<D>(w.ub + u, w.ks);
   const int I = un.I + w.J0, J = un.J + w.J0;
   const bool diag = un.I == un.J;
   double2 v[2];
@@ -431,14 +510,16 @@ __device__ void hs_build(const HsCol &w, const HsSmem<NS> &m, int u, int ug, con
       ev[dir] = row_exp((unsigned long long)hb << 32);
     }
     if (dir == 1 && diag) break;
-    uint32_t d[S];
-    digit_pairs(v[dir].x, v[dir].y, ev[dir], d);
+    constexpr int ND = D::wide ? DigWide::VD : S;
+    uint32_t d[ND];
+    if constexpr (D::wide) vector_digits(v[dir].x, v[dir].y, ev[dir], d);
+    else digit_pairs(v[dir].x, v[dir].y, ev[dir], d);
     unsigned short *col =
-        (unsigned short *)(m.base + HsL<NS>::OFF_B + (2 * (ug & 1) + dir) * BDIR + (et >> 3) * BKC) + (et & 7);
+        (unsigned short *)(m.base + HsL<NS, D>::OFF_B + (2 * (ug & 1) + dir) * D::BDIR + (et >> 3) * D::BKC) + (et & 7);
 #pragma unroll
-    for (int t = 0; t < S; ++t) {
-      col[(2 * (t + 7)) * 8] = (unsigned short)d[t];
-      col[(2 * (t + 7) + 1) * 8] = (unsigned short)(d[t] >> 16);
+    for (int t = 0; t < ND; ++t) {
+      col[(2 * (t + D::T0)) * 8] = (unsigned short)d[t];
+      col[(2 * (t + D::T0) + 1) * 8] = (unsigned short)(d[t] >> 16);
     }
   }
   // the B operands (generic-proxy writes) to the tensor core, and the
@@ -449,14 +530,14 @@ __device__ void hs_build(const HsCol &w, const HsSmem<NS> &m, int u, int ug, con
 }
 
 // warps 2..5: unit u's sums (buffer ug & 1) into the partial slots
-template <int NS>
-__device__ bool hs_epilogue(const HsCol &w, const HsSmem<NS> &m, uint32_t tmem, int u, int ug, int eA, const int (&ev)[2]) {
+template <int NS, class D>
+__device__ bool hs_epilogue(const HsCol &w, const HsSmem<NS, D> &m, uint32_t tmem, int u, int ug, int eA, const int (&ev)[2]) {
   if (!mbar_wait(&m.mdone[ug & 1], (uint32_t)(ug >> 1) & 1)) { atomicOr(w.err, 4); return false; }
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const int q4 = (threadIdx.x >> 5) & 3, lane = threadIdx.x & 31;   // tensor-memory lane quarter
   const uint32_t lanes = (uint32_t)(q4 * 32) << 16;
   const int o = w.c + 1;
-  const Unit un = unit_of(w.ub + u, w.ks);
+  const Unit un = unit_of<D>(w.ub + u, w.ks);
   const int part = un.part;
   const int I = un.I + w.J0, J = un.J + w.J0;
   uint32_t r[32];
@@ -465,15 +546,31 @@ __device__ bool hs_epilogue(const HsCol &w, const HsSmem<NS> &m, uint32_t tmem, 
     if (dir == 1 && I == J) break;
     tmem_ld32(tmem + lanes + (uint32_t)((ug & 1) * 64 + dir * 32), r);
     long long R = 0, Q = 0;                     // Re v part, Im v part
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
+    if constexpr (D::wide) {
+      // group j has the weight 2^-4(j + 4): the upper and the lower eight groups
+      // exactly, at 2^-44 and 2^-76, then rounded once
+      long long lR = 0, lQ = 0;
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
-        const int sh = LFIX - BETA * (j + 2);
-        R += shifted(f2i_exact(r[h * 16 + 2 * j]), sh);
-        Q += shifted(f2i_exact(r[h * 16 + 2 * j + 1]), sh);
+        const int sh = 4 * (7 - j);
+        R += (long long)__float2int_rn(__uint_as_float(r[2 * j])) << sh;
+        Q += (long long)__float2int_rn(__uint_as_float(r[2 * j + 1])) << sh;
+        lR += (long long)__float2int_rn(__uint_as_float(r[16 + 2 * j])) << sh;
+        lQ += (long long)__float2int_rn(__uint_as_float(r[16 + 2 * j + 1])) << sh;
       }
-    const int ksc = -LFIX - eA - ev[dir];         // value = acc 2^ksc
+      R = (R << 12) + ((lR + (1ll << 19)) >> 20);
+      Q = (Q << 12) + ((lQ + (1ll << 19)) >> 20);
+    } else {
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const int sh = LFIX - BETA * (j + 2);
+          R += shifted(f2i_exact(r[h * 16 + 2 * j]), sh);
+          Q += shifted(f2i_exact(r[h * 16 + 2 * j + 1]), sh);
+        }
+    }
+    const int ksc = -(D::wide ? LFIX_WIDE : LFIX) - eA - ev[dir];   // value = acc 2^ksc
     // A = Ar + i Ai, v = vr + i vi; rows (dir 0): Ar v -> (R, Q), i Ai v -> (-Q, R);
     // columns (dir 1, conj(A)^T v): Ar -> (R, Q), -i Ai -> (Q, -R)
     long long yr, yi;
@@ -490,8 +587,8 @@ __device__ bool hs_epilogue(const HsCol &w, const HsSmem<NS> &m, uint32_t tmem, 
 
 // warps 2..5 over the column: the first two units' B operands, then each
 // unit's sums before the B operands of the unit two later replace its buffer
-template <int NS, class Vec>
-__device__ void hs_epi(const HsCol &w, const HsSmem<NS> &m, uint32_t tmem, const Vec &vec, int eA, int &ug) {
+template <int NS, class D, class Vec>
+__device__ void hs_epi(const HsCol &w, const HsSmem<NS, D> &m, uint32_t tmem, const Vec &vec, int eA, int &ug) {
   int e0[2], e1[2], e2[2];             // exponents of unit u, u + 1, u + 2
   if (w.nunit > 0) hs_build(w, m, 0, ug, vec, e0);
   if (w.nunit > 1) hs_build(w, m, 1, ug + 1, vec, e1);
@@ -564,9 +661,10 @@ struct HsArgs {
 };
 
 __global__ void __launch_bounds__(NTHR, 1) k_hemv_tc(const __grid_constant__ HsArgs a) {
-  constexpr int NS = NST_HEMV;
+  constexpr int NS = NST_WIDE;
+  using D = DigWide;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
-  const HsSmem<NS> m((unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023));
+  const HsSmem<NS, D> m((unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   HsCol w;
   w.n = a.h.n;
@@ -591,7 +689,7 @@ __global__ void __launch_bounds__(NTHR, 1) k_hemv_tc(const __grid_constant__ HsA
       // launched without overlap, so the producer needs no dependency wait
       int k = 0;
       uint32_t issued = 0, last_ph = 0;
-      hs_produce(w, m, 0, hs_subtiles(w), k, issued, last_ph);
+      hs_produce(w, m, 0, hs_subtiles<D>(w), k, issued, last_ph);
       hs_produce_drain(m, issued, last_ph, w.err);
     }
   } else if (warp == 1) {
@@ -613,7 +711,7 @@ __global__ void __launch_bounds__(NTHR, 1) k_hemv_tc(const __grid_constant__ HsA
     if (warp < 6) {
       const VecCol vec{a.h, k2};
       int ug = 0;
-      hs_epi(w, m, tmem, vec, row_exp(*a.slot), ug);
+      hs_epi(w, m, tmem, vec, row_exp(*a.slot) - 1, ug);
     } else {
       // the finished column (a share of the rows per CTA, warp 6), then the
       // dots, one (dot, chunk) per warp
@@ -677,7 +775,7 @@ __global__ void __launch_bounds__(NTHR_PANEL, 1) k_hemv_tc_fixed(const __grid_co
       // launches back, so the producer needs no dependency wait
       int k = 0;
       uint32_t issued = 0, last_ph = 0;
-      hs_produce(w, m, 0, hs_subtiles(w), k, issued, last_ph);
+      hs_produce(w, m, 0, hs_subtiles<DigNarrow>(w), k, issued, last_ph);
       hs_produce_drain(m, issued, last_ph, w.err);
     }
   } else if (warp == 1) {
@@ -780,7 +878,7 @@ __global__ void __launch_bounds__(NTHR_PANEL, 1) k_panel_tc(const __grid_constan
     const int nslots = 2 * ntp * w.ks;
     // the first stages of this column's slices, while phase A runs
     if (warp == 0 && lane == 0) {
-      pos0 = min(NS, hs_subtiles(w));
+      pos0 = min(NS, hs_subtiles<DigNarrow>(w));
       hs_produce(w, m, 0, pos0, kprod, issued, last_ph);
     }
     // ---- phase A: column c receives the panel's earlier rank-2 updates.
@@ -862,7 +960,7 @@ __global__ void __launch_bounds__(NTHR_PANEL, 1) k_panel_tc(const __grid_constan
     }
     // ---- phase B: the tensor-core product, v into the panel, the dots
     if (warp == 0) {
-      if (lane == 0) hs_produce(w, m, pos0, hs_subtiles(w), kprod, issued, last_ph);
+      if (lane == 0) hs_produce(w, m, pos0, hs_subtiles<DigNarrow>(w), kprod, issued, last_ph);
     } else if (warp == 1) {
       if (lane == 0) hs_mma(w, m, tmem, kmma, ug_mma);
     } else if (warp < 6) {
@@ -961,7 +1059,8 @@ pw_status allow_smem() {
   if (dev < 0 || dev >= 64) return PW_ERR_ARG;
   std::lock_guard<std::mutex> lk(mu);
   if (!done[dev]) {
-    PW_CUDA(cudaFuncSetAttribute(k_hemv_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, HsL<NST_HEMV>::SMEM));
+    PW_CUDA(cudaFuncSetAttribute(k_hemv_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 HsL<NST_WIDE, DigWide>::SMEM));
     PW_CUDA(
         cudaFuncSetAttribute(k_hemv_tc_fixed, cudaFuncAttributeMaxDynamicSharedMemorySize, HsL<NST_HEMV>::SMEM));
     PW_CUDA(cudaFuncSetAttribute(k_panel_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, HsL<NST_PANEL>::SMEM));
@@ -975,16 +1074,17 @@ pw_status allow_smem() {
 size_t pw_hs_bytes(int nmax) {
   if (nmax < PW_HS_MIN_ORDER) return 0;
   const size_t nt = (size_t)(nmax + HT - 1) / HT;
-  return nt * (nt + 1) / 2 * 2 * (size_t)UNIT;
+  return nt * (nt + 1) / 2 * 2 * (size_t)DigNarrow::UNIT;   // the larger of the two schemes
 }
 
-pw_status pw_hs_slice(pw_dense_ws *ws, const double2 *A, int n, int j0, cudaStream_t st) {
+pw_status pw_hs_slice(pw_dense_ws *ws, const double2 *A, int n, int j0, bool wide, cudaStream_t st) {
   unsigned long long *slot = ws->hsmax + j0 / 32;
   pw_count_launch();
   k_hs_max<<<n - j0, 256, 0, st>>>(A, n, j0, slot);
   const int J0 = j0 / HT, ntp = (n + HT - 1) / HT - J0;
   pw_count_launch();
-  k_hs_slice<<<ntp * (ntp + 1) / 2 * 8, 256, 0, st>>>(A, n, j0, J0, slot, (unsigned char *)ws->hsl);
+  (wide ? k_hs_slice<DigWide> : k_hs_slice<DigNarrow>)<<<ntp * (ntp + 1) / 2 * 8, 256, 0, st>>>(
+      A, n, j0, J0, slot, (unsigned char *)ws->hsl);
   return pw_check_launch("householder slices");
 }
 
@@ -1010,7 +1110,7 @@ pw_status pw_hs_hemv(pw_dense_ws *ws, const HhCol &h, int j0, int *nslots, int *
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(NTHR);
-  cfg.dynamicSmemBytes = HsL<NST_HEMV>::SMEM;
+  cfg.dynamicSmemBytes = HsL<NST_WIDE, DigWide>::SMEM;
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributePreferredSharedMemoryCarveout;

@@ -21,7 +21,7 @@
 // spreads: RB rows per CTA, the panel's columns over the other threads, the
 // scalars in a warp of their own meanwhile.
 // Measured: order-1,458 eigensolve 49.1 -> 40.6 ms, order 3,456 183 -> 161 ms
-// (145 ms with the row kernel resident beside k_hemv_tc);
+// (145 ms with the row kernel resident beside k_hemv_tc, 129 with wide digits there);
 // a column of trailing order 500 takes 15 us: launches 2, k2 3-4, product 5,
 // scalars 2.5, sums 1, the rows' tail 1.5.
 #include <algorithm>

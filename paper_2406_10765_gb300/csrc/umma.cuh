@@ -154,11 +154,13 @@ __device__ __forceinline__ int row_exp(unsigned long long mb) {
 // the half 1024 + that, and one packed subtraction takes the offset off.  About
 // 60 integer instructions per value against 120 for peeling remainders and
 // converting each digit.
-__device__ __forceinline__ long long fixed_point56(double x, int e) {
+// x 2^(e + U), rounded (U = 56..60)
+template <int U>
+__device__ __forceinline__ long long fixed_point(double x, int e) {
   const long long b = __double_as_longlong(x);
   const int ex = (int)((b >> 52) & 0x7FF);
-  // mantissa (53 bits) times 2^4, shifted right by r >= 0 to the unit 2^-56
-  const long long mant = ((b & 0xFFFFFFFFFFFFFll) | 0x10000000000000ll) << 4;
+  // mantissa (53 bits) times 2^(U-52), shifted right by r >= 0 to the unit 2^-U
+  const long long mant = ((b & 0xFFFFFFFFFFFFFll) | 0x10000000000000ll) << (U - 52);
   const int r = max(0, 1023 - ex - e);
   long long F = 0;
   if (ex != 0 && r < 62) F = (mant + ((1ll << r) >> 1)) >> r;
@@ -166,7 +168,7 @@ __device__ __forceinline__ long long fixed_point56(double x, int e) {
 }
 __device__ __forceinline__ void digit_pairs(double x0, double x1, int e, uint32_t *out) {
   static_assert(BETA * S == 56, "unit of the fixed-point value");
-  const long long F0 = fixed_point56(x0, e), F1 = fixed_point56(x1, e);
+  const long long F0 = fixed_point<56>(x0, e), F1 = fixed_point<56>(x1, e);
   uint32_t q0 = 0, q1 = 0;             // R_(p-1), low words
 #pragma unroll
   for (int p = 1; p <= S; ++p) {
