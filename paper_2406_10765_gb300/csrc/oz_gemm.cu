@@ -81,6 +81,7 @@ constexpr int NG = S;                 // accumulator groups g = 2..S+1
 // operations (pw_oz_ws::fixed) 64, after which every group is rounded to the
 // sum's binary point
 constexpr int CHUNK_KB = 3, CHUNK_KB_FIXED = 2;
+constexpr int PERSIST_KB = 16;        // K blocks up to which a CTA takes several tiles
 constexpr int STEPS_KB = BK / 16;     // MMA steps (16 real K) per K block
 constexpr int NH = 2;
 constexpr int SMEM_BYTES = NSTAGE * STAGE + 1024 + 512;
@@ -130,7 +131,70 @@ __device__ __forceinline__ uint32_t biased(uint32_t v) {
   return __float_as_uint(__uint_as_float(v) + 12582912.0f);
 }
 
+// The tiles of a product in the order of their rows, each row's range of column
+// tiles [lo, hi) without those that hold nothing wanted of a Hermitian output
+// (herm 1: strictly below the diagonal, mirrored later; herm 2: no element with
+// j/64 <= i/64; ioff, joff: the block's place in the whole product).
+struct OzTiles {
+  int mtiles, ntiles, bj, herm, ioff, joff;
+  __host__ __device__ void range(int mt, int &lo, int &hi) const {
+    lo = 0;
+    hi = ntiles;
+    const int gm0 = ioff + mt * BM;
+    if (herm == 1) {
+      const int d = gm0 - joff - (BN / 2 - 1);   // wanted: (BN / 2) nt >= d
+      lo = d <= 0 ? 0 : (d + BN / 2 - 1) / (BN / 2);
+      if (lo > ntiles) lo = ntiles;
+    }
+    if (herm == 2) {
+      const int e = (((gm0 + BM - 1) >> 6) + 1) * 64 - joff;   // wanted: (BN / 2) nt < e
+      hi = e <= 0 ? 0 : (e + BN / 2 - 1) / (BN / 2);
+      if (hi > ntiles) hi = ntiles;
+    }
+  }
+};
+// item's tile, or false past the last one
+__device__ __forceinline__ bool oz_tile(const OzTiles &g, int item, int &m0, int &j0) {
+  if (g.herm != 1 && g.herm != 2) {
+    const int mt = item / g.ntiles;
+    m0 = mt * BM;
+    j0 = (item - mt * g.ntiles) * g.bj;
+    return mt < g.mtiles;
+  }
+  for (int mt = 0; mt < g.mtiles; ++mt) {
+    int lo, hi;
+    g.range(mt, lo, hi);
+    if (item < hi - lo) {
+      m0 = mt * BM;
+      j0 = (lo + item) * g.bj;
+      return true;
+    }
+    item -= max(0, hi - lo);
+  }
+  return false;
+}
+// the K range of a tile (real K blocks; triangular operands are zero outside),
+// of its part z: an equal share, in whole chunks
 template <int CKB>
+__device__ __forceinline__ void oz_krange(const OzTiles &g, int m0, int j0, int kblocks, int &kb_beg, int &nkb) {
+  const int gm0 = g.ioff + m0, gj0 = g.joff + j0;
+  int kb_lo = 0, kb_hi = kblocks;
+  if (g.herm == 3) kb_lo = min(kblocks, (2 * gm0) / BK);
+  if (g.herm == 4) kb_lo = min(kblocks, (2 * gj0) / BK);
+  if (g.herm == 5) kb_hi = min(kblocks, (2 * (gm0 + BM) + BK - 1) / BK);
+  const int ntot = max(0, kb_hi - kb_lo);
+  const int nch = (ntot + CKB - 1) / CKB;
+  const int per = (nch + (int)gridDim.y - 1) / (int)gridDim.y;
+  const int c0 = min(nch, (int)blockIdx.y * per), c1 = min(nch, c0 + per);
+  kb_beg = kb_lo + c0 * CKB;
+  nkb = max(0, min(kb_hi, kb_lo + c1 * CKB) - kb_beg);
+}
+
+// PERSIST: a CTA takes every gridDim.x-th tile, so that the copies and MMAs
+// of its next tile run while the sums of this one are converted and written.  A
+// K of one chunk is mostly that: the rank-64 update of order 3,400 takes 218 us
+// so and 236 us with one CTA per tile (84 us of it MMAs).
+template <int CKB, bool PERSIST>
 __global__ void __launch_bounds__(NTHREADS, 1)
     k_oz_gemm(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
               int a_slice_rows, int b_slice_rows, int m, int n, int kblocks, int mtiles, int ntiles,
@@ -145,31 +209,16 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   uint64_t *acce = accf + NH;          // [NH] a half's accumulators drained
   uint32_t *tmem_slot = (uint32_t *)(acce + NH);
 
-  const int tile = blockIdx.x;
-  const int mt = tile / ntiles, nt = tile % ntiles;
-  if (mt >= mtiles) return;
-  const int m0 = mt * BM;              // complex rows m0 .. m0 + 127 (of this block)
-  // complex columns j0 .. j0 + 31, or with real_out (real operands: one
-  // slice row per real column of B, output real, ld ldc in doubles) real
-  // columns j0 .. j0 + 63
-  const int j0 = nt * (real_out ? BN : BN / 2);
-  const int gm0 = ioff + m0, gj0 = joff + j0;   // the same in the whole product
-  // Hermitian output, upper part (mirrored later): skip tiles strictly below
-  // the diagonal; lower part: tiles holding no element with j/64 <= i/64
-  if (herm == 1 && gm0 > gj0 + BN / 2 - 1) return;
-  if (herm == 2 && (gj0 >> 6) > ((gm0 + BM - 1) >> 6)) return;
-  // K range of the tile (real K blocks): triangular operands are zero outside
-  int kb_lo = 0, kb_hi = kblocks;
-  if (herm == 3) kb_lo = min(kblocks, (2 * gm0) / BK);
-  if (herm == 4) kb_lo = min(kblocks, (2 * gj0) / BK);
-  if (herm == 5) kb_hi = min(kblocks, (2 * (gm0 + BM) + BK - 1) / BK);
-  // K split: part z of gridDim.y takes an equal share, in whole chunks
-  const int ntot = max(0, kb_hi - kb_lo);
-  const int nch = (ntot + CKB - 1) / CKB;
-  const int per = (nch + (int)gridDim.y - 1) / (int)gridDim.y;
-  const int c0 = min(nch, (int)blockIdx.y * per), c1 = min(nch, c0 + per);
-  const int kb_beg = kb_lo + c0 * CKB;
-  const int nkb = max(0, min(kb_hi, kb_lo + c1 * CKB) - kb_beg);
+  // a tile is 128 complex rows and 32 complex columns, or with real_out (real
+  // operands: one slice row per real column of B, output real, ld ldc in
+  // doubles) 64 real columns
+  const OzTiles g{mtiles, ntiles, real_out ? BN : BN / 2, herm, ioff, joff};
+  int m0, j0;
+  if (!oz_tile(g, blockIdx.x, m0, j0)) return;
+  // every tile of the CTA has the K range of the first (one with its own, of a
+  // triangular operand, is alone)
+  int kb_beg, nkb;
+  oz_krange<CKB>(g, m0, j0, kblocks, kb_beg, nkb);
   const int nsteps = nkb * STEPS_KB;
   // binary point of the fixed-point sum: |sum| <= K' (scaled entries < 1)
   int lg = 0;
@@ -200,18 +249,23 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   if (warp == 0) {
     if (lane == 0) {
       // ---------------- TMA producer: all S slices of the A and B tiles per stage
-      for (int i = 0; i < nkb; ++i) {
-        const int s = i % NSTAGE;
-        const uint32_t u = i / NSTAGE;
-        if (!mbar_wait(&empty[s], (u & 1) ^ 1)) { atomicOr(err, 1); break; }
-        unsigned char *st = smem + s * STAGE;
-        mbar_expect_tx(&full[s], STAGE_LOAD);
-        const int x = (kb_beg + i) * BK;
+      int kc = 0;
+      bool ok = true;
+      for (int item = blockIdx.x;;) {
+        for (int i = 0; i < nkb; ++i, ++kc) {
+          const int s = kc % NSTAGE;
+          const uint32_t u = kc / NSTAGE;
+          if (!mbar_wait(&empty[s], (u & 1) ^ 1)) { atomicOr(err, 1); ok = false; break; }
+          unsigned char *st = smem + s * STAGE;
+          mbar_expect_tx(&full[s], STAGE_LOAD);
+          const int x = (kb_beg + i) * BK;
 #pragma unroll
-        for (int p = 0; p < S; ++p) {
-          tma_load_2d(st + p * A_T, &mapA, &full[s], x, p * a_slice_rows + m0);
-          tma_load_2d(st + OFF_B + p * B_T, &mapB, &full[s], x, p * b_slice_rows + (real_out ? j0 : 2 * j0));
+          for (int p = 0; p < S; ++p) {
+            tma_load_2d(st + p * A_T, &mapA, &full[s], x, p * a_slice_rows + m0);
+            tma_load_2d(st + OFF_B + p * B_T, &mapB, &full[s], x, p * b_slice_rows + (real_out ? j0 : 2 * j0));
+          }
         }
+        if (!PERSIST || !ok || !oz_tile(g, item += gridDim.x, m0, j0)) break;
       }
     }
   } else if (warp == 1) {
@@ -221,41 +275,48 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       // low 14 bits, which cover all of shared memory, so nothing carries out)
       const uint64_t da0 = smem_desc_sw64(smem_u32(smem)), db0 = smem_desc_sw64(smem_u32(smem + OFF_Z));
       uint32_t nfl0 = 0, nfl1 = 0;          // times each half was handed to the epilogue
-      bool first0 = true, first1 = true;    // the next step opens the half's chunk
-      for (int i = 0; i < nkb; ++i) {
-        const int s = i % NSTAGE;
-        const uint32_t u = i / NSTAGE;
-        if (!mbar_wait(&full[s], u & 1)) { atomicOr(err, 2); break; }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        bool ok = true;
+      int kc = 0;
+      bool ok = true;
+      for (int item = blockIdx.x;;) {
+        bool first0 = true, first1 = true;  // the next step opens the half's chunk
+        for (int i = 0; i < nkb; ++i, ++kc) {
+          const int s = kc % NSTAGE;
+          const uint32_t u = kc / NSTAGE;
+          if (!mbar_wait(&full[s], u & 1)) { atomicOr(err, 2); ok = false; break; }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
-        for (int kk = 0; kk < STEPS_KB; ++kk) {
-          const int t = i * STEPS_KB + kk;
-          const uint64_t off = (uint64_t)(s * (STAGE >> 4) + 2 * kk);
-          if (first1) {
-            // the epilogue has read the half's previous chunk
-            if (!mbar_wait(&acce[1], (nfl1 & 1) ^ 1)) { atomicOr(err, 8); ok = false; break; }
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          for (int kk = 0; kk < STEPS_KB; ++kk) {
+            const int t = i * STEPS_KB + kk;
+            const uint64_t off = (uint64_t)(s * (STAGE >> 4) + 2 * kk);
+            if (first1) {
+              // the epilogue has read the half's previous chunk
+              if (!mbar_wait(&acce[1], (nfl1 & 1) ^ 1)) { atomicOr(err, 8); ok = false; break; }
+              asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            }
+            oz_mmas<1>(tmem, da0 + off, db0 + off, first1);
+            first1 = oz_flush<CKB>(1, t, nsteps);
+            if (first1) { mma_commit(&accf[1]); ++nfl1; }
+            if (first0) {
+              if (!mbar_wait(&acce[0], (nfl0 & 1) ^ 1)) { atomicOr(err, 8); ok = false; break; }
+              asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            }
+            oz_mmas<0>(tmem, da0 + off, db0 + off, first0);
+            first0 = oz_flush<CKB>(0, t, nsteps);
+            if (first0) { mma_commit(&accf[0]); ++nfl0; }
           }
-          oz_mmas<1>(tmem, da0 + off, db0 + off, first1);
-          first1 = oz_flush<CKB>(1, t, nsteps);
-          if (first1) { mma_commit(&accf[1]); ++nfl1; }
-          if (first0) {
-            if (!mbar_wait(&acce[0], (nfl0 & 1) ^ 1)) { atomicOr(err, 8); ok = false; break; }
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          }
-          oz_mmas<0>(tmem, da0 + off, db0 + off, first0);
-          first0 = oz_flush<CKB>(0, t, nsteps);
-          if (first0) { mma_commit(&accf[0]); ++nfl0; }
+          if (!ok) break;
+          mma_commit(&empty[s]);
         }
-        if (!ok) break;
-        mma_commit(&empty[s]);
+        if (!PERSIST || !ok || !oz_tile(g, item += gridDim.x, m0, j0)) break;
       }
     }
   } else {
     // ---------------- epilogue: warps 2..9; lane quarter q, column half h
     const int q = warp & 3, h = (warp - 2) >> 2;
     const uint32_t lanes = (uint32_t)(q * 32) << 16;
+    bool ok = true;
+    uint32_t nfl[NH] = {0, 0};
+    for (int item = blockIdx.x;;) {
     // 64-bit fixed-point sums modulo 2^64; groups with a left shift add
     // kBias + v, and the biases are taken off at the end
     unsigned long long acc[32];
@@ -270,8 +331,6 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     for (int i = 0; i < 32; ++i) rem[i] = 0;
     const int slow = BETA * (S + 1) - Lfix;      // 7..
     const uint32_t mlow = (1u << slow) - 1u;
-    bool ok = true;
-    uint32_t nfl[NH] = {0, 0};
     unsigned long long bias = 0;
     for (int t = 0; t < nsteps && ok; ++t) {
 #pragma unroll
@@ -282,15 +341,15 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const int gend = CARRY && hh == NH - 1 ? NG - 2 : (hh + 1) * HG;
 #pragma unroll 1
-        for (int g = hh * HG; g < gend; ++g) {
+        for (int gr = hh * HG; gr < gend; ++gr) {
           uint32_t v[32];
-          tmem_ld32(tmem + lanes + (uint32_t)(g * BN + h * 32), v);
-          if (g == HG - 1 || (!CARRY && g == NG - 1)) {
+          tmem_ld32(tmem + lanes + (uint32_t)(gr * BN + h * 32), v);
+          if (gr == HG - 1 || (!CARRY && gr == NG - 1)) {
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
             if (lane == 0) mbar_arrive(&acce[hh]);
           }
-          const int sh = Lfix - BETA * (g + 2);
+          const int sh = Lfix - BETA * (gr + 2);
           if (sh >= 32) {
 #pragma unroll
             for (int i = 0; i < 32; ++i) acc[i] += (unsigned long long)(biased(v[i]) << (sh - 32)) << 32;
@@ -335,6 +394,11 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     }
 #pragma unroll
     for (int i = 0; i < 32; ++i) acc[i] -= bias;
+    if (PERSIST) {
+      // the tile's place again rather than in registers over its sums, which fill them
+      asm volatile("" : "+r"(item));
+      oz_tile(g, item, m0, j0);
+    }
     // alpha = +-1, beta = 0 or 1 (all products of the eigensolver): no products,
     // which would take the FP64 pipe eight instructions per element besides the
     // two conversions and two additions, and the old values all requested first.
@@ -357,17 +421,17 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       const int ka = -Lfix - ea[i];
       if (unit && !part) {
 #pragma unroll
-        for (int t0 = 0; t0 < 16; t0 += 8) {
-          double2 c[8];
-          bool on[8];
+        for (int t0 = 0; t0 < 16; t0 += 4) {
+          double2 c[4];
+          bool on[4];
 #pragma unroll
-          for (int t = 0; t < 8; ++t) {
+          for (int t = 0; t < 4; ++t) {
             const int j = jb + t0 + t;
             on[t] = j < n && !(herm == 2 && ((joff + j) >> 6) > ((ioff + i) >> 6));
             if (on[t] && beta.x != 0.0) c[t] = C[i + (long)j * ldc];
           }
 #pragma unroll
-          for (int t = 0; t < 8; ++t) {
+          for (int t = 0; t < 4; ++t) {
             if (!on[t]) continue;
             const int j = jb + t0 + t, k = ka - eb[j];
             long long ar = (long long)acc[2 * (t0 + t)], ai = (long long)acc[2 * (t0 + t) + 1];
@@ -404,6 +468,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           C[i + (long)j * ldc] = r;
         }
       }
+    }
+    if (!PERSIST || !ok || !oz_tile(g, item += gridDim.x, m0, j0)) break;
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -683,6 +749,19 @@ pw_status slice_operand(char op, int bside, const double2 *X, int ld, int nrows,
   return pw_check_launch("oz slice");
 }
 
+using OzKernel = decltype(&k_oz_gemm<CHUNK_KB, false>);
+OzKernel oz_kernel(bool fixed, bool persist) {
+  if (fixed) return persist ? k_oz_gemm<CHUNK_KB_FIXED, true> : k_oz_gemm<CHUNK_KB_FIXED, false>;
+  return persist ? k_oz_gemm<CHUNK_KB, true> : k_oz_gemm<CHUNK_KB, false>;
+}
+// One CTA per SM over its share of the tiles for a short K, where the next tile's
+// start hides the sums' conversion (order-1,458 eigensolve 35.2 -> 34.7 ms, 3,456
+// 125.9 -> 124.9 ms); else one per tile: the loop over tiles takes registers that
+// the sums need (K = 3,456: 3.72 ms with it, 3.49 without), except in the fixed
+// order, which carries no remainders (Si-512 mixed step 379 -> 374-378 ms).  One
+// per tile also for triangular operands, whose tiles differ in K.
+bool oz_persist(bool fixed, int kblocks, int herm) { return herm < 3 && (fixed || kblocks <= PERSIST_KB); }
+
 int g_max_parts = 16;
 
 // the kernel's shared-memory opt-in, once per device (outside any later
@@ -695,8 +774,8 @@ pw_status allow_smem() {
   if (dev < 0 || dev >= 64) return PW_ERR_ARG;
   std::lock_guard<std::mutex> g(mu);
   if (!done[dev]) {
-    PW_CUDA(cudaFuncSetAttribute(k_oz_gemm<CHUNK_KB>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
-    PW_CUDA(cudaFuncSetAttribute(k_oz_gemm<CHUNK_KB_FIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
+    for (auto kern : {oz_kernel(false, false), oz_kernel(false, true), oz_kernel(true, false), oz_kernel(true, true)})
+      PW_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
     done[dev] = true;
   }
   return PW_OK;
@@ -790,8 +869,8 @@ pw_status oz_block(pw_oz_ws *w, char opA, char opB, int mb, int nb, int k, doubl
     }
   }
   pw_count_launch();
-  const auto kern = w->fixed ? k_oz_gemm<CHUNK_KB_FIXED> : k_oz_gemm<CHUNK_KB>;
-  kern<<<dim3(tiles, parts), NTHREADS, SMEM_BYTES, st>>>(ma, mbm, arows, brows, mb, nb, kblocks, mtiles,
+  const bool persist = parts == 1 && oz_persist(w->fixed, kblocks, herm);
+  oz_kernel(w->fixed, persist)<<<dim3(persist ? std::min(tiles, 152) : tiles, parts), NTHREADS, SMEM_BYTES, st>>>(ma, mbm, arows, brows, mb, nb, kblocks, mtiles,
                                                                ntiles, ea, eb, alpha, beta, C, ldc, herm, ioff,
                                                                joff, parts > 1 ? w->part : nullptr, w->err, 0);
   PW_TRY(pw_check_launch("oz gemm"));
@@ -853,8 +932,8 @@ pw_status pw_dgemm_oz(pw_oz_ws *w, int m, int n, int k, const double *A, int lda
   PW_TRY(allow_smem());
   const int mtiles = arows / BM, ntiles = brows / BN;
   pw_count_launch();
-  const auto kern = w->fixed ? k_oz_gemm<CHUNK_KB_FIXED> : k_oz_gemm<CHUNK_KB>;
-  kern<<<dim3(mtiles * ntiles, 1), NTHREADS, SMEM_BYTES, st>>>(
+  const bool persist = oz_persist(w->fixed, kblocks, 0);
+  oz_kernel(w->fixed, persist)<<<dim3(persist ? std::min(mtiles * ntiles, 152) : mtiles * ntiles, 1), NTHREADS, SMEM_BYTES, st>>>(
       ma, mbm, arows, brows, m, n, kblocks, mtiles, ntiles, ea, eb, make_double2(1.0, 0.0), make_double2(0.0, 0.0),
       (double2 *)C, ldc, 0, 0, 0, nullptr, w->err, 1);
   return pw_check_launch("oz gemm (real)");
