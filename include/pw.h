@@ -398,7 +398,7 @@ pw_status pw_zgemm_tc(char opA, int m, int n, int k, const void *A, int lda, con
  * real row of op(A) and each real column of op(B) is scaled by a power of
  * two and written exactly as 8 integer slices of 7 bits (FP16 values); the
  * slice products whose weights reach 2^-63 are accumulated exactly (FP32
- * tensor-core sums over 64-wide K chunks are integers below 2^22) into a
+ * tensor-core sums over chunks of at most 96 K are integers below 2^22) into a
  * 64-bit fixed-point sum and converted to FP64 once.  Error per entry at
  * most 11K 2^-55 max_k |op(A)_ik| max_k |op(B)_kj|, within the FP64 product
  * bound for rows without large internal range.
@@ -406,7 +406,8 @@ pw_status pw_zgemm_tc(char opA, int m, int n, int k, const void *A, int lda, con
  *   op(A) = A (m x k, lda >= m) or A^H (A k x m, lda >= k);
  *   op(B) = B (k x n, ldb >= k) or B^H (B n x k, ldb >= n).
  * All device complex128, column-major; alpha, beta: host pointers to
- * (re, im).  Allocates and frees its slice buffers; synchronises `stream`.
+ * (re, im).  Takes its slice buffers from a bounded pool and gives them back;
+ * synchronises `stream`.
  * Errors: PW_ERR_ARG (bad op, sizes, leading dimensions, NULL), PW_ERR_OOM,
  * PW_ERR_CUDA, PW_ERR_TIMEOUT (a bounded device wait ran out). */
 pw_status pw_zgemm_f64tc(char opA, char opB, int m, int n, int k, const double *alpha, const void *A,
@@ -431,8 +432,10 @@ pw_status pw_dense_products(int mode);
 pw_status pw_dense_graphs(int on);
 
 /* Householder reduction of the eigensolver (Syevd, Sec. III-D),
- * process-wide.  mode = 0 (default) chains three kernels per column with
- * programmatic dependent launch; while the product mode (pw_dense_products)
+ * process-wide.  mode = 0 (default) chains two kernels per column (three in the
+ * mixed iteration's Rayleigh-Ritz, whose order of operations is fixed) with
+ * programmatic dependent launch, the last 256 columns, or all of a smaller
+ * matrix, in one thread-block cluster; while the product mode (pw_dense_products)
  * is 1, the Hermitian products A22 v of panels whose trailing order is at
  * least 1024 run on the FP16 tensor cores at FP64 accuracy (the panel's
  * trailing matrix split once into integer digit slices), the others on the
