@@ -377,6 +377,11 @@ pw_status pw_scf(pw_cell *cell, const pw_scf_opts *opts, double *eig, double *n_
  * nb < 1, nb > n, NULL pointer), PW_ERR_OOM, PW_ERR_CUDA. */
 pw_status pw_heev(int n, int nb, void *A, double *w, void *Y, void *stream);
 
+/* The same eigensolve in the order of operations of the mixed iteration's
+ * Rayleigh-Ritz (pw_subspace_step, PW_MIXED), which is fixed: its results do not
+ * change by a bit when pw_heev's kernels do.  Arguments and errors as pw_heev. */
+pw_status pw_heev_fixed(int n, int nb, void *A, double *w, void *Y, void *stream);
+
 /* Complex matrix product on the tensor cores in split-FP16 arithmetic (the
  * mixed-precision form of the dense contractions: projector products of
  * Sec. III-A, S^H S, S^H (H S) and the rotations of Sec. II-B).  Each operand
@@ -413,6 +418,11 @@ pw_status pw_zgemm_tc(char opA, int m, int n, int k, const void *A, int lda, con
 pw_status pw_zgemm_f64tc(char opA, char opB, int m, int n, int k, const double *alpha, const void *A,
                          int lda, const void *B, int ldb, const double *beta, void *C, int ldc,
                          void *stream);
+/* The same product in the order of operations that pw_heev_fixed keeps (chunks
+ * of 64 K, every digit group rounded to the sum's binary point after each). */
+pw_status pw_zgemm_f64tc_fixed(char opA, char opB, int m, int n, int k, const double *alpha, const void *A,
+                               int lda, const void *B, int ldb, const double *beta, void *C, int ldc,
+                               void *stream);
 
 /* Products of the FP64 Rayleigh-Ritz solve (Cholesky updates, triangular
  * inverse, L^-1 A L^-H, Householder panel updates, back-transformation),

@@ -117,11 +117,21 @@ _eigsolve = _sig("pw_eigsolve", ct.c_int, [_vp, ct.POINTER(pw_solve_opts), ct.PO
 
 
 _heev = _sig("pw_heev", ct.c_int, [ct.c_int, ct.c_int, _vp, _vp, _vp, _vp])
+_heev_fixed = _sig("pw_heev_fixed", ct.c_int, [ct.c_int, ct.c_int, _vp, _vp, _vp, _vp])
 
 
 def pw_heev(A, nb, stream=None):
     """Lowest nb eigenpairs of a Hermitian CUDA complex128 (n, n) tensor (column-major
     copy is made).  Returns (w (n,), Y (n, nb)) as CUDA tensors."""
+    return _run_heev(_heev, "pw_heev", A, nb, stream)
+
+
+def pw_heev_fixed(A, nb, stream=None):
+    """pw_heev in the fixed order of operations of the mixed iteration's Rayleigh-Ritz."""
+    return _run_heev(_heev_fixed, "pw_heev_fixed", A, nb, stream)
+
+
+def _run_heev(fn, name, A, nb, stream):
     import torch
     n = A.shape[0]
     a = A.t().contiguous().t().clone()       # column-major working copy
@@ -129,7 +139,7 @@ def pw_heev(A, nb, stream=None):
         a = a.t().contiguous().t()
     w = torch.empty(n, dtype=torch.float64, device=A.device)
     Y = torch.empty((nb, n), dtype=torch.complex128, device=A.device).T
-    _check(_heev(n, nb, _dptr(a), _dptr(w), _dptr(Y), _stream(stream)), "pw_heev")
+    _check(fn(n, nb, _dptr(a), _dptr(w), _dptr(Y), _stream(stream)), name)
     return w, Y
 
 
@@ -155,14 +165,24 @@ def pw_zgemm_tc(opA, A, B, C=None, beta=0.0, stream=None):
     return C
 
 
-_zgemm_f64tc = _sig("pw_zgemm_f64tc", ct.c_int, [ct.c_char, ct.c_char, ct.c_int, ct.c_int, ct.c_int,
-                                                  ct.POINTER(ct.c_double), _vp, ct.c_int, _vp, ct.c_int,
-                                                  ct.POINTER(ct.c_double), _vp, ct.c_int, _vp])
+_F64TC_ARGS = [ct.c_char, ct.c_char, ct.c_int, ct.c_int, ct.c_int, ct.POINTER(ct.c_double), _vp, ct.c_int, _vp,
+               ct.c_int, ct.POINTER(ct.c_double), _vp, ct.c_int, _vp]
+_zgemm_f64tc = _sig("pw_zgemm_f64tc", ct.c_int, _F64TC_ARGS)
+_zgemm_f64tc_fixed = _sig("pw_zgemm_f64tc_fixed", ct.c_int, _F64TC_ARGS)
 
 
 def pw_zgemm_f64tc(opA, opB, A, B, C=None, alpha=1.0, beta=0.0, stream=None):
     """C = alpha op(A) op(B) + beta C, FP64-accurate on the FP16 tensor cores.
     A, B, C: column-major CUDA complex128 tensors (stride(0) == 1)."""
+    return _run_f64tc(_zgemm_f64tc, "pw_zgemm_f64tc", opA, opB, A, B, C, alpha, beta, stream)
+
+
+def pw_zgemm_f64tc_fixed(opA, opB, A, B, C=None, alpha=1.0, beta=0.0, stream=None):
+    """pw_zgemm_f64tc in the fixed order of operations of pw_heev_fixed."""
+    return _run_f64tc(_zgemm_f64tc_fixed, "pw_zgemm_f64tc_fixed", opA, opB, A, B, C, alpha, beta, stream)
+
+
+def _run_f64tc(fn, name, opA, opB, A, B, C, alpha, beta, stream):
     import torch
     m, k = (A.shape if opA == "N" else A.shape[::-1])
     n = B.shape[1] if opB == "N" else B.shape[0]
@@ -173,8 +193,8 @@ def pw_zgemm_f64tc(opA, opB, A, B, C=None, alpha=1.0, beta=0.0, stream=None):
     a = (ct.c_double * 2)(complex(alpha).real, complex(alpha).imag)
     b = (ct.c_double * 2)(complex(beta).real, complex(beta).imag)
     ld = lambda t: max(t.stride(1), t.shape[0], 1)
-    _check(_zgemm_f64tc(opA.encode(), opB.encode(), m, n, k, a, _dptr(A), ld(A), _dptr(B), ld(B), b,
-                        _dptr(C), ld(C), _stream(stream)), "pw_zgemm_f64tc")
+    _check(fn(opA.encode(), opB.encode(), m, n, k, a, _dptr(A), ld(A), _dptr(B), ld(B), b,
+              _dptr(C), ld(C), _stream(stream)), name)
     return C
 
 

@@ -2011,18 +2011,28 @@ pw_status pw_rayleigh_ritz(pw_dense_ws *ws, int n, int nb, const double2 *G, int
   return pw_check_launch("rayleigh_ritz");
 }
 
-extern "C" pw_status pw_heev(int n, int nb, void *A, double *w, void *Y, void *stream) {
+namespace {
+pw_status heev(int n, int nb, void *A, double *w, void *Y, bool fixed, void *stream) {
   if (n < 1 || nb < 1 || nb > n || !A || !w || !Y) return PW_ERR_ARG;
   cudaStream_t st = (cudaStream_t)stream;
   pw_dense_ws ws;
   ws.mem = ws.oz.mem = pw_mem{true, st};
   ws.timed = false;
   PW_TRY(pw_dense_alloc(&ws, n, nb));
+  ws.fixed = fixed;
   pw_status r = pw_heev_lowest(&ws, n, nb, (double2 *)A, w, (double2 *)Y, st);
   if (r == PW_OK && cudaStreamSynchronize(st) != cudaSuccess) r = PW_ERR_CUDA;
   if (r == PW_OK) r = pw_oz_check(&ws.oz, st);
   pw_dense_free(&ws);
   return r;
+}
+}  // namespace
+
+extern "C" pw_status pw_heev(int n, int nb, void *A, double *w, void *Y, void *stream) {
+  return heev(n, nb, A, w, Y, false, stream);
+}
+extern "C" pw_status pw_heev_fixed(int n, int nb, void *A, double *w, void *Y, void *stream) {
+  return heev(n, nb, A, w, Y, true, stream);
 }
 
 // ---------------------------------------------------------------------------

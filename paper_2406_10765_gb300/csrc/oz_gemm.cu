@@ -1018,18 +1018,31 @@ pw_status pw_gemm64(pw_oz_ws *w, char opA, char opB, int m, int n, int k, double
   return pw_zgemm_ex(opA, opB, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, ws, ws_elems, st, herm);
 }
 
-extern "C" pw_status pw_zgemm_f64tc(char opA, char opB, int m, int n, int k, const double *alpha,
-                                    const void *A, int lda, const void *B, int ldb, const double *beta, void *C,
-                                    int ldc, void *stream) {
+namespace {
+pw_status zgemm_f64tc(char opA, char opB, int m, int n, int k, const double *alpha, const void *A, int lda,
+                      const void *B, int ldb, const double *beta, void *C, int ldc, bool fixed, void *stream) {
   if (!alpha || !beta || m < 0 || n < 0 || k < 1 || !A || !B || !C) return PW_ERR_ARG;
   if (ldc < m || lda < (opA == 'N' ? m : k) || ldb < (opB == 'N' ? k : n)) return PW_ERR_ARG;
   cudaStream_t st = (cudaStream_t)stream;
   pw_oz_ws w;
   w.mem = pw_mem{true, st};
+  w.fixed = fixed;
   pw_status r = pw_zgemm_oz(&w, opA, opB, m, n, k, make_double2(alpha[0], alpha[1]), (const double2 *)A, lda,
                             (const double2 *)B, ldb, make_double2(beta[0], beta[1]), (double2 *)C, ldc, st, 0);
   if (r == PW_OK) r = pw_oz_check(&w, st);
   if (r == PW_OK && cudaStreamSynchronize(st) != cudaSuccess) r = PW_ERR_CUDA;
   pw_oz_free(&w);
   return r;
+}
+}  // namespace
+
+extern "C" pw_status pw_zgemm_f64tc(char opA, char opB, int m, int n, int k, const double *alpha,
+                                    const void *A, int lda, const void *B, int ldb, const double *beta, void *C,
+                                    int ldc, void *stream) {
+  return zgemm_f64tc(opA, opB, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, false, stream);
+}
+extern "C" pw_status pw_zgemm_f64tc_fixed(char opA, char opB, int m, int n, int k, const double *alpha,
+                                          const void *A, int lda, const void *B, int ldb, const double *beta,
+                                          void *C, int ldc, void *stream) {
+  return zgemm_f64tc(opA, opB, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, true, stream);
 }
