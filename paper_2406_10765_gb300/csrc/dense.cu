@@ -582,7 +582,8 @@ __global__ void __launch_bounds__(CO_THREADS) k_panel_coop(double2 *A, int n, in
 // The trailing updates' product operands hold v (at most 1) and w (of the matrix's
 // size) in one row with one scale, so a matrix far from 1 is brought to it by a
 // power of two before its reduction, and the tridiagonal entries back after it;
-// within 2^+-6 it is left as it is.
+// within 2^+-6 it is left as it is.  (Unscaled, 2^100 A of order 520 came out with
+// eigenvalues off by 1e-2 of its norm.)
 // exponent of the scaling from the largest part's bits (0: none)
 __device__ __forceinline__ int matrix_scale(const unsigned long long *slot) {
   const int ex = (int)(*slot >> 52);
@@ -1665,8 +1666,8 @@ pw_status tridiag_run(pw_dense_ws *ws, int n, double2 *A, cudaStream_t st) {
 }
 
 pw_status stage_tridiag(pw_dense_ws *ws, int n, double2 *A, cudaStream_t st) {
-  // only where the updates may be digit products, and not in the fixed order
-  if (ws->fixed || pw_dense_products_mode() != 1 || n <= pw_house_cluster_max()) return tridiag_run(ws, n, A, st);
+  // only where the updates may be digit products
+  if (pw_dense_products_mode() != 1 || n <= pw_house_cluster_max()) return tridiag_run(ws, n, A, st);
   unsigned long long *slot = (unsigned long long *)((char *)ws->hscal + 64);
   PW_CUDA(cudaMemsetAsync(slot, 0, 8, st));
   pw_count_launch();

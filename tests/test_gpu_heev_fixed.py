@@ -117,3 +117,18 @@ def test_bits_of_the_product(m, n, k, c_bits):
         return torch.from_numpy((u[0] + 1j * u[1]).T.copy()).cuda().T
 
     assert _digest(pw.pw_zgemm_f64tc_fixed("N", "N", op(m, k, 1), op(k, n, 2))) == c_bits
+
+
+@pytest.mark.parametrize("n", [257, 520, 1060])
+@pytest.mark.parametrize("e", [-400, -100, 9, 100, 400])
+def test_scaled(n, e):
+    """Matrices far from 1 in size, as tests/test_gpu_heev_scale.py has them for pw_heev."""
+    import paper_2406_10765_gb300 as pw
+    A = _rand(n)
+    w, Y = pw.pw_heev_fixed(torch.from_numpy(A * 2.0 ** e).cuda(), 24)
+    w, Y = w.cpu().numpy() * 2.0 ** -e, Y.cpu().numpy()
+    ref = np.linalg.eigvalsh(A)
+    scale = np.abs(ref).max()
+    assert np.abs(w - ref).max() <= 1e-13 * scale * n ** 0.5
+    assert np.abs(A @ Y - Y * w[:24]).max() <= 1e-12 * scale
+    assert np.abs(Y.conj().T @ Y - np.eye(24)).max() <= 1e-12
