@@ -373,7 +373,8 @@ pw_status pw_scf(pw_cell *cell, const pw_scf_opts *opts, double *eig, double *n_
  * tridiagonal, divide and conquer, back-transformation.  A: device complex128
  * n x n Hermitian, column-major, ld n; destroyed.  w: device n doubles (all
  * eigenvalues, ascending).  Y: device complex128 n x nb (ld n), eigenvectors
- * of the nb lowest.  Synchronises `stream`.  Errors: PW_ERR_ARG (n < 1,
+ * of the nb lowest.  Takes its workspace from the library's pool, which keeps at
+ * most 2 GiB per device after a call; synchronises `stream`.  Errors: PW_ERR_ARG (n < 1,
  * nb < 1, nb > n, NULL pointer), PW_ERR_OOM, PW_ERR_CUDA. */
 pw_status pw_heev(int n, int nb, void *A, double *w, void *Y, void *stream);
 
@@ -391,7 +392,8 @@ pw_status pw_heev_fixed(int n, int nb, void *A, double *w, void *Y, void *stream
  *   opA = 'C': C (m x n) = A^H B, A: k x m (lda), B: k x n (ldb)
  *   opA = 'N': C (m x n) = A B,   A: m x k (lda), B: k x n (ldb)
  * All device complex128, column-major.  beta: 0 (overwrite) or 1 (C += ...).
- * Allocates and frees its own operand buffers; synchronises `stream`.
+ * Takes its operand buffers from the library's pool and gives them back before
+ * it returns; synchronises `stream`.
  * Errors: PW_ERR_ARG (bad op, sizes < 1, ld too small, beta not 0/1),
  * PW_ERR_OOM, PW_ERR_CUDA, PW_ERR_TIMEOUT (a bounded device wait ran out). */
 pw_status pw_zgemm_tc(char opA, int m, int n, int k, const void *A, int lda, const void *B,
@@ -411,8 +413,8 @@ pw_status pw_zgemm_tc(char opA, int m, int n, int k, const void *A, int lda, con
  *   op(A) = A (m x k, lda >= m) or A^H (A k x m, lda >= k);
  *   op(B) = B (k x n, ldb >= k) or B^H (B n x k, ldb >= n).
  * All device complex128, column-major; alpha, beta: host pointers to
- * (re, im).  Takes its slice buffers from a bounded pool and gives them back;
- * synchronises `stream`.
+ * (re, im).  Takes its slice buffers from the library's pool and gives them back
+ * before it returns; synchronises `stream`.
  * Errors: PW_ERR_ARG (bad op, sizes, leading dimensions, NULL), PW_ERR_OOM,
  * PW_ERR_CUDA, PW_ERR_TIMEOUT (a bounded device wait ran out). */
 pw_status pw_zgemm_f64tc(char opA, char opB, int m, int n, int k, const double *alpha, const void *A,

@@ -2019,13 +2019,11 @@ pw_status heev(int n, int nb, void *A, double *w, void *Y, bool fixed, void *str
   pw_dense_ws ws;
   ws.mem = ws.oz.mem = pw_mem{true, st};
   ws.timed = false;
-  PW_TRY(pw_dense_alloc(&ws, n, nb));
+  pw_status r = pw_dense_alloc(&ws, n, nb);
   ws.fixed = fixed;
-  pw_status r = pw_heev_lowest(&ws, n, nb, (double2 *)A, w, (double2 *)Y, st);
-  if (r == PW_OK && cudaStreamSynchronize(st) != cudaSuccess) r = PW_ERR_CUDA;
-  if (r == PW_OK) r = pw_oz_check(&ws.oz, st);
-  pw_dense_free(&ws);
-  return r;
+  if (r == PW_OK) r = pw_heev_lowest(&ws, n, nb, (double2 *)A, w, (double2 *)Y, st);
+  // (no stage ran twice, so the workspace holds no graphs)
+  return pw_finish(r, ws.oz.err, st, [&] { pw_dense_free(&ws); });
 }
 }  // namespace
 

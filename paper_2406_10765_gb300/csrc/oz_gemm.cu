@@ -1027,12 +1027,9 @@ pw_status zgemm_f64tc(char opA, char opB, int m, int n, int k, const double *alp
   pw_oz_ws w;
   w.mem = pw_mem{true, st};
   w.fixed = fixed;
-  pw_status r = pw_zgemm_oz(&w, opA, opB, m, n, k, make_double2(alpha[0], alpha[1]), (const double2 *)A, lda,
-                            (const double2 *)B, ldb, make_double2(beta[0], beta[1]), (double2 *)C, ldc, st, 0);
-  if (r == PW_OK) r = pw_oz_check(&w, st);
-  if (r == PW_OK && cudaStreamSynchronize(st) != cudaSuccess) r = PW_ERR_CUDA;
-  pw_oz_free(&w);
-  return r;
+  const pw_status r = pw_zgemm_oz(&w, opA, opB, m, n, k, make_double2(alpha[0], alpha[1]), (const double2 *)A, lda,
+                                  (const double2 *)B, ldb, make_double2(beta[0], beta[1]), (double2 *)C, ldc, st, 0);
+  return pw_finish(r, w.err, st, [&] { pw_oz_free(&w); });
 }
 }  // namespace
 

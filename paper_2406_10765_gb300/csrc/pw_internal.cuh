@@ -235,6 +235,21 @@ struct pw_mem {
 cudaError_t pw_mem_alloc(const pw_mem &m, void **p, size_t bytes);
 void pw_mem_free(const pw_mem &m, void *p);
 void pw_pool_trim();
+// The end of a call that has its workspaces from the pool: its error word (device,
+// may be nullptr) to the host, `release` frees the workspaces, and only then the
+// call waits, so that they are released for the host too when it returns.
+int *pw_host_word();
+template <typename F>
+pw_status pw_finish(pw_status r, const int *err, cudaStream_t st, F &&release) {
+  int local = 0, *h = pw_host_word();
+  if (!h) h = &local;
+  *h = 0;
+  if (err && cudaMemcpyAsync(h, err, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess && r == PW_OK)
+    r = PW_ERR_CUDA;
+  release();
+  if (cudaStreamSynchronize(st) != cudaSuccess && r == PW_OK) r = PW_ERR_CUDA;
+  return r == PW_OK && *h ? PW_ERR_TIMEOUT : r;
+}
 template <typename T>
 cudaError_t pw_cuda_malloc(T **p, size_t bytes) {
   return pw_mem_alloc(pw_mem{}, (void **)p, bytes);

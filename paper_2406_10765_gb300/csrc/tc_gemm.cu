@@ -1089,16 +1089,12 @@ extern "C" pw_status pw_zgemm_tc(char opA, int m, int n, int k, const void *A, i
         (r = pw_tc_split_coef(Bd, ldb, k, n, nullptr, &b, st)) == PW_OK)
       r = pw_tc_gemm(&a, m, &b, 2 * n, (double2 *)C, ldc, 1, beta != 0.0, 0, err, st);
   }
-  int herr = 0;
-  if (cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-      cudaStreamSynchronize(st) != cudaSuccess)
-    r = PW_ERR_CUDA;
-  if (r == PW_OK && herr) r = PW_ERR_TIMEOUT;
-  pw_mem_free(mem, err);
-  pw_mem_free(mem, rmax);
-  pw_tc_operand_free(&a);
-  pw_tc_operand_free(&b);
-  return r;
+  return pw_finish(r, err, st, [&] {
+    pw_mem_free(mem, err);
+    pw_mem_free(mem, rmax);
+    pw_tc_operand_free(&a);
+    pw_tc_operand_free(&b);
+  });
 }
 
 extern "C" pw_status pw_selftest_bounded_wait(long long cycles, void *stream) {
