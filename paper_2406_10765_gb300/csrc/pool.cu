@@ -8,9 +8,9 @@
 // what is above that at a synchronisation, and a trim only what the host has seen
 // released, so a call releases its workspaces before its last wait (pw_finish),
 // never after it (after it, 9.8 GB of operands stayed on).  All of it goes back when any
-// allocation of the library fails and when a serving run without a budget of its
-// caller's starts.  The driver orders the reuse of a block by another stream
-// after its release, so concurrent calls on any streams and threads share it.
+// allocation of the library fails and when a serving run starts.  The driver
+// orders the reuse of a block by another stream after its release, so concurrent
+// calls on any streams and threads share it.
 #include <mutex>
 
 #include "pw_internal.cuh"

@@ -330,9 +330,9 @@ extern "C" pw_status pw_serve(const pw_serve_opts *opts, const pw_request *req, 
     if (!res[i].eig || req[i].ncell < 1 || req[i].nbands < 1 || !(req[i].ecut > 0)) return PW_ERR_ARG;
   int device = 0;
   PW_CUDA(cudaGetDevice(&device));
+  pw_pool_trim();      // whatever the budget: the requests' memory comes from outside the pool
   size_t budget = opts->hbm_budget;
   if (budget == 0) {
-    pw_pool_trim();
     size_t fr = 0, tot = 0;
     PW_CUDA(cudaMemGetInfo(&fr, &tot));
     budget = fr / 10 * 8;

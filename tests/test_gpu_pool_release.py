@@ -1,7 +1,6 @@
 """Device memory that the library keeps after a call: at most the pool's bound as
 soon as the call has returned, nothing once it is asked for or a serving run has
 started."""
-import numpy as np
 import pytest
 
 import synth
@@ -43,3 +42,16 @@ def test_bounded_on_return(make):
     for _ in range(2):
         call()
         assert _held() - before <= KEEP + SLACK
+
+
+@pytest.mark.parametrize("budget", [0, 64 << 30])
+def test_serving_run_starts_with_an_empty_pool(budget):
+    import paper_2406_10765_gb300 as pw
+    req = dict(synth.serving_requests(1, rate_per_s=20.0, seed=77)[0], n=1, nbands=18, t_arrival=0.0)
+    pw.pw_serve([req], max_slots=1)
+    call = _tc()
+    before = _held()
+    call()
+    assert _held() - before > KEEP // 2
+    assert pw.pw_serve([req], max_slots=1, hbm_budget=budget)[0]["status"] == 0
+    assert _held() - before <= SLACK
