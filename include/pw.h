@@ -374,7 +374,7 @@ pw_status pw_scf(pw_cell *cell, const pw_scf_opts *opts, double *eig, double *n_
  * n x n Hermitian, column-major, ld n; destroyed.  w: device n doubles (all
  * eigenvalues, ascending).  Y: device complex128 n x nb (ld n), eigenvectors
  * of the nb lowest.  Takes its workspace from the library's pool, which keeps at
- * most 2 GiB per device after a call; synchronises `stream`.  Errors: PW_ERR_ARG (n < 1,
+ * most 2 GiB per device after a call (pw_release_memory); synchronises `stream`.  Errors: PW_ERR_ARG (n < 1,
  * nb < 1, nb > n, NULL pointer), PW_ERR_OOM, PW_ERR_CUDA. */
 pw_status pw_heev(int n, int nb, void *A, double *w, void *Y, void *stream);
 
@@ -539,6 +539,13 @@ int pw_autotune_gemm_table(char *buf, size_t len);
  * case nothing from `text` is added (the table is unchanged).  Host only: no
  * device work. */
 int pw_autotune_gemm_load(const char *text);
+
+/* Gives the device memory that the library's pool keeps after pw_heev,
+ * pw_zgemm_tc and pw_zgemm_f64tc (at most 2 GiB per device) back, on the current
+ * device, for the process's other allocators; what calls that still run in other
+ * threads hold stays with them.  The next call takes new memory.  Does not
+ * synchronise.  Errors: PW_ERR_CUDA. */
+pw_status pw_release_memory(void);
 
 /* Failure-detection self-test: one kernel waits, with the bounded wait of
  * the tensor-core GEMM pipeline and a limit of `cycles` SM clocks (1 ..

@@ -646,6 +646,14 @@ def pw_cell_fft_tune_log(cell):
     return buf.value.decode()
 
 
+_release = _sig("pw_release_memory", ct.c_int, [])
+
+
+def pw_release_memory():
+    """Gives the memory that the library's pool keeps between calls back (current device)."""
+    _check(_release(), "pw_release_memory")
+
+
 _selftest_wait = _sig("pw_selftest_bounded_wait", ct.c_int, [ct.c_longlong, _vp])
 
 

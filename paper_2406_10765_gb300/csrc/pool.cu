@@ -7,10 +7,11 @@
 // The pool keeps at most PW_POOL_KEEP bytes between calls.  The driver gives back
 // what is above that at a synchronisation, and a trim only what the host has seen
 // released, so a call releases its workspaces before its last wait (pw_finish),
-// never after it (after it, 9.8 GB of operands stayed on).  All of it goes back when any
-// allocation of the library fails and when a serving run starts.  The driver
-// orders the reuse of a block by another stream after its release, so concurrent
-// calls on any streams and threads share it.
+// never after it (after it, 9.8 GB of operands stayed on).  All of it goes back
+// when an allocation of the library fails, when a serving run starts and on
+// pw_release_memory (another allocator of the process cannot ask for it).  The
+// driver orders the reuse of a block by another stream after its release, so
+// concurrent calls on any streams and threads share it.
 #include <mutex>
 
 #include "pw_internal.cuh"
@@ -48,6 +49,13 @@ cudaMemPool_t pool(bool create) {
 void pw_pool_trim() {
   if (cudaMemPool_t p = pool(false))
     if (cudaMemPoolTrimTo(p, 0) != cudaSuccess) cudaGetLastError();
+}
+
+extern "C" pw_status pw_release_memory(void) {
+  int dev = 0;
+  PW_CUDA(cudaGetDevice(&dev));
+  pw_pool_trim();
+  return PW_OK;
 }
 
 cudaError_t pw_mem_alloc(const pw_mem &m, void **p, size_t bytes) {

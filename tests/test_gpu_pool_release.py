@@ -55,3 +55,17 @@ def test_serving_run_starts_with_an_empty_pool(budget):
     assert _held() - before > KEEP // 2
     assert pw.pw_serve([req], max_slots=1, hbm_budget=budget)[0]["status"] == 0
     assert _held() - before <= SLACK
+
+
+@pytest.mark.parametrize("make", [_tc, _heev])
+def test_release_memory(make):
+    import paper_2406_10765_gb300 as pw
+    call = make()
+    call()
+    pw.pw_release_memory()
+    before = _held()
+    call()
+    assert _held() - before > KEEP // 2
+    pw.pw_release_memory()
+    assert _held() - before <= SLACK
+    call()                                       # and takes new memory
