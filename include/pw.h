@@ -555,6 +555,16 @@ pw_status pw_release_memory(void);
  * PW_ERR_ARG, PW_ERR_CUDA.  Synchronises `stream`. */
 pw_status pw_selftest_bounded_wait(long long cycles, void *stream);
 
+/* Self-test of the eigensolver's FP64 operations that stand in for CUDA's rounded
+ * ones: op = 0: out[i] = 1 / a[i]; op = 1: a[i] / b[i]; op = 2: the Householder
+ * reflector of a vector with the head b[i] + i c[i] and the squared norm a[i] below
+ * it: out[k n + i], k = 0..4, = beta, Re tau, Im tau, Re s, Im s (v = x s below its
+ * unit head).  Device doubles, n of them each (out: 5 n for op = 2); arrays that the
+ * op does not read may be NULL.  Synchronises `stream`.  Errors: PW_ERR_ARG (op, n
+ * outside 1..2^30, NULL), PW_ERR_CUDA. */
+pw_status pw_selftest_fp64_ops(int op, long n, const void *a, const void *b, const void *c, void *out,
+                               void *stream);
+
 /* Number of CUDA kernel launches the library has issued in this process
  * (all devices, all threads); a diagnostic counter for launch accounting. */
 uint64_t pw_kernel_launches(void);

@@ -662,6 +662,20 @@ def pw_selftest_bounded_wait(cycles, stream=None):
     return int(_selftest_wait(int(cycles), _stream(stream)))
 
 
+_selftest_ops = _sig("pw_selftest_fp64_ops", ct.c_int, [ct.c_int, ct.c_long, _vp, _vp, _vp, _vp, _vp])
+
+
+def pw_selftest_fp64_ops(op, a, b=None, c=None, stream=None):
+    """The eigensolver's 1/a (op 0), a/b (op 1) or reflector scalars (op 2: (5, n)) of CUDA float64 tensors."""
+    import torch
+    n = a.numel()
+    args = [t.contiguous() if t is not None else None for t in (a, b, c)]
+    out = torch.empty((5, n) if op == 2 else (n,), dtype=torch.float64, device=a.device)
+    _check(_selftest_ops(op, n, *[_dptr(t) if t is not None else None for t in args], _dptr(out), _stream(stream)),
+           "pw_selftest_fp64_ops")
+    return out
+
+
 def pw_autotune_gemm_load(text):
     """Add K-split choices saved from pw_autotune_gemm_table; returns the lines added."""
     n = _tune_load(text.encode())

@@ -61,11 +61,15 @@ __device__ double block_max(double v, double *sh) {
   return r;
 }
 
-// 1 / x by one cubic Newton-Raphson step on the hardware's approximate
-// reciprocal (relative error e -> e^3, about an ulp for normal x): three FP64
-// operations instead of the ten of a rounded reciprocal.  The FP64 pipe issues
-// one warp instruction per sub-partition in 64 clocks on this part, so the
-// count of FP64 instructions is what the kernels below cost.
+// 1 / x: Householder's iteration of order two for the root of 1/r - x (A. S.
+// Householder, The Numerical Treatment of a Single Nonlinear Equation, 1970), once,
+// from the hardware's approximate reciprocal: with e = 1 - x r, 1/x = r / (1 - e) =
+// r (1 + e + e^2 + ..), the relative error e becoming e^3.  The instruction looks at
+// 20 bits of the mantissa, so |e| < 2^-18 and e^3 < 2^-54: at most one ulp from the
+// rounded reciprocal, for normal x with a normal reciprocal (0, infinities and
+// subnormal numbers give NaN or 0).  Three FP64 operations besides the instruction;
+// the FP64 pipe issues one warp instruction per sub-partition in 64 clocks on this
+// part, so the count of FP64 instructions is what the kernels below cost.
 __device__ __forceinline__ double rcp_approx(double x) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
@@ -76,8 +80,10 @@ __device__ __forceinline__ double rcp_newton(double x) {
   const double e = fma(-x, r, 1.0);
   return fma(r, fma(e, e, e), r);
 }
-// a / x with the remainder of the first quotient folded in (error below one
-// ulp for normal quotients)
+// a / x: the quotient q = a (1/x) corrected by its remainder a - q x from an FMA
+// (P. W. Markstein, Computation of elementary functions on the IBM RISC
+// System/6000 processor, 1990): at most one ulp from the rounded quotient where
+// that is a normal number and |a| > 2^-960 (a smaller one's remainder is subnormal)
 __device__ __forceinline__ double div_newton(double a, double x) {
   const double r = rcp_newton(x);
   const double q = a * r;
@@ -105,6 +111,25 @@ __device__ __forceinline__ void warp_sum4(double &a, double &b, double &c, doubl
 __device__ __forceinline__ long long ordered_bits(double v) {
   const long long b = __double_as_longlong(v + 0.0);   // -0 -> +0
   return b < 0 ? (long long)0x8000000000000000ull - b : b;
+}
+
+// the operations above and reflector_scalars_fast on arrays (pw_selftest_fp64_ops)
+__global__ void __launch_bounds__(256) k_fp64_ops(int op, long n, const double *a, const double *b, const double *c,
+                                                  double *out) {
+  const long i = blockIdx.x * 256l + threadIdx.x;
+  if (i >= n) return;
+  if (op == 0) out[i] = rcp_newton(a[i]);
+  else if (op == 1) out[i] = div_newton(a[i], b[i]);
+  else {
+    double beta;
+    double2 tk, scal;
+    reflector_scalars_fast(a[i], make_double2(b[i], c[i]), beta, tk, scal);
+    out[i] = beta;
+    out[n + i] = tk.x;
+    out[2 * n + i] = tk.y;
+    out[3 * n + i] = scal.x;
+    out[4 * n + i] = scal.y;
+  }
 }
 
 // ======================================================================
@@ -2026,6 +2051,17 @@ pw_status heev(int n, int nb, void *A, double *w, void *Y, bool fixed, void *str
   return pw_finish(r, ws.oz.err, st, [&] { pw_dense_free(&ws); });
 }
 }  // namespace
+
+extern "C" pw_status pw_selftest_fp64_ops(int op, long n, const void *a, const void *b, const void *c, void *out,
+                                          void *stream) {
+  if (op < 0 || op > 2 || n < 1 || n > (1l << 30) || !a || (op > 0 && !b) || (op > 1 && !c) || !out) return PW_ERR_ARG;
+  cudaStream_t st = (cudaStream_t)stream;
+  pw_count_launch();
+  k_fp64_ops<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(op, n, (const double *)a, (const double *)b,
+                                                          (const double *)c, (double *)out);
+  PW_TRY(pw_check_launch("fp64 ops"));
+  return cudaStreamSynchronize(st) == cudaSuccess ? PW_OK : PW_ERR_CUDA;
+}
 
 extern "C" pw_status pw_heev(int n, int nb, void *A, double *w, void *Y, void *stream) {
   return heev(n, nb, A, w, Y, false, stream);

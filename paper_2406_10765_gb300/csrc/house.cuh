@@ -121,10 +121,14 @@ __device__ __forceinline__ double2 warp_sum_c(double2 s) {
   return make_double2(__shfl_sync(0xffffffffu, v, 0), __shfl_sync(0xffffffffu, v, 16));
 }
 
-// reflector_scalars with Newton steps on the hardware's approximate reciprocal
-// square root and reciprocal (cubic each, then the square root's remainder):
-// about an ulp, a third of the time; outside the range where the squares are
-// normal numbers the rounded operations
+// reflector_scalars without CUDA's square root and divisions, a third of the time.
+// 1/sqrt(s) from the hardware's approximation r: with h = 1 - s r^2, r (1 - h)^(-1/2)
+// = r (1 + h/2 + 3 h^2 / 8 + ..), and sqrt(s) by one step of Heron's iteration from
+// s r; 1/dd by Householder's iteration of order two (rcp_newton in dense.cu).
+// Against exact arithmetic beta is within 4, tau 8 and s 16 units of 2^-53 of
+// each component (the bounds of the operations' roundings; the rounded form's are
+// the same).  Outside the range where the squares are normal numbers the rounded
+// operations.
 __device__ __forceinline__ void reflector_scalars_fast(double xn2, double2 alpha, double &beta, double2 &tk,
                                                        double2 &scal) {
   const double s2 = fma(alpha.x, alpha.x, fma(alpha.y, alpha.y, xn2));
