@@ -106,10 +106,10 @@ __device__ __forceinline__ void warp_sum4(double &a, double &b, double &c, doubl
   b = __shfl_sync(0xffffffffu, v, 16);
   d = __shfl_sync(0xffffffffu, v, 24);
 }
-// order-preserving integer of a (finite or infinite) double: comparisons then
-// run on the integer pipe
+// order-preserving integer of a double (-0 as +0): comparisons then run on the
+// integer pipe, and NaNs have a place in the order too, beyond the infinities
 __device__ __forceinline__ long long ordered_bits(double v) {
-  const long long b = __double_as_longlong(v + 0.0);   // -0 -> +0
+  const long long b = __double_as_longlong(v);
   return b < 0 ? (long long)0x8000000000000000ull - b : b;
 }
 
@@ -745,22 +745,25 @@ __global__ void __launch_bounds__(256) k_dc_deflate(const int *nodes, int n, con
   const int size = hi - lo, m1 = mid - lo;
   const double beta = e[mid - 1] * a.scale[0];
   const double rho = fabs(beta), sgn = beta >= 0.0 ? 1.0 : -1.0;
-  // 1. merge: left value -> its index + #(right < v); right -> index + #(left <= v)
+  // 1. merge: left value -> its index + #(right < v); right -> index + #(left <= v).
+  // In the order of k_dc_rank, which sorted the halves: the places are then a
+  // permutation whatever the values.  (Compared as doubles, NaNs left places of
+  // perm unwritten, and what the memory held before became an index.)
   for (int p = threadIdx.x; p < size; p += blockDim.x) {
-    const double v = a.lam[lo + p];
+    const long long v = ordered_bits(a.lam[lo + p]);
     int out;
     if (p < m1) {
       int l = 0, r = size - m1;
       while (l < r) {
         const int mm = (l + r) >> 1;
-        if (a.lam[lo + m1 + mm] < v) l = mm + 1; else r = mm;
+        if (ordered_bits(a.lam[lo + m1 + mm]) < v) l = mm + 1; else r = mm;
       }
       out = p + l;
     } else {
       int l = 0, r = m1;
       while (l < r) {
         const int mm = (l + r) >> 1;
-        if (a.lam[lo + mm] <= v) l = mm + 1; else r = mm;
+        if (ordered_bits(a.lam[lo + mm]) <= v) l = mm + 1; else r = mm;
       }
       out = (p - m1) + l;
     }
