@@ -2132,19 +2132,3 @@ pw_status pw_rr_finish_tall(pw_dense_ws *ws, int n, int nb, const double2 *At, i
   cudaEventRecord(ws->ev[5], st);
   return pw_check_launch("rr_finish_tall");
 }
-
-pw_status pw_rr_finish(pw_dense_ws *ws, int n, int nb, const double2 *At, int lda, const double2 *M,
-                       int ldm, double *theta, double2 *C, int ldc, cudaStream_t st) {
-  if (n > ws->nmax || nb > ws->nbmax || nb > n) return PW_ERR_ARG;
-  // Hermitian order-n matrix into the workspace (ld n), eigensolve, C = M Y
-  pw_count_launch();
-  const dim3 g2((n + 31) / 32, (n + 31) / 32), b2(32, 32);
-  k_copy_herm<<<g2, b2, 0, st>>>(At, lda, n, ws->A);
-  PW_TRY(pw_heev_lowest(ws, n, nb, ws->A, ws->lam, ws->Y, st));
-  PW_CUDA(cudaMemcpyAsync(theta, ws->lam, nb * 8, cudaMemcpyDeviceToDevice, st));
-  const double2 one = make_double2(1.0, 0.0), zero = make_double2(0.0, 0.0);
-  // M is upper triangular: each row tile skips the zero part of its K range
-  PW_TRY(pw_dense_gemm(ws, 'N', 'N', n, nb, n, one, M, ldm, ws->Y, n, zero, C, ldc, st, 3));
-  cudaEventRecord(ws->ev[5], st);
-  return pw_check_launch("rr_finish");
-}

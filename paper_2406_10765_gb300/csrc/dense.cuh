@@ -144,17 +144,15 @@ pw_status pw_rayleigh_ritz(pw_dense_ws *ws, int n, int nb, const double2 *G, int
 
 // Rayleigh-Ritz in two halves.  pw_rr_factor: Jacobi scaling d and Cholesky
 // of G (same pivot test), L^-1, and M = d o L^-H (n x n upper triangular,
-// ld ldm); synchronises.  pw_rr_finish: eigensolve of the Hermitian matrix
-// At = M^H A M (given, ld lda), theta (nb), C = M Y (n x nb, ldc).  The
-// sub-stage events are recorded as for pw_rayleigh_ritz.
+// ld ldm); synchronises.
 pw_status pw_rr_factor(pw_dense_ws *ws, int n, const double2 *G, int ldg, double2 *M, int ldm,
                        int *chol_ok, cudaStream_t st, double piv_tol);
-pw_status pw_rr_finish(pw_dense_ws *ws, int n, int nb, const double2 *At, int lda, const double2 *M,
-                       int ldm, double *theta, double2 *C, int ldc, cudaStream_t st);
-// Variant for callers that hold the orthonormalised basis S~ = S M: leaves
-// the eigenvectors Y (n x nb, ld n) in ws->Y for X' = S~ Y and forms only
-// the rows nb..n-1 of C = M Y (= M[nb:, nb:] Y[nb:], M upper triangular) in
-// Cp, whose rows 0..nb-1 are set to zero: P' = S Cp.
+// pw_rr_finish_tall, for callers that hold the orthonormalised basis S~ = S M:
+// eigensolve of the Hermitian matrix At = M^H A M (given, ld lda), theta (nb);
+// leaves the eigenvectors Y (n x nb, ld n) in ws->Y for X' = S~ Y and forms only
+// the rows nb..n-1 of C = M Y (= M[nb:, nb:] Y[nb:], M upper triangular) in Cp,
+// whose rows 0..nb-1 are set to zero: P' = S Cp.  The sub-stage events are
+// recorded as for pw_rayleigh_ritz.
 pw_status pw_rr_finish_tall(pw_dense_ws *ws, int n, int nb, const double2 *At, int lda, const double2 *M,
                             int ldm, double *theta, double2 *Cp, int ldc, cudaStream_t st);
 
