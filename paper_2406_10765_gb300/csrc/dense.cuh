@@ -69,11 +69,13 @@ struct pw_dense_ws {
   pw_mem mem;
   bool timed = true;          // with the events below
   // One fixed order of operations in the dense solves of the mixed iteration
-  // (set by pw_rr_factor and pw_rr_finish_tall): the iteration multiplies a
-  // difference of rounding (1e-15) through its FP16 splits and FP32 FFTs to
-  // 1e-7 in the Ritz values of an unconverged block, so another order is
-  // another trajectory.  Its kernels keep the sums they had; the FP64 solves
-  // take the faster ones.
+  // (set by pw_rr_factor and pw_rr_finish_tall; pw_heev_fixed has it too): the
+  // iteration multiplies a difference of rounding (1e-15) through its FP16 splits
+  // and FP32 FFTs to 1e-7 in the Ritz values of an unconverged block.  That is
+  // noise of the size that the iteration makes itself and converges away, so the
+  // order is there for steps that repeat bit for bit, not for accuracy; it costs
+  // about 60 of the 370 ms of a Si-512 mixed step.  The FP64 solves take the
+  // faster kernels.
   bool fixed = false;
   unsigned *ticket = nullptr;   // last-block-done counter of house_chain.cu
   // sub-stage timing of the last Rayleigh-Ritz: events at the boundaries of

@@ -47,8 +47,10 @@
 // limits the rate.  The two halves of the groups are emptied half a chunk
 // apart, so that the MMAs of one run while the epilogue reads the other.
 // Measured, 3,456 x 1,152 x 3,456: 6.15 ms with one MMA per slice pair, 3.35 ms
-// so (33 TFLOP/s FP64-equivalent); what it issues, zeros included, is 1.58
-// PFLOP/s, 0.82 of the measured cuBLAS burst rate: the tensor pipe bounds it.
+// so (33 TFLOP/s FP64-equivalent).  What it issues, zeros included, is 1.58
+// PFLOP/s, 0.82 of the measured cuBLAS burst rate, with the tensor pipe active
+// 74% of the time: that pipe bounds it, a quarter of its work for zeros, and the
+// last of 6.4 waves (81% without it).  Operand reads are not at their limit.
 // Every mbarrier wait is bounded; on timeout the CTA records an error word,
 // frees its tensor memory and returns.
 #include <cuda.h>

@@ -1,8 +1,9 @@
 // Device memory of calls that need a workspace only while they run (pw_heev,
-// pw_zgemm_tc, pw_zgemm_f64tc): a stream-ordered pool of the library's own per
-// device.  Allocating and freeing them with cudaMalloc / cudaFree mapped and
-// unmapped gigabytes on every call: 1.6 of the 4.8 ms of a 1,458 x 1,458 x
-// 43,819 split-FP16 product, 0.4 of the 1.3 ms of an order-54 eigensolve.
+// pw_zgemm_f64tc, their fixed forms, pw_zgemm_tc): a
+// stream-ordered pool of the library's own per device.  Allocating and freeing
+// them with cudaMalloc / cudaFree mapped and unmapped gigabytes on every call: 1.6
+// of the 4.8 ms of a 1,458 x 1,458 x 43,819 split-FP16 product, 0.4 of the 1.3 ms
+// of an order-54 eigensolve.
 //
 // The pool keeps at most PW_POOL_KEEP bytes between calls.  The driver gives back
 // what is above that at a synchronisation, and a trim only what the host has seen

@@ -145,15 +145,6 @@ __device__ __forceinline__ int row_exp(unsigned long long mb) {
   if (ex == 0) return 0;                 // zero (or subnormal): any scale works
   return 1022 - ex;                      // max in [2^(ex-1023), 2^(ex-1022)) -> [1/2, 1)
 }
-// The S digits of x0 2^e and x1 2^e (|x 2^e| <= 1) as FP16 pairs (x0 low): the
-// fixed-point value F = round(x 2^(e + 56)) is cut from the top, BETA bits at a
-// time, each digit rounded to nearest; |d_1| <= 2^BETA, |d_p| <= 2^(BETA-1)
-// after it, and x 2^e = sum_p d_p 2^(-BETA p) to 2^-57.  The digits up to p add
-// up to F rounded at digit p, R_p = (F + half) >> shift, so d_p = R_p - 2^BETA
-// R_(p-1) needs no remainder; d + 64 (d_1 + 128) under the exponent of 1024 is
-// the half 1024 + that, and one packed subtraction takes the offset off.  About
-// 60 integer instructions per value against 120 for peeling remainders and
-// converting each digit.
 // x 2^(e + U), rounded (U = 56..60)
 template <int U>
 __device__ __forceinline__ long long fixed_point(double x, int e) {
@@ -166,6 +157,15 @@ __device__ __forceinline__ long long fixed_point(double x, int e) {
   if (ex != 0 && r < 62) F = (mant + ((1ll << r) >> 1)) >> r;
   return b < 0 ? -F : F;
 }
+// The S digits of x0 2^e and x1 2^e (|x 2^e| <= 1) as FP16 pairs (x0 low): the
+// fixed-point value F = round(x 2^(e + 56)) is cut from the top, BETA bits at a
+// time, each digit rounded to nearest; |d_1| <= 2^BETA, |d_p| <= 2^(BETA-1)
+// after it, and x 2^e = sum_p d_p 2^(-BETA p) to 2^-57.  The digits up to p add
+// up to F rounded at digit p, R_p = (F + half) >> shift, so d_p = R_p - 2^BETA
+// R_(p-1) needs no remainder; d + 64 (d_1 + 128) under the exponent of 1024 is
+// the half 1024 + that, and one packed subtraction takes the offset off.  About
+// 60 integer instructions per value against 120 for peeling remainders and
+// converting each digit.
 __device__ __forceinline__ void digit_pairs(double x0, double x1, int e, uint32_t *out) {
   static_assert(BETA * S == 56, "unit of the fixed-point value");
   const long long F0 = fixed_point<56>(x0, e), F1 = fixed_point<56>(x1, e);
